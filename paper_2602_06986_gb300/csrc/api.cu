@@ -144,6 +144,7 @@ void group_tiles(std::vector<Tile> &t, int64_t ia, int BI, int G) {
 
 struct ScreenPlan {
   int prec64, nt, passes;
+  int npt = 0, tile_rows = 0;    // CUDA-core pair kernels: targets side by side, i-rows of a tile
   int64_t cap;
   std::vector<Tile> mul_tiles, add_tiles;
   bool use_pairlist = false;     // additive slots from the equal-unit pair list
@@ -294,7 +295,7 @@ __global__ void k_screen_reset(unsigned *count, unsigned *hist, unsigned *hist_h
 }
 
 static dse_status run_screen(dse_result *R, const ScreenPlan &plan, void *scr_tiles_mul, void *scr_tiles_add,
-                             ScreenArgs &A, SelectArgs &S, unsigned int *tile_ctr) {
+                             ScreenArgs &A, SelectArgs &S) {
   dse_space *sp = R->space;
   cudaStream_t st = R->stream;
   const int sms = sm_count();
@@ -362,20 +363,11 @@ static dse_status run_screen(dse_result *R, const ScreenPlan &plan, void *scr_ti
       DSE_TRY(launch_pair_gmt(A, sp->gmt_buf, plan.gmt_scr, plan.gmt_tiles_dev, (int)plan.gmt_tiles.size(), sms,
                               st));
     } else if (!plan.mul_tiles.empty()) {
+      // (one launch: the CTAs take the leading seed tiles first)
       A.rowid = sp->rowid_ident;
-      A.tile_counter = tile_ctr;
-      const Tile *t0p = reinterpret_cast<const Tile *>(scr_tiles_mul);
-      const int32_t nall = (int32_t)plan.mul_tiles.size(), ns = plan.n_seed_tiles;
-      if (ns > 0) {
-        A.tiles = t0p;
-        A.n_tiles = ns;
-        DSE_CUDA(cudaMemsetAsync(tile_ctr, 0, sizeof(unsigned), st));
-        DSE_TRY(launch_pair(plan.prec64, KIND_MUL, plan.nt, A, plan.block_len, sms, st));
-      }
-      A.tiles = t0p + ns;
-      A.n_tiles = nall - ns;
-      DSE_CUDA(cudaMemsetAsync(tile_ctr, 0, sizeof(unsigned), st));
-      DSE_TRY(launch_pair(plan.prec64, KIND_MUL, plan.nt, A, plan.block_len, sms, st));
+      A.tiles = reinterpret_cast<const Tile *>(scr_tiles_mul);
+      A.n_tiles = (int32_t)plan.mul_tiles.size();
+      DSE_TRY(launch_pair(plan.prec64, KIND_MUL, plan.npt, plan.tile_rows, A, plan.block_len, sms, st));
     }
     DSE_TRY(mark(2));
     if (plan.use_pairlist) {
@@ -384,9 +376,7 @@ static dse_status run_screen(dse_result *R, const ScreenPlan &plan, void *scr_ti
       A.tiles = reinterpret_cast<const Tile *>(scr_tiles_add);
       A.n_tiles = (int32_t)plan.add_tiles.size();
       A.rowid = plan.add_by_id ? sp->rowid_ident : sp->class_rows;
-      A.tile_counter = tile_ctr + 1;
-      DSE_CUDA(cudaMemsetAsync(tile_ctr + 1, 0, sizeof(unsigned), st));
-      DSE_TRY(launch_pair(plan.prec64, KIND_ADD, plan.nt, A, plan.block_len, sms, st));
+      DSE_TRY(launch_pair(plan.prec64, KIND_ADD, plan.npt, plan.tile_rows, A, plan.block_len, sms, st));
     }
   }
   DSE_TRY(mark(3));
@@ -408,7 +398,6 @@ struct Keep {
   ScreenArgs A;
   SelectArgs S;
   Tile *tmul, *tadd;
-  unsigned *tile_ctr;
 };
 
 // Plan a screen and allocate everything; with launch, also upload the
@@ -459,7 +448,9 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
   plan.p1 = std::min(pe, g.um);
   // binary block range in pair space
   const uint64_t bb = std::max(pb, g.um), be = std::max(pe, g.um);
-  int BI = plan.nt == 1 ? 32 : 16, BJ = BI;
+  int BI, BJ;
+  plan.npt = pair_targets(plan.prec64, d->n_targets);
+  pair_tile_shape(plan.prec64, plan.npt, g.nb > 0 && be > bb ? (int64_t)((be - bb) / g.nb) : 0, sm_count(), &BI, &BJ);
   if (plan.use_tc) {
     BI = 16;  // 128-pair tensor-core tiles
     BJ = 8;
@@ -489,10 +480,11 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
                    !(d->flags & DSE_FLAG_DIRECT);
     if (plan.use_gmt) {
       plan.use_tc = false;
-      BI = BJ = 16;
+      pair_tile_shape(0, plan.npt, 0, 1, &BI, &BJ);
     }
     // a+b and a-b come from the same contraction (the centred cross term);
     // the additive kernels then run for |a-b| alone, or not at all
+    plan.tile_rows = BI;
     plan.gram_addsub = (plan.use_gram || plan.use_gmt) && any_addsub;
     const bool add_kernels = any_add && !(plan.gram_addsub && !any_absdiff);
     if (plan.use_gram) {
@@ -590,7 +582,6 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
   SelectArgs S{};
   double *Yd = nullptr;
   Tile *tmul = nullptr, *tadd = nullptr;
-  unsigned *tile_ctr = nullptr;
   const int64_t cap = plan.cap;
   const int64_t T = d->n_targets;
   if (launch && !d->y_on_device) sc.add(&Yd, (size_t)T * d->ld_y);
@@ -638,7 +629,6 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
   sc.add(&S.r_key, (size_t)n_lists * cap);
   sc.add(&tmul, plan.mul_tiles.size());
   sc.add(&tadd, plan.add_tiles.size());
-  sc.add(&tile_ctr, 2);
   sc.add(&plan.bsplit, plan.use_tc ? tc_bsplit_bytes(plan.ntp, (int)N) : 1);
   unsigned char *gram_scr = nullptr;
   sc.add(&plan.gram_tiles_dev, plan.gram_tiles.size());
@@ -737,7 +727,7 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
   S.stats = R->stats;
 
   if (launch) {
-    s = run_screen(R, plan, tmul, tadd, A, S, tile_ctr);
+    s = run_screen(R, plan, tmul, tadd, A, S);
     if (s != DSE_OK) return fail(s);
   }
 
@@ -750,13 +740,13 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
                               : plan.use_tc && !plan.mul_tiles.empty()   ? DSE_PATH_TENSOR
                               : !plan.mul_tiles.empty()                  ? DSE_PATH_CUDA_CORE
                                                                          : 0;
-  Keep *keep = new (std::nothrow) Keep{plan, A, S, tmul, tadd, tile_ctr};
+  Keep *keep = new (std::nothrow) Keep{plan, A, S, tmul, tadd};
   if (!keep) return fail(DSE_ENOMEM);
   R->keep = keep;
   R->keep_free = [](void *p) { delete reinterpret_cast<Keep *>(p); };
   R->rerun = [](dse_result *r) -> dse_status {
     Keep *k = reinterpret_cast<Keep *>(r->keep);
-    return run_screen(r, k->plan, k->tmul, k->tadd, k->A, k->S, k->tile_ctr);
+    return run_screen(r, k->plan, k->tmul, k->tadd, k->A, k->S);
   };
   R->add_total = plan.add_total;
   R->buf_count = A.B.count;
@@ -779,7 +769,7 @@ static dse_status screen_enqueue_target(dse_result *R, const double *Y, int64_t 
   R->launches = 1;
   R->fetched = false;
   R->reruns = 0;
-  return run_screen(R, k->plan, k->tmul, k->tadd, k->A, k->S, k->tile_ctr);
+  return run_screen(R, k->plan, k->tmul, k->tadd, k->A, k->S);
 }
 
 // The statistics of a finished screen from its device counters (stats,

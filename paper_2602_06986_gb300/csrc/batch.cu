@@ -251,12 +251,17 @@ dse_status plan(const dse_batch_item *items, int32_t n, const dse_batch_desc *d,
   }
   b->ldy = (int32_t)ldy;
 
-  // jobs, tiles, pair lists
+  // jobs, tiles, pair lists; the problems by falling sample count, so that the
+  // longest tiles start first and the CTAs' static shares end together
+  const int BI = b->prec64 ? 32 : 16, BJ = 32;  // the batched pair kernels' tiles (PairCfg)
+  std::vector<int> order(n);
+  for (int p = 0; p < n; ++p) order[p] = p;
+  std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->spaces[x]->N > b->spaces[y]->N; });
   std::vector<Job> fjobs, pjobs;
   std::vector<Tile> mul, add;
   std::vector<int64_t> pair_off(n, 0), pair_cnt(n, 0);
   int64_t n_pairs = 0;
-  for (int p = 0; p < n; ++p) {
+  for (int p : order) {
     dse_space *sp = b->spaces[p];
     const RungGeom &g = sp->geom;
     b->total[p] = (uint64_t)sp->n + g.slots;
@@ -276,7 +281,7 @@ dse_status plan(const dse_batch_item *items, int32_t n, const dse_batch_desc *d,
     }
     if (any_mul) {
       const size_t t0 = mul.size();
-      triangle_tiles(g.o, g.n - 1, 32, 32, mul);
+      triangle_tiles(g.o, g.n - 1, BI, BJ, mul);
       for (size_t t = t0; t < mul.size(); ++t) mul[t].prob = p;
     }
     if (any_add) {
@@ -300,9 +305,9 @@ dse_status plan(const dse_batch_item *items, int32_t n, const dse_batch_desc *d,
         // products serves; else tiles over the unit classes
         const size_t t0 = add.size();
         if (one_class)
-          triangle_tiles(g.o, g.n - 1, 32, 32, add);
+          triangle_tiles(g.o, g.n - 1, BI, BJ, add);
         else
-          class_tiles(sp->h_class_begin, sp->n, 32, 32, 0, add);
+          class_tiles(sp->h_class_begin, sp->n, BI, BJ, 0, add);
         for (size_t t = t0; t < add.size(); ++t) add[t].prob = p;
       }
     }
@@ -445,11 +450,9 @@ dse_status plan(const dse_batch_item *items, int32_t n, const dse_batch_desc *d,
   b->A0_mul = L;
   b->A0_mul.tiles = b->tmul;
   b->A0_mul.n_tiles = b->n_mul;
-  b->A0_mul.tile_counter = b->counters + 1;
   b->A0_add = L;
   b->A0_add.tiles = b->tadd;
   b->A0_add.n_tiles = b->n_add;
-  b->A0_add.tile_counter = b->counters + 2;
 
   S.B = B;
   S.n_lists = n;

@@ -201,7 +201,6 @@ struct ScreenArgs {
   // pair kernels
   const Tile *tiles;
   int32_t n_tiles;
-  unsigned int *tile_counter;
   const int32_t *rowid;
   int32_t slot_pos[6];         // flat slot position of each binary op code 6..11 (-1 = off)
   int32_t first_pass;          // count statistics and escalate only in the first target pass

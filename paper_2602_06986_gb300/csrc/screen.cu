@@ -26,6 +26,7 @@
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "dse_internal.cuh"
 #include "eval64.cuh"
@@ -1103,6 +1104,402 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && NT == 1) ? 2 : 1)
   if (cur >= 0) flush_stats(BATCH ? batch[cur] : A0, ls, kGroup);
 }
 
+// ------------------------------------- FP32 pairs, one to eight targets
+
+// Two FP32 values in one 64-bit register pair and the packed FP32
+// instructions on them: each half is rounded exactly as the scalar
+// instruction rounds it, at half the issue slots.
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 f2_pack(float x, float y) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float f2_half(F2 v, int h) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+  return h ? y : x;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
+// A CTA of 4 warps owns a tile of 8 MI x 32 operand rows; warp w owns the
+// j-rows 8 w .. 8 w + 7 and a lane MI x 2 pairs, all three slots, for the
+// whole sample range.  The kernel is bound by the FP32 pipe (an evaluation
+// and 2 + NT sums a candidate and sample).  What kept the former kernel (32 x
+// 32 rows, 8 warps, operands by bulk copies into a ring) at 37% of it:
+//   * issue slots: with scalar instructions, reciprocals in every lane and
+//     copies between registers, 62% of the slots went to a pipe 51% busy.
+//     Here the pairs (r, 0), (r, 1) share packed registers, and the operands
+//     lie in shared memory as the packed instructions want them: a sample of
+//     an i-row is {a, a, 1/a, 1/a}, of a pair of j-rows {b0, b1, 1/b0, 1/b1}
+//     (sums: centred and plain values), of a target {y, y}; the CTA builds
+//     them once a 32-sample chunk from rows read ahead into registers.  A
+//     sample then takes 24 packed instructions and 4 loads a warp: 65 cycles
+//     at 4 warps a scheduler, 77 at one (95 with packed sums alone);
+//   * the tail: 1.5 large tiles a CTA slot left SMs idle for 28% of the
+//     launch.  The tiles are half the size, one CTA each, handed out by the
+//     hardware as others end;
+//   * 12 unrolled copies of the scoring code, which overflowed the
+//     instruction cache.
+// Block totals lie in shared memory, [sum][thread].
+// N = 9973, 449 k pairs, one target: 3.86 -> 2.61 ms a launch; the 256-problem
+// batch: 48.9 -> 35 ms; 4 targets, N = 1000, 224 k pairs: 874 -> 320 us.
+template <int NT, int MI>
+struct PackedPairCfg {
+  static constexpr int WARPS = 4, THREADS = 32 * WARPS;
+  static constexpr int BI = 8 * MI, BJ = 32, CH = 32;
+  static constexpr int A_Q = CH * BI, B_Q = CH * (BJ / 2);      // 16-byte quads a buffer
+  static constexpr int BUF = 16 * (A_Q + B_Q) + 8 * CH * NT;    // bytes
+  static constexpr int SUMS = MI * 3 * (2 + NT);                // packed sums a lane
+  static constexpr size_t SMEM = 2 * (size_t)BUF + (size_t)SUMS * THREADS * 8;
+  static constexpr int MIN_CTAS = NT > 4 ? 3 : 4;
+};
+
+// A lane's shift constants and running sums of its MI x 2 pairs.
+template <int KIND, int NT, int MI>
+struct PairSums {
+  static constexpr int STRIDE = PackedPairCfg<NT, MI>::THREADS;
+  F2 nk0[MI], nk1[MI], nk2[MI];  // negated shift constants (sums: the last only)
+  F2 acc[MI][3][2 + NT];
+  F2 *tot;  // this lane's block totals
+  __device__ __forceinline__ void zero() {
+#pragma unroll
+    for (int r = 0; r < MI; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int e = 0; e < 2 + NT; ++e) {
+          acc[r][k][e] = 0ull;
+          tot[((r * 3 + k) * (2 + NT) + e) * STRIDE] = 0ull;
+        }
+  }
+  // A: a sample's quads of the lane's i-rows, B: of its j-rows, Y: targets
+  __device__ __forceinline__ void update(const ulonglong2 (&A)[MI], const ulonglong2 &B, const F2 (&Y)[NT]) {
+    const F2 minus = f2_pack(-1.f, -1.f);
+    F2 w[MI][3];
+#pragma unroll
+    for (int r = 0; r < MI; ++r) {
+      if (KIND == KIND_MUL) {
+        w[r][0] = f2_fma(A[r].x, B.x, nk0[r]);
+        w[r][1] = f2_fma(A[r].x, B.y, nk1[r]);
+        w[r][2] = f2_fma(B.x, A[r].y, nk2[r]);
+      } else {
+        // (a product by -1 is exact: one rounding, as in a subtraction)
+        w[r][0] = f2_add(A[r].x, B.x);
+        w[r][1] = f2_fma(B.x, minus, A[r].x);
+        w[r][2] = f2_add(f2_fma(B.y, minus, A[r].y) & 0x7fffffff7fffffffull, nk2[r]);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < MI; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        acc[r][k][0] = f2_add(acc[r][k][0], w[r][k]);
+        acc[r][k][1] = f2_fma(w[r][k], w[r][k], acc[r][k][1]);
+#pragma unroll
+        for (int t = 0; t < NT; ++t) acc[r][k][2 + t] = f2_fma(w[r][k], Y[t], acc[r][k][2 + t]);
+      }
+  }
+  // the block's sums into the totals
+  __device__ __forceinline__ void fold() {
+#pragma unroll
+    for (int r = 0; r < MI; ++r)
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int e = 0; e < 2 + NT; ++e) {
+          F2 &t = tot[((r * 3 + k) * (2 + NT) + e) * STRIDE];
+          t = f2_add(t, acc[r][k][e]);
+          acc[r][k][e] = 0ull;
+        }
+  }
+  // (run-time indices: the epilogue is a loop over the lane's pairs)
+  __device__ __forceinline__ float total(int r, int c, int k, int e) const {
+    return reinterpret_cast<const float *>(&tot[((r * 3 + k) * (2 + NT) + e) * STRIDE])[c];
+  }
+};
+
+// BATCH: the tiles of every problem of a batched screen; each names its
+// problem, whose arguments are read from `batch`.
+template <int KIND, int NT, int MI, bool BATCH>
+__global__ void __launch_bounds__(PackedPairCfg<NT, MI>::THREADS, PackedPairCfg<NT, MI>::MIN_CTAS)
+    k_pair_packed(const ScreenArgs A0, const ScreenArgs *batch, int block_len0) {
+  using C = PackedPairCfg<NT, MI>;
+  constexpr int MJ = 2;
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, li = lane >> 2, lj = lane & 3;
+  const float u = 5.9604644775390625e-8f;
+  const Tile tl = A0.tiles[blockIdx.x];
+  const ScreenArgs &A = BATCH ? batch[tl.prob] : A0;
+  const int block_len = BATCH ? A.block_len : block_len0;
+  const int n_smp = A.N, nchunks = (n_smp + C::CH - 1) / C::CH;
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto row_i = [&](int r) -> int { return r < tl.ni ? A.rowid[tl.ibase + r] : -1; };
+  auto row_j = [&](int r) -> int { return r < tl.nj ? A.rowid[tl.jbase + r] : -1; };
+
+  // this thread's share of a chunk: four samples (group q) of one i-row, of
+  // the j-rows that make pair p, and of one target
+  const int pr = tid % C::BI, pq = tid / C::BI, p = tid & 15, q = tid >> 4, yt = tid % NT, yq = tid / NT;
+  const float *src_a = nullptr, *src_b0 = nullptr, *src_b1 = nullptr, *src_y = nullptr;
+  float ca = 0.f, cb0 = 0.f, cb1 = 0.f;  // (sums) the rows' means
+  {
+    const int ia = pq < 8 ? row_i(pr) : -1, ib0 = row_j((p >> 2) * 8 + (p & 3)), ib1 = row_j((p >> 2) * 8 + (p & 3) + 4);
+    if (ia >= 0) src_a = A.F.v32 + (int64_t)ia * A.F.ld + 4 * pq, ca = A.F.fa[ia].x;
+    if (ib0 >= 0) src_b0 = A.F.v32 + (int64_t)ib0 * A.F.ld + 4 * q, cb0 = A.F.fa[ib0].x;
+    if (ib1 >= 0) src_b1 = A.F.v32 + (int64_t)ib1 * A.F.ld + 4 * q, cb1 = A.F.fa[ib1].x;
+    if (yq < 8 && yt < A.T) src_y = A.y32 + (int64_t)(A.t0 + yt) * A.ldy + 4 * yq;
+  }
+  const int ld = (int)A.F.ld, ldy = A.ldy;
+  float4 va = none, vb0 = none, vb1 = none, vy = none;
+  auto fetch = [&](int c) {
+    const int s0 = c * C::CH;
+    if (c < nchunks) {
+      va = src_a && s0 + 4 * pq < ld ? __ldg(reinterpret_cast<const float4 *>(src_a + s0)) : none;
+      const bool in = s0 + 4 * q < ld;
+      vb0 = src_b0 && in ? __ldg(reinterpret_cast<const float4 *>(src_b0 + s0)) : none;
+      vb1 = src_b1 && in ? __ldg(reinterpret_cast<const float4 *>(src_b1 + s0)) : none;
+      vy = src_y && s0 + 4 * yq < ldy ? *reinterpret_cast<const float4 *>(src_y + s0) : none;
+    }
+  };
+  auto store = [&](int buf) {
+    unsigned char *B0 = smem_raw + buf * C::BUF;
+    float4 *qa = reinterpret_cast<float4 *>(B0), *qb = qa + C::A_Q;
+    float2 *qy = reinterpret_cast<float2 *>(qb + C::B_Q);
+    const float a4[4] = {va.x, va.y, va.z, va.w}, b4[4] = {vb0.x, vb0.y, vb0.z, vb0.w},
+                d4[4] = {vb1.x, vb1.y, vb1.z, vb1.w}, y4[4] = {vy.x, vy.y, vy.z, vy.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (pq < 8) {
+        const float z = KIND == KIND_MUL ? rcp_approx(a4[i]) : a4[i] - ca;
+        qa[(4 * pq + i) * C::BI + pr] = KIND == KIND_MUL ? make_float4(a4[i], a4[i], z, z) : make_float4(z, z, a4[i], a4[i]);
+      }
+      const float z0 = KIND == KIND_MUL ? rcp_approx(b4[i]) : b4[i] - cb0,
+                  z1 = KIND == KIND_MUL ? rcp_approx(d4[i]) : d4[i] - cb1;
+      qb[(4 * q + i) * 16 + p] = KIND == KIND_MUL ? make_float4(b4[i], d4[i], z0, z1) : make_float4(z0, z1, b4[i], d4[i]);
+      if (yq < 8) qy[(4 * yq + i) * NT + yt] = make_float2(y4[i], y4[i]);
+    }
+  };
+
+  // the lane's pairs: i-rows li + 8 r, j-rows 8 warp + lj + 4 c; a warp whose
+  // pairs all lie above the diagonal or past the tile's rows only helps to copy
+  const bool busy = warp * 8 < tl.nj && tl.jbase + warp * 8 < tl.ibase + tl.ni - 1;
+  PairSums<KIND, NT, MI> ps;
+  ps.tot = reinterpret_cast<F2 *>(smem_raw + 2 * C::BUF) + tid;
+  {
+    float4 fj[MJ];
+#pragma unroll
+    for (int c = 0; c < MJ; ++c) {
+      const int f = row_j(8 * warp + lj + 4 * c);
+      fj[c] = f >= 0 ? A.F.fa[f] : none;
+    }
+#pragma unroll
+    for (int r = 0; r < MI; ++r) {
+      const int f = row_i(li + 8 * r);
+      const float4 fi = f >= 0 ? A.F.fa[f] : none;
+      ps.nk0[r] = f2_pack(-(fi.x * fj[0].x), -(fi.x * fj[1].x));
+      ps.nk1[r] = f2_pack(-(fi.x * fj[0].y), -(fi.x * fj[1].y));
+      ps.nk2[r] = KIND == KIND_MUL ? f2_pack(-(fj[0].x * fi.y), -(fj[1].x * fi.y))
+                                   : f2_pack(-fabsf(fi.x - fj[0].x), -fabsf(fi.x - fj[1].x));
+    }
+  }
+  ps.zero();
+
+  fetch(0);
+  store(0);
+  fetch(1);
+  __syncthreads();
+  int blk = 0;
+  for (int ch = 0; ch < nchunks; ++ch) {
+    if (ch + 1 < nchunks) {
+      store((ch + 1) & 1);  // (read last in the chunk before this one)
+      fetch(ch + 2);
+    }
+    if (busy) {
+      const unsigned char *B0 = smem_raw + (ch & 1) * C::BUF;
+      const ulonglong2 *qa = reinterpret_cast<const ulonglong2 *>(B0) + li;
+      const ulonglong2 *qb = reinterpret_cast<const ulonglong2 *>(B0) + C::A_Q + warp * 4 + lj;
+      const F2 *qy = reinterpret_cast<const F2 *>(B0 + 16 * (C::A_Q + C::B_Q));
+      const int ns = min(C::CH, n_smp - ch * C::CH);
+      auto sample = [&](int s) {
+        ulonglong2 Aq[MI];
+        F2 Yq[NT];
+#pragma unroll
+        for (int r = 0; r < MI; ++r) Aq[r] = qa[s * C::BI + 8 * r];
+#pragma unroll
+        for (int t = 0; t < NT; ++t) Yq[t] = qy[s * NT + t];
+        ps.update(Aq, qb[s * 16], Yq);
+      };
+      // (straight-line groups of samples: in a loop of one or two samples the
+      // compiler rotates the operands through registers, 13 moves a turn)
+      auto samples = [&](int s, auto n) {
+#pragma unroll
+        for (int i = 0; i < decltype(n)::value; ++i) sample(s + i);
+        asm volatile("" ::: "memory");
+      };
+      for (int s = 0; s < ns;) {
+        // to the end of the chunk or of the summation block
+        const int e = min(ns, s + block_len - blk);
+        blk += e - s;
+#pragma unroll 1
+        for (; s + 8 <= e; s += 8) samples(s, std::integral_constant<int, 8>());
+        if (e - s >= 4) {
+          samples(s, std::integral_constant<int, 4>());
+          s += 4;
+        }
+        if (e - s >= 2) {
+          samples(s, std::integral_constant<int, 2>());
+          s += 2;
+        }
+        if (e - s >= 1) {
+          samples(s, std::integral_constant<int, 1>());
+          s += 1;
+        }
+        if (blk >= block_len) {
+          blk = 0;
+          ps.fold();
+        }
+      }
+    }
+    __syncthreads();
+  }
+  if (!busy) return;
+  ps.fold();
+
+  // ------------------------------------------------------------ epilogue
+  LaneStats ls;
+  ls.zero();
+  const float gamma = A.gamma;
+  const float N = (float)A.N, invN = (float)A.invN, sqrtN = sqrtf(N);
+  const float fmin = (float)A.fmin_std_rel64;
+  float ysum[NT];
+  load_ysum<float, NT>(A, ysum);
+#pragma unroll 1
+  for (int e = 0; e < MI * MJ; ++e) {
+    const int r = e / MJ, c = e % MJ;
+    const int64_t x = row_i(li + 8 * r), y = row_j(8 * warp + lj + 4 * c);
+    bool pv = x >= 0 && y >= 0 && tl.ibase + li + 8 * r > tl.jbase + 8 * warp + lj + 4 * c;
+    const int64_t ia = x > y ? x : y, ib = x > y ? y : x;
+    pv = pv && ia >= A.G.o;
+    uint64_t pbase = 0;
+    if (pv) pbase = A.G.um + (tri((uint64_t)ia) + (uint64_t)ib - A.G.tri_o) * (uint64_t)A.G.nb;
+    const float4 fx = x >= 0 ? A.F.fa[x] : none, fy = y >= 0 ? A.F.fa[y] : none;
+    unsigned pushed = 0;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int opc = KIND == KIND_MUL ? (k == 0 ? DSE_OP_MUL : k == 1 ? DSE_OP_DIV : DSE_OP_RDIV)
+                                       : (k == 0 ? DSE_OP_ADD : k == 1 ? DSE_OP_SUB : DSE_OP_ABSDIFF);
+      const float kk = k == 0 ? fx.x * fy.x : k == 1 ? fx.x * fy.y : KIND == KIND_MUL ? fy.x * fx.y : fabsf(fx.x - fy.x);
+      float Sy[NT];
+#pragma unroll
+      for (int t = 0; t < NT; ++t) Sy[t] = ps.total(r, c, k, 2 + t);
+      pushed |= binary_candidate<float, NT>(A, ls, true, pv, ia, ib, opc, pbase, x > y ? fx : fy, x > y ? fy : fx, kk,
+                                            fx.x, fy.x, ps.total(r, c, k, 0), ps.total(r, c, k, 1), Sy, N, invN,
+                                            sqrtN, gamma, u, fmin, ysum);
+    }
+    refresh_pushed<NT>(A, pushed);
+  }
+  flush_stats(A, ls, KIND == KIND_MUL ? 1 : 2);
+}
+
+// ------------------------------------------- FP64 pairs, one target
+//
+// The plain FP64 screen is bound by the FP64 pipe (2 operations a clock and
+// SM), so a tile needs few warps and what counts is that every SM has a tile
+// and that nothing is computed twice: a thread owns one pair of a T x T tile,
+// and the reciprocals (products) or centred values (sums) of the tile's 2 T
+// rows are taken once a chunk by the whole block.  With 32 x 32 tiles each
+// reciprocal was computed 16 times and a space of 185 features filled 26 of
+// the 152 SMs: 2.40 ms a launch at N = 500, 17 k pairs (0.20 ms of FP64
+// multiply-adds).  The samples are summed in order, as k_pair sums them.
+constexpr int k64Chunk = 32;
+
+template <int KIND, int T>
+__global__ void __launch_bounds__(T *T) k_pair64(const ScreenArgs A) {
+  constexpr int ROWS = 2 * T, STR = ROWS + 1;  // sample-major, odd stride: neither loads nor stores conflict
+  __shared__ double xs[k64Chunk * STR], zs[k64Chunk * STR], ys[k64Chunk];
+  const int tid = threadIdx.x, ti = tid / T, tj = tid % T;
+  const Tile tl = A.tiles[blockIdx.x];
+  auto row_id = [&](int r) -> int {
+    if (r < T) return r < tl.ni ? A.rowid[tl.ibase + r] : -1;
+    return r - T < tl.nj ? A.rowid[tl.jbase + r - T] : -1;
+  };
+  const int64_t x = row_id(ti), y = row_id(T + tj);
+  const double mi = x >= 0 ? A.F.mean64[x] : 0.0, mj = y >= 0 ? A.F.mean64[y] : 0.0;
+  const double rmi = x >= 0 ? A.F.rmean64[x] : 0.0, rmj = y >= 0 ? A.F.rmean64[y] : 0.0;
+  double k[3] = {mi * mj, mi * rmj, KIND == KIND_MUL ? mj * rmi : (mi - mj < 0.0 ? mj - mi : mi - mj)};
+  double acc[3][3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) acc[q][0] = acc[q][1] = acc[q][2] = 0.0;
+  const double *yrow = A.y64 + (int64_t)A.t0 * A.ldy;
+  for (int s0 = 0; s0 < A.N; s0 += k64Chunk) {
+    const int ns = min(k64Chunk, A.N - s0);
+    __syncthreads();
+    for (int e = tid; e < ROWS * k64Chunk; e += T * T) {
+      const int r = e / k64Chunk, s = e % k64Chunk;
+      const int f = row_id(r);
+      const double v = f >= 0 && s < ns ? A.F.v64[(int64_t)f * A.F.ld + s0 + s] : 1.0;
+      xs[s * STR + r] = v;
+      zs[s * STR + r] = KIND == KIND_MUL ? __drcp_rn(v) : v - (f >= 0 ? A.F.mean64[f] : 0.0);
+    }
+    if (tid < ns) ys[tid] = yrow[s0 + tid];
+    __syncthreads();
+#pragma unroll 4
+    for (int s = 0; s < ns; ++s) {
+      const double a = xs[s * STR + ti], b = xs[s * STR + T + tj], za = zs[s * STR + ti], zb = zs[s * STR + T + tj];
+      double w[3];
+      if (KIND == KIND_MUL) {
+        w[0] = fma(a, b, -k[0]);
+        w[1] = fma(a, zb, -k[1]);
+        w[2] = fma(b, za, -k[2]);
+      } else {
+        const double d = a - b;
+        w[0] = za + zb;
+        w[1] = za - zb;
+        w[2] = (d < 0.0 ? -d : d) - k[2];
+      }
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        acc[q][0] += w[q];
+        acc[q][1] = fma(w[q], w[q], acc[q][1]);
+        acc[q][2] = fma(w[q], ys[s], acc[q][2]);
+      }
+    }
+  }
+  LaneStats ls;
+  ls.zero();
+  const double u = 1.1102230246251565e-16;
+  const double N = (double)A.N, invN = A.invN, sqrtN = sqrt(N);
+  double ysum[1] = {0.0};
+  bool pv = x >= 0 && y >= 0 && (tl.ibase + ti) > (tl.jbase + tj);
+  const int64_t ia = x > y ? x : y, ib = x > y ? y : x;
+  pv = pv && ia >= A.G.o;
+  const uint64_t pbase = pv ? A.G.um + (tri((uint64_t)ia) + (uint64_t)ib - A.G.tri_o) * (uint64_t)A.G.nb : 0;
+  const float4 none = make_float4(0.f, 0.f, 0.f, 0.f);
+  const float4 fa_a = ia >= 0 ? A.F.fa[ia] : none, fa_b = ib >= 0 ? A.F.fa[ib] : none;
+  unsigned pushed = 0;
+#pragma unroll 1
+  for (int q = 0; q < 3; ++q) {
+    const int opc = (KIND == KIND_MUL ? DSE_OP_MUL : DSE_OP_ADD) + (KIND == KIND_ADD && q == 2 ? 5 : q);
+    const double Sy[1] = {0.0 + (q == 0 ? acc[0][2] : q == 1 ? acc[1][2] : acc[2][2])};
+    pushed |= binary_candidate<double, 1>(A, ls, true, pv, ia, ib, opc, pbase, fa_a, fa_b,
+                                          q == 0 ? k[0] : q == 1 ? k[1] : k[2], mi, mj,
+                                          0.0 + (q == 0 ? acc[0][0] : q == 1 ? acc[1][0] : acc[2][0]),
+                                          0.0 + (q == 0 ? acc[0][1] : q == 1 ? acc[1][1] : acc[2][1]), Sy, N, invN,
+                                          sqrtN, (double)A.gamma, u, A.fmin_std_rel64, ysum);
+  }
+  refresh_pushed<1>(A, pushed);
+  flush_stats(A, ls);
+}
+
 // ------------------------------------------------ explicit pair lists
 
 // The additive slots (a+b, a-b, |a-b|) of an explicit list of pairs (i > j,
@@ -1757,6 +2154,27 @@ dse_status launch_pair_t(const ScreenArgs &A, int block_len, int sms, cudaStream
   return DSE_OK;
 }
 
+// block_len: see accum_factors (batched: in each problem's arguments)
+template <int KIND, int NT, int MI, bool BATCH = false>
+dse_status launch_pair_packed(const ScreenArgs &A, int block_len, cudaStream_t st,
+                              const ScreenArgs *batch = nullptr) {
+  using C = PackedPairCfg<NT, MI>;
+  if (A.n_tiles <= 0) return DSE_OK;
+  static bool attr[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!attr[dev & 63]) {
+    DSE_CUDA(cudaFuncSetAttribute(k_pair_packed<KIND, NT, MI, BATCH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)C::SMEM));
+    attr[dev & 63] = true;
+  }
+  note_launches(1);
+  ScreenArgs B = A;
+  B.group = KIND == KIND_MUL ? 1 : 2;
+  k_pair_packed<KIND, NT, MI, BATCH><<<A.n_tiles, C::THREADS, C::SMEM, st>>>(B, batch, block_len);
+  return DSE_OK;
+}
+
 void launch_feature(int prec64, int nt, const ScreenArgs &A, uint64_t id0, uint64_t id1, uint64_t p0, uint64_t p1,
                     float gamma, int sms, cudaStream_t st) {
   if (prec64) {
@@ -1768,17 +2186,50 @@ void launch_feature(int prec64, int nt, const ScreenArgs &A, uint64_t id0, uint6
   }
 }
 
-dse_status launch_pair(int prec64, int kind, int nt, const ScreenArgs &A, int block_len, int sms, cudaStream_t st) {
+// Targets the pair kernel of a screen with T targets sums side by side: the
+// kernels cost about 3 + nt operations a candidate and sample, so a few
+// targets take a few-target kernel (4 targets at N = 1000, 224 k pairs: 16
+// targets' sums took 874 us).
+int pair_targets(int prec64, int T) { return T == 1 ? 1 : prec64 || T > 8 ? 16 : T > 4 ? 8 : 4; }
+
+// Operand rows of a pair tile (n_pairs pairs in the screen).  FP64, one
+// target: a thread owns one pair; tiles of 16 x 16 share each row's
+// reciprocals among 16 pairs, tiles of 8 x 8 fill the SMs when there are
+// fewer than 8 large tiles for each.
+void pair_tile_shape(int prec64, int npt, int64_t n_pairs, int sms, int *BI, int *BJ) {
+  if (prec64 && npt == 1) *BI = *BJ = n_pairs >= (int64_t)sms * 8 * 256 ? 16 : 8;
+  else if (prec64 || npt == 16) *BI = *BJ = 16;
+  else *BI = npt == 1 ? 16 : 8, *BJ = 32;
+}
+
+template <int KIND>
+static dse_status launch_pair64(const ScreenArgs &A, int tile, cudaStream_t st) {
+  if (A.n_tiles <= 0) return DSE_OK;
+  ScreenArgs B = A;
+  B.group = KIND == KIND_MUL ? 1 : 2;
+  note_launches(1);
+  if (tile == 16) k_pair64<KIND, 16><<<A.n_tiles, 256, 0, st>>>(B);
+  else k_pair64<KIND, 8><<<A.n_tiles, 64, 0, st>>>(B);
+  return DSE_OK;
+}
+
+dse_status launch_pair(int prec64, int kind, int nt, int tile_rows, const ScreenArgs &A, int block_len, int sms,
+                       cudaStream_t st) {
   if (prec64) {
     if (nt == 1)
-      return kind == KIND_MUL ? launch_pair_t<double, KIND_MUL, 1, 2, 2>(A, block_len, sms, st)
-                              : launch_pair_t<double, KIND_ADD, 1, 2, 2>(A, block_len, sms, st);
+      return kind == KIND_MUL ? launch_pair64<KIND_MUL>(A, tile_rows, st) : launch_pair64<KIND_ADD>(A, tile_rows, st);
     return kind == KIND_MUL ? launch_pair_t<double, KIND_MUL, 16, 1, 1>(A, block_len, sms, st)
                             : launch_pair_t<double, KIND_ADD, 16, 1, 1>(A, block_len, sms, st);
   }
   if (nt == 1)
-    return kind == KIND_MUL ? launch_pair_t<float, KIND_MUL, 1, 2, 2>(A, block_len, sms, st)
-                            : launch_pair_t<float, KIND_ADD, 1, 2, 2>(A, block_len, sms, st);
+    return kind == KIND_MUL ? launch_pair_packed<KIND_MUL, 1, 2>(A, block_len, st)
+                            : launch_pair_packed<KIND_ADD, 1, 2>(A, block_len, st);
+  if (nt == 4)
+    return kind == KIND_MUL ? launch_pair_packed<KIND_MUL, 4, 1>(A, block_len, st)
+                            : launch_pair_packed<KIND_ADD, 4, 1>(A, block_len, st);
+  if (nt == 8)
+    return kind == KIND_MUL ? launch_pair_packed<KIND_MUL, 8, 1>(A, block_len, st)
+                            : launch_pair_packed<KIND_ADD, 8, 1>(A, block_len, st);
   return kind == KIND_MUL ? launch_pair_t<float, KIND_MUL, 16, 1, 1>(A, block_len, sms, st)
                           : launch_pair_t<float, KIND_ADD, 16, 1, 1>(A, block_len, sms, st);
 }
@@ -1823,8 +2274,8 @@ dse_status launch_pair_batched(int prec64, int kind, const ScreenArgs &A0, const
   if (prec64)
     return kind == KIND_MUL ? launch_pair_t<double, KIND_MUL, 1, 2, 2, true>(A0, 0, sms, st, args)
                             : launch_pair_t<double, KIND_ADD, 1, 2, 2, true>(A0, 0, sms, st, args);
-  return kind == KIND_MUL ? launch_pair_t<float, KIND_MUL, 1, 2, 2, true>(A0, 0, sms, st, args)
-                          : launch_pair_t<float, KIND_ADD, 1, 2, 2, true>(A0, 0, sms, st, args);
+  return kind == KIND_MUL ? launch_pair_packed<KIND_MUL, 1, 2, true>(A0, 0, st, args)
+                          : launch_pair_packed<KIND_ADD, 1, 2, true>(A0, 0, st, args);
 }
 
 void launch_pairlist_batched(int prec64, const ScreenArgs *args, const int2 *pairs, const Job *jobs, int n_jobs,

@@ -11,7 +11,11 @@ void launch_targets(const double *Y, int64_t ldY, int T, int64_t N, int32_t ldy,
                     float2 *ydf, float *ysum32, int *err, cudaStream_t st);
 void launch_feature(int prec64, int nt, const ScreenArgs &A, uint64_t id0, uint64_t id1, uint64_t p0, uint64_t p1,
                     float gamma, int sms, cudaStream_t st);
-dse_status launch_pair(int prec64, int kind, int nt, const ScreenArgs &A, int block_len, int sms, cudaStream_t st);
+// nt: pair_targets of the screen; tile_rows: the i-rows of its tiles.
+dse_status launch_pair(int prec64, int kind, int nt, int tile_rows, const ScreenArgs &A, int block_len, int sms,
+                       cudaStream_t st);
+int pair_targets(int prec64, int T);
+void pair_tile_shape(int prec64, int npt, int64_t n_pairs, int sms, int *BI, int *BJ);
 void launch_escalate(const ScreenArgs &A, int sms, cudaStream_t st, const ScreenArgs *batch = nullptr);
 // With A.why: the reason of the candidates no kernel visits (additive slots
 // of pairs with unequal units).

@@ -125,6 +125,30 @@ void triangle_tiles(int64_t ia, int64_t ib, int BI, int BJ, std::vector<Tile> &o
   }
 }
 
+// Tiles of the tensor-core kernel (128 pairs: 16 x 8, 8 x 16 or 4 x 32 rows,
+// which the kernel tells apart by ni) over the pairs from (ia, ja) to (ib, jb).
+// A block of 16 rows costs J / 8 tiles, one of 8 J / 16, one of 4 J / 32: the
+// last rows of a range (a block of ids holds few long rows) take the shapes
+// that cost least.  A first or last row by itself is cut to its own j's.
+static void tc_tiles(int64_t ia, int64_t ja, int64_t ib, int64_t jb, std::vector<Tile> &out) {
+  for (int64_t i0 = ia; i0 <= ib;) {
+    const int64_t left = ib - i0 + 1;
+    const int64_t BI = left > 12 ? 16 : left > 4 ? 8 : 4, BJ = 128 / BI;
+    const int64_t i1 = std::min(i0 + BI, ib + 1);
+    const int64_t jlo = i1 - 1 == ia ? ja : 0, jhi = i0 == ib ? jb + 1 : i1 - 1;
+    for (int64_t j0 = jlo; j0 < jhi; j0 += BJ) {
+      Tile t;
+      t.ibase = (int32_t)i0;
+      t.ni = (int16_t)(i1 - i0);
+      t.jbase = (int32_t)j0;
+      t.nj = (int16_t)std::min<int64_t>(BJ, jhi - j0);
+      t.prob = 0;
+      out.push_back(t);
+    }
+    i0 = i1;
+  }
+}
+
 // Order pair tiles so that the tiles resident at the same time share their
 // operand rows: groups of G consecutive i-blocks, j-block major inside a
 // group.  A wave of one CTA per SM then covers a compact block of the
@@ -156,7 +180,6 @@ struct ScreenPlan {
   // tensor-core path (BF16x3 contraction of the binary block)
   bool use_tc = false;
   int ntp = 0, tc_passes = 0, gen_blk = 1;
-  int32_t n_seed_tiles = 0;      // leading product/quotient tiles launched first
   float gamma_gen = 0.f, gamma_num = 0.f;
   unsigned char *bsplit = nullptr;
   // Gram path of the product/quotient slots (single-target FP32 screens)
@@ -234,18 +257,11 @@ static dse_status run_tc_passes(dse_result *R, const ScreenPlan &plan, void *scr
         launch_rcp_rows(sp->v32, cnt, sp->rcp32, sms, st);
       }
       A.rowid = sp->rowid_ident;
-      const Tile *t0p = reinterpret_cast<const Tile *>(scr_tiles_mul);
-      const int32_t nall = (int32_t)plan.mul_tiles.size(), ns = plan.n_seed_tiles;
-      if (ns > 0) {
-        A.tiles = t0p;
-        A.n_tiles = ns;
-        DSE_TRY(launch_pair_tc(KIND_MUL, plan.ntp, A, plan.bsplit, sp->v32, sp->rcp32, sp->n, plan.gamma_gen, plan.gamma_num, plan.gen_blk,
-                               sms, st));
-      }
-      A.tiles = t0p + ns;
-      A.n_tiles = nall - ns;
-      DSE_TRY(launch_pair_tc(KIND_MUL, plan.ntp, A, plan.bsplit, sp->v32, sp->rcp32, sp->n, plan.gamma_gen, plan.gamma_num, plan.gen_blk, sms,
-                             st));
+      // (one launch: the CTAs take the leading seed tiles first)
+      A.tiles = reinterpret_cast<const Tile *>(scr_tiles_mul);
+      A.n_tiles = (int32_t)plan.mul_tiles.size();
+      DSE_TRY(launch_pair_tc(KIND_MUL, plan.ntp, A, plan.bsplit, sp->v32, sp->rcp32, sp->n, plan.gamma_gen,
+                             plan.gamma_num, plan.gen_blk, sms, st));
     }
     DSE_TRY(mark(2));
     if (!plan.use_pairlist && !plan.add_tiles.empty()) {
@@ -492,20 +508,21 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
     } else if (plan.use_gmt) {
       gmt_tiles(sp, id_begin, id_end, plan.gmt_tiles);
     } else if (any_mul) {
-      triangle_tiles((int64_t)ia, (int64_t)ib2, BI, BJ, plan.mul_tiles);
+      if (plan.use_tc)
+        tc_tiles((int64_t)ia, (int64_t)ja, (int64_t)ib2, (int64_t)jb, plan.mul_tiles);
+      else
+        triangle_tiles((int64_t)ia, (int64_t)ib2, BI, BJ, plan.mul_tiles);
       const Tuning tn = tuning();
       group_tiles(plan.mul_tiles, (int64_t)ia, BI, plan.use_tc ? tn.tile_group_tc : tn.tile_group_cc);
-      // A large tile list is launched in two parts: every seed_stride-th
-      // tile first (64 by default), so that the thresholds have risen from a
-      // spread sample of the space before the bulk of the candidates is
-      // filtered.
+      // A large tile list starts with every seed_stride-th tile (64 by
+      // default), so that the thresholds rise from a spread sample of the
+      // space.
       const size_t nt = plan.mul_tiles.size(), stride = (size_t)tn.seed_stride;
       if (nt >= 64 * stride) {
         std::vector<Tile> seed, rest;
         seed.reserve(nt / stride + 1);
         rest.reserve(nt);
         for (size_t t = 0; t < nt; ++t) (t % stride == 0 ? seed : rest).push_back(plan.mul_tiles[t]);
-        plan.n_seed_tiles = (int32_t)seed.size();
         seed.insert(seed.end(), rest.begin(), rest.end());
         plan.mul_tiles.swap(seed);
       }
@@ -515,7 +532,10 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
       if (one_class) {
         // every pair may be added: the same id triangle as the products,
         // restricted to the rows of the range
-        triangle_tiles((int64_t)ia, (int64_t)ib2, BI, BJ, plan.add_tiles);
+        if (plan.use_tc)
+          tc_tiles((int64_t)ia, (int64_t)ja, (int64_t)ib2, (int64_t)jb, plan.add_tiles);
+        else
+          triangle_tiles((int64_t)ia, (int64_t)ib2, BI, BJ, plan.add_tiles);
         plan.add_by_id = true;
       } else {
         // sparse equal-unit pairs: an explicit list (built once per space);

@@ -335,6 +335,31 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return r;
 }
 
+// Two FP32 values in one 64-bit register pair and the packed FP32
+// instructions on them: each half is rounded exactly as the scalar
+// instruction rounds it, at half the issue slots.
+typedef unsigned long long F2;
+__device__ __forceinline__ F2 f2_pack(float x, float y) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float f2_half(F2 v, int h) {
+  float x, y;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+  return h ? y : x;
+}
+__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+
 // Raise a non-negative float threshold monotonically.
 __device__ __forceinline__ void atomic_max_nonneg(float *addr, float v) {
   atomicMax(reinterpret_cast<int *>(addr), __float_as_int(v));

@@ -1106,31 +1106,6 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && NT == 1) ? 2 : 1)
 
 // ------------------------------------- FP32 pairs, one to eight targets
 
-// Two FP32 values in one 64-bit register pair and the packed FP32
-// instructions on them: each half is rounded exactly as the scalar
-// instruction rounds it, at half the issue slots.
-typedef unsigned long long F2;
-__device__ __forceinline__ F2 f2_pack(float x, float y) {
-  F2 r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ float f2_half(F2 v, int h) {
-  float x, y;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
-  return h ? y : x;
-}
-__device__ __forceinline__ F2 f2_fma(F2 a, F2 b, F2 c) {
-  F2 r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-__device__ __forceinline__ F2 f2_add(F2 a, F2 b) {
-  F2 r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-
 // A CTA of 4 warps owns a tile of 8 MI x 32 operand rows; warp w owns the
 // j-rows 8 w .. 8 w + 7 and a lane MI x 2 pairs, all three slots, for the
 // whole sample range.  The kernel is bound by the FP32 pipe (an evaluation

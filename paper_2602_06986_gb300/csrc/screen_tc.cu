@@ -25,7 +25,7 @@
 //                 next to the value rows), FP32 S1/S2, BF16 hi/lo split,
 //                 16-byte stores into the canonical K-major layout (8x8 core
 //                 matrices, no swizzle), proxy fence, arrive;
-//   warps 10-13   epilogue: tcgen05.ld of TMEM lane quadrant (warp % 4),
+//   warps 10-17   epilogue: tcgen05.ld of TMEM lane quadrant (warp % 4),
 //                 block accumulation, scores, error bounds, threshold pushes.
 // Accumulators are double-buffered in TMEM by accumulation block (up to 16
 // chunks = 512 samples), so the epilogue of one block overlaps the MMAs of
@@ -56,25 +56,45 @@ namespace dse {
 namespace tc {
 
 constexpr int M = 128;  // pairs per tile
-constexpr int BI = 16, BJ = 8, ROWS = BI + BJ;
+// A tile is 16 x 8, 8 x 16 or 4 x 32 operand rows (the planner's choice, by
+// the rows left in a range: a 4 x 32 tile of a range that ends one row into
+// a 16-row block has 32 pairs where a 16 x 8 tile has 8).  The rows arrive in
+// boxes of eight: the i-rows, then the j-rows.
+constexpr int BOX = 8, MAX_BOXES = 5, ROWS = BOX * MAX_BOXES;
+struct Shape {
+  int log_nj;    // j-rows of a tile: 8, 16 or 32
+  int i_boxes, boxes;
+};
+__host__ __device__ inline Shape shape_of(const Tile &t) {
+  Shape s;
+  s.log_nj = t.ni > 8 ? 3 : t.ni > 4 ? 4 : 5;
+  s.i_boxes = t.ni > 8 ? 2 : 1;
+  s.boxes = s.i_boxes + (1 << (s.log_nj - 3));
+  return s;
+}
 constexpr int NS = 3;     // stages of the A operands (and, with A in shared memory, of everything)
 constexpr int NR_MAX = 6;  // stages of the operand rows and target blocks with A in TMEM
 constexpr int KB = 16;    // chunks per accumulation block (512 samples)
 constexpr int NGEN = 8;   // generation warps: two per row quadrant, one per half of a chunk
 constexpr int NPART = NGEN / 4;  // parts of a chunk's samples
 constexpr int SPP = 32 / NPART;  // samples per part (a multiple of 8)
-constexpr int WARPS = 2 + NGEN + 4;
+// two sets of four epilogue warps (one TMEM lane quadrant each) that take
+// alternate tiles where a tile is one accumulation block: a tile's scoring is
+// a chain of table look-ups and takes longer than its contraction.  Longer
+// sample ranges keep running sums for one tile: one set.
+constexpr int SETS = 2;
+constexpr int WARPS = 2 + NGEN + 4 * SETS;
 constexpr int THREADS = WARPS * 32;
 constexpr uint32_t kWait = 1u << 22;
 // polls of the epilogue's waits, each followed by a short sleep (the
 // epilogue has a whole accumulation block of slack, so it polls gently)
 constexpr uint32_t kWaitLazy = 1u << 22;
 
-// Operand rows in shared memory: the 16 i-rows, then the 8 j-rows, 128 bytes
-// (32 samples) each, written by 2-D tensor copies (boxes of 8 rows) with the
+// Operand rows in shared memory: the i-rows, then the j-rows, 128 bytes (32
+// samples) each, written by 2-D tensor copies (boxes of 8 rows) with the
 // 128-byte swizzle: 16-byte group q of row r sits at group q ^ (r & 7), so
 // the rows a warp reads at one sample offset lie in different banks.
-constexpr uint32_t ROWS_BYTES = 2 * ROWS * 128;  // 6144: the rows, then their reciprocals (products)
+constexpr uint32_t ROWS_BYTES = 2 * ROWS * 128;  // 10240: the rows, then their reciprocals (products)
 constexpr int RCP_ROW = ROWS;                      // row index of the first reciprocal row
 constexpr uint32_t A_TILE = M * KC * 2;         // 8192 per slot per hi/lo
 constexpr uint32_t A_OFF = ROWS_BYTES;
@@ -111,9 +131,10 @@ __host__ __device__ constexpr uint32_t row_off(int r, int s) {
   return (uint32_t)(r * 128 + ((((s >> 2) ^ (r & 7))) << 4));
 }
 
-// Offsets of the eight samples s .. s+7 a generation thread reads from each
-// of its four rows (value rows ri, rj and their reciprocals); the same in
-// every stage, so computed once.
+// Offsets of the first eight of the samples a generation thread reads from
+// each of its four rows (value rows ri, rj and their reciprocals); the same
+// in every stage of a tile.  The next eight (s + 8, s a multiple of 16) are
+// at the offset with bit 5 flipped.
 struct GenAddr {
   uint32_t a[2], b[2], ia[2], ib[2];
 };
@@ -136,9 +157,8 @@ struct Shared {
   uint32_t tmem_base;
   int abort;
   float hand[2][NPART][M][6];  // [tile parity][sample part][row][S1, S2 per slot]
-  float theta[4][64];        // each epilogue warp's copy of the pass's list thresholds
-  float ysum[4][64];         // and of the targets' sums
-  float sy[4][16][32];       // each epilogue warp's spill of 16 numerators for its rare full scores
+  alignas(16) float theta[4 * SETS][64];  // each epilogue warp's copy of the pass's list thresholds
+  alignas(16) float ysum[64];             // the targets' sums
 };
 
 constexpr size_t shared_bytes() { return (sizeof(Shared) + 1023) / 1024 * 1024; }
@@ -234,17 +254,20 @@ __device__ __forceinline__ TcCand tc_prepare(const ScreenArgs &A, LaneStats &ls,
   return o;
 }
 
-// Targets t0 .. t0+15 of a prepared candidate; returns the lists pushed to.
-// The cheap bound is evaluated for all 16 without branches (independent
-// chains); the few survivors are scored in full from a per-lane copy of
-// their numerators in shared memory (sy: [16][32] of this warp).
+// Targets t0 .. t0+15 of the warp's prepared candidates (every lane calls it;
+// c.ok: the lane has one); returns the lists whose thresholds are due.  The cheap bound is
+// evaluated for all 16 without branches (independent chains); the few
+// survivors are scored in full (once to decide, once to write).  A list's slots are reserved once
+// for all lanes, all 16 lists' reservations in one instruction: taken entry
+// by entry, the round trips of the first tiles, whose thresholds are low,
+// took 1.5 ms of a launch of 18.8.
 __device__ __forceinline__ uint64_t tc_targets16(const ScreenArgs &A, const TcCand &c, const float (&Sy)[16], int t0,
                                                  float gamma_gen, float gamma_num, const float *ysum,
-                                                 const float *theta, float (*sy)[32]) {
+                                                 float *theta) {
   const float u = 5.9604644775390625e-8f;
   const float invN = (float)A.invN;
   const int lane = threadIdx.x & 31;
-  if (A.ivl) {
+  if (A.ivl && c.ok) {
     // every target's interval, for checking the error model
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
@@ -256,29 +279,76 @@ __device__ __forceinline__ uint64_t tc_targets16(const ScreenArgs &A, const TcCa
     }
   }
   unsigned mask = 0;
+  const float4 *ys4 = reinterpret_cast<const float4 *>(ysum + t0), *th4 = reinterpret_cast<const float4 *>(theta + t0);
 #pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    const int t = t0 + i;
-    const float ys = ysum[t];
-    const float aP = fabsf(fmaf(-c.S1, ys * invN, Sy[i]));
-    const float num = fmaf(aP, c.a2, fmaf(c.a1, fabsf(ys), c.a0)) * (1.0f + 8.0f * u);
-    const bool pass = t < A.T && !(c.qlo > 0.0f && num < theta[t] * c.qlo);
-    mask |= pass ? 1u << i : 0u;
+  for (int q = 0; q < 4; ++q) {
+    const float4 y4 = ys4[q], h4 = th4[q];
+    const float yq[4] = {y4.x, y4.y, y4.z, y4.w}, hq[4] = {h4.x, h4.y, h4.z, h4.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int i = 4 * q + j;
+      const float aP = fabsf(fmaf(-c.S1, yq[j] * invN, Sy[i]));
+      const float num = fmaf(aP, c.a2, fmaf(c.a1, fabsf(yq[j]), c.a0)) * (1.0f + 8.0f * u);
+      const bool pass = t0 + i < A.T && !(c.qlo > 0.0f && num < hq[j] * c.qlo);
+      mask |= pass ? 1u << i : 0u;
+    }
   }
-  if (!mask) return 0;
+  if (!c.ok) mask = 0;
+  unsigned todo = __reduce_or_sync(0xffffffffu, mask);
+  if (!todo) return 0;
+  // the thresholds as they are now
+  if (lane < 16 && t0 + lane < A.T) theta[t0 + lane] = ld_relaxed(&A.B.theta[A.t0 + t0 + lane]);
+  __syncwarp();
+  auto full = [&](int i, float *s, float *e) {
+    float v = Sy[0];
 #pragma unroll
-  for (int i = 0; i < 16; ++i) sy[i][lane] = Sy[i];
-  uint64_t pushed = 0;
+    for (int j = 1; j < 16; ++j) v = i == j ? Sy[j] : v;
+    cand_score_num<float>(c.ci, c.S1, v, invN, ysum[t0 + i], gamma_gen, gamma_num, u, s, e);
+    *e = *e * (1.0f + 2.4e-7f);
+  };
+  unsigned keep = 0;  // lists this lane's candidate is pushed to
   while (mask) {
     const int i = __ffs(mask) - 1;
     mask &= mask - 1;
-    const int t = t0 + i;
-    const float v = sy[i][lane];
     float s, e;
-    cand_score_num<float>(c.ci, c.S1, v, invN, ysum[t], gamma_gen, gamma_num, u, &s, &e);
-    if (iv_hi(s, e) < theta[t]) continue;
-    if (push_one(A.B, A.t0 + t, c.gid, s, e * (1.0f + 2.4e-7f))) pushed |= 1ull << t;
+    full(i, &s, &e);
+    if (iv_hi(s, e) >= theta[t0 + i]) keep |= 1u << i;
   }
+  __syncwarp();
+  unsigned mine = 0;  // lane i: list i's pushes in this warp
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    const unsigned b = __ballot_sync(0xffffffffu, keep >> i & 1u);
+    if (lane == i) mine = b;
+  }
+  const unsigned every = A.k >= 1024 ? 64u : A.k >= 16 ? (unsigned)(A.k >> 4) : 1u;
+  unsigned base = 0;
+  if (mine) base = atomicAdd(&A.B.count[A.t0 + t0 + lane], (unsigned)__popc(mine));
+  uint64_t pushed = 0;
+  todo = __ballot_sync(0xffffffffu, mine != 0);
+  while (todo) {
+    const int i = __ffs(todo) - 1;
+    todo &= todo - 1;
+    const unsigned b = __shfl_sync(0xffffffffu, mine, i), at = __shfl_sync(0xffffffffu, base, i);
+    const bool act = b >> lane & 1u;
+    const int l = A.t0 + t0 + i;
+    float s = 0.f, e = 0.f;
+    if (act) {
+      full(i, &s, &e);
+      const unsigned pos = at + __popc(b & ((1u << lane) - 1u));
+      if ((int64_t)pos < A.B.cap) {
+        const size_t x = (size_t)l * (size_t)A.B.cap + pos;
+        A.B.id[x] = c.gid;
+        A.B.score[x] = s;
+        A.B.eps[x] = e;
+      }
+    }
+    count_bounds_warp(A.B, l, act, s, e);
+    // a list's threshold is looked at again each time `every` more entries
+    // are in it: a look costs more than the entry
+    if (at / every != (at + (unsigned)__popc(b)) / every) pushed |= 1ull << (t0 + i);
+  }
+  __syncwarp();
   return pushed;
 }
 
@@ -299,50 +369,62 @@ struct TcGen {
 template <int KIND, bool CHECK, bool TA>
 __device__ __forceinline__ void tc_gen8(TcGen &g, const unsigned char *S, const tc::GenAddr &ad, int k, int kbase, int lim,
                                         unsigned char *Aop, uint32_t acol, int m) {
+  const uint32_t flip = (uint32_t)k << 2;  // k: 0 or 8
   using namespace tc;
-  float av[8], bv[8], iav[8], ibv[8];
+  // (packed pairs of samples; the sums take the samples one by one, in order)
+  F2 av[4], bv[4], iav[4], ibv[4];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    *reinterpret_cast<float4 *>(av + 4 * h) = *reinterpret_cast<const float4 *>(S + ad.a[h]);
-    *reinterpret_cast<float4 *>(bv + 4 * h) = *reinterpret_cast<const float4 *>(S + ad.b[h]);
+    *reinterpret_cast<ulonglong2 *>(av + 2 * h) = *reinterpret_cast<const ulonglong2 *>(S + (ad.a[h] ^ flip));
+    *reinterpret_cast<ulonglong2 *>(bv + 2 * h) = *reinterpret_cast<const ulonglong2 *>(S + (ad.b[h] ^ flip));
     if (KIND == KIND_MUL) {
-      *reinterpret_cast<float4 *>(iav + 4 * h) = *reinterpret_cast<const float4 *>(S + ad.ia[h]);
-      *reinterpret_cast<float4 *>(ibv + 4 * h) = *reinterpret_cast<const float4 *>(S + ad.ib[h]);
+      *reinterpret_cast<ulonglong2 *>(iav + 2 * h) = *reinterpret_cast<const ulonglong2 *>(S + (ad.ia[h] ^ flip));
+      *reinterpret_cast<ulonglong2 *>(ibv + 2 * h) = *reinterpret_cast<const ulonglong2 *>(S + (ad.ib[h] ^ flip));
     }
   }
-  float wv[3][8];
+  const F2 minus = f2_pack(-1.f, -1.f), n0 = f2_pack(-g.c0, -g.c0), n1 = f2_pack(-g.c1, -g.c1),
+           n2 = f2_pack(-g.c2, -g.c2);
+  F2 wv[3][4];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) {
-    if (!CHECK || k + e < lim) {
-      const float a = av[e], b = bv[e];
-      if (KIND == KIND_MUL) {
-        wv[0][e] = fmaf(a, b, -g.c0);
-        wv[1][e] = fmaf(a, ibv[e], -g.c1);
-        wv[2][e] = fmaf(b, iav[e], -g.c2);
-      } else {
-        const float ac = a - g.c0, bc = b - g.c1, d = a - b;
-        wv[0][e] = ac + bc;
-        wv[1][e] = ac - bc;
-        wv[2][e] = fabsf(d) - g.c2;
-      }
-#pragma unroll
-      for (int sl = 0; sl < 3; ++sl) {
-        g.t1[sl] += wv[sl][e];
-        g.t2[sl] = fmaf(wv[sl][e], wv[sl][e], g.t2[sl]);
-      }
+  for (int e = 0; e < 4; ++e) {
+    const F2 a = av[e], b = bv[e];
+    if (KIND == KIND_MUL) {
+      wv[0][e] = f2_fma(a, b, n0);
+      wv[1][e] = f2_fma(a, ibv[e], n1);
+      wv[2][e] = f2_fma(b, iav[e], n2);
     } else {
-      wv[0][e] = wv[1][e] = wv[2][e] = 0.f;
+      // (a product by -1 is exact: one rounding, as in a subtraction)
+      const F2 ac = f2_add(a, n0), bc = f2_add(b, n1);
+      wv[0][e] = f2_add(ac, bc);
+      wv[1][e] = f2_fma(bc, minus, ac);
+      wv[2][e] = f2_add(f2_fma(b, minus, a) & 0x7fffffff7fffffffull, n2);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (!CHECK || k + 2 * e + h < lim) {
+#pragma unroll
+        for (int sl = 0; sl < 3; ++sl) {
+          const float w = f2_half(wv[sl][e], h);
+          g.t1[sl] += w;
+          g.t2[sl] = fmaf(w, w, g.t2[sl]);
+        }
+      } else {
+#pragma unroll
+        for (int sl = 0; sl < 3; ++sl)
+          wv[sl][e] = h ? f2_pack(f2_half(wv[sl][e], 0), 0.f) : f2_pack(0.f, f2_half(wv[sl][e], 1));
+      }
     }
   }
 #pragma unroll
   for (int sl = 0; sl < 3; ++sl) {
     uint32_t hi[4], lo[4];
 #pragma unroll
-    for (int e = 0; e < 8; e += 2) {
-      const __nv_bfloat162 h = __floats2bfloat162_rn(wv[sl][e], wv[sl][e + 1]);
-      const __nv_bfloat162 l = __floats2bfloat162_rn(wv[sl][e] - __low2float(h), wv[sl][e + 1] - __high2float(h));
-      hi[e >> 1] = *reinterpret_cast<const uint32_t *>(&h);
-      lo[e >> 1] = *reinterpret_cast<const uint32_t *>(&l);
+    for (int e = 0; e < 4; ++e) {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(f2_half(wv[sl][e], 0), f2_half(wv[sl][e], 1));
+      hi[e] = *reinterpret_cast<const uint32_t *>(&h);
+      const F2 r = f2_fma(f2_pack(__uint_as_float(hi[e] << 16), __uint_as_float(hi[e] & 0xffff0000u)), minus, wv[sl][e]);
+      const __nv_bfloat162 l = __floats2bfloat162_rn(f2_half(r, 0), f2_half(r, 1));
+      lo[e] = *reinterpret_cast<const uint32_t *>(&l);
     }
     if (TA) {
       // this lane's row: four columns (eight samples) per component
@@ -412,6 +494,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
     sh.abort = 0;
     mbar_fence_init();
   }
+  if (threadIdx.x < 64) sh.ysum[threadIdx.x] = (int)threadIdx.x < A.T ? A.ysum32[A.t0 + threadIdx.x] : 0.f;
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem_base)),
                  "r"((uint32_t)TMEM_COLS)
@@ -458,15 +541,15 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    // lane 0: three 2-D tensor copies of the chunk's operand rows (i-rows
-    // 0-7, 8-15, j-rows 0-7 at the tile's row positions; rows past the end
-    // and samples past N arrive as zeros), three more of their reciprocal
-    // rows for the products and quotients, and one bulk copy of the target
-    // block
+    // lane 0: 2-D tensor copies of the chunk's operand rows in boxes of eight
+    // (i-rows, then j-rows; rows past the end and samples past N arrive as
+    // zeros), as many of their reciprocal rows for the products and
+    // quotients, and one bulk copy of the target block
     int lt = 0;
     uint32_t issued = 0;  // chunks whose copies were issued
     for (int tile = blockIdx.x; tile < A.n_tiles && !aborted_warp(); tile += gridDim.x, ++lt) {
       const Tile tl = A.tiles[tile];
+      const Shape shp = shape_of(tl);
       bool ok = true;
       for (int c = 0; c < nchunks; ++c) {
         const uint32_t gc = (uint32_t)lt * nchunks + c, st = gc % NR, u = gc / NR;
@@ -476,15 +559,13 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
         }
         unsigned char *S = stages + (size_t)st * SB;
         if (lane == 0) {
-          mbar_arrive_expect_tx(&sh.full_rows[st], (KIND == KIND_MUL ? 6u : 3u) * 1024u + b_bytes(NTP));
+          mbar_arrive_expect_tx(&sh.full_rows[st],
+                                (KIND == KIND_MUL ? 2u : 1u) * 1024u * (uint32_t)shp.boxes + b_bytes(NTP));
           const int x = c * KC;
-          tma_load_2d(S, &rows_map, x, tl.ibase, &sh.full_rows[st]);
-          tma_load_2d(S + 1024, &rows_map, x, tl.ibase + 8, &sh.full_rows[st]);
-          tma_load_2d(S + 2048, &rows_map, x, tl.jbase, &sh.full_rows[st]);
-          if (KIND == KIND_MUL) {
-            tma_load_2d(S + 3072, &rcp_map, x, tl.ibase, &sh.full_rows[st]);
-            tma_load_2d(S + 4096, &rcp_map, x, tl.ibase + 8, &sh.full_rows[st]);
-            tma_load_2d(S + 5120, &rcp_map, x, tl.jbase, &sh.full_rows[st]);
+          for (int q = 0; q < shp.boxes; ++q) {
+            const int row = q < shp.i_boxes ? tl.ibase + BOX * q : tl.jbase + BOX * (q - shp.i_boxes);
+            tma_load_2d(S + 1024 * q, &rows_map, x, row, &sh.full_rows[st]);
+            if (KIND == KIND_MUL) tma_load_2d(S + 128 * RCP_ROW + 1024 * q, &rcp_map, x, row, &sh.full_rows[st]);
           }
           bulk_g2s(S + B_OFF, bsplit + (size_t)c * b_bytes(NTP), b_bytes(NTP), &sh.full_rows[st]);
         }
@@ -559,13 +640,13 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
     // lanes its tcgen05 stores may address
     const int m = (warp & 3) * 32 + lane;
     const int part = gw >> 2;            // which SPP samples of a chunk
-    static_assert(SPP == 8 || SPP == 16, "one or two eight-sample steps per chunk and thread");
-    const GenAddr gad = gen_addr(m >> 3, BI + (m & 7), part * SPP);
-    const GenAddr gad2 = gen_addr(m >> 3, BI + (m & 7), part * SPP + (SPP - 8));
-    const int ti = m >> 3, tj = m & 7;
+    static_assert(SPP == 16, "two eight-sample steps per chunk and thread");
     int lt = 0;
     for (int tile = blockIdx.x; tile < A.n_tiles && !aborted_warp(); tile += gridDim.x, ++lt) {
       const Tile tl = A.tiles[tile];
+      const Shape shp = shape_of(tl);
+      const int ti = m >> shp.log_nj, tj = m & ((1 << shp.log_nj) - 1);
+      const GenAddr gad = gen_addr(ti, BOX * shp.i_boxes + tj, part * SPP);
       const int fi = ti < tl.ni ? A.rowid[tl.ibase + ti] : -1;
       const int fj = tj < tl.nj ? A.rowid[tl.jbase + tj] : -1;
       const float4 fa_i = fi >= 0 ? A.F.fa[fi] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -599,13 +680,15 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
         unsigned char *S = stages + (size_t)st * SB;
         unsigned char *Aop = S + A_OFF;
         const uint32_t acol = tmem + ((uint32_t)((warp & 3) * 32) << 16) + ACOL + sa * A_STAGE_COLS;
+        // (loops: one copy of the code, which the epilogue's code displaces
+        // from the instruction cache otherwise)
         if ((c + 1) * KC <= A.N) {
-          tc_gen8<KIND, false, TA>(g, S, gad, 0, part * SPP, 0, Aop, acol, m);
-          if (SPP == 16) tc_gen8<KIND, false, TA>(g, S, gad2, 8, part * SPP, 0, Aop, acol, m);
+#pragma unroll 1
+          for (int k = 0; k < SPP; k += 8) tc_gen8<KIND, false, TA>(g, S, gad, k, part * SPP, 0, Aop, acol, m);
         } else {
           const int lim = A.N - c * KC - part * SPP;
-          tc_gen8<KIND, true, TA>(g, S, gad, 0, part * SPP, lim, Aop, acol, m);
-          if (SPP == 16) tc_gen8<KIND, true, TA>(g, S, gad2, 8, part * SPP, lim, Aop, acol, m);
+#pragma unroll 1
+          for (int k = 0; k < SPP; k += 8) tc_gen8<KIND, true, TA>(g, S, gad, k, part * SPP, lim, Aop, acol, m);
         }
         if (++blk == gen_blk) {
           blk = 0;
@@ -639,15 +722,18 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
     }
   } else {
     // ------------------------------------------------------------ epilogue
-    const int q = warp & 3;
+    const int q = warp & 3, ew = warp - 2 - NGEN;
+    const int sets = nblocks == 1 ? SETS : 1, set = ew >> 2;
     const int m = q * 32 + lane;
-    const int ti = m >> 3, tj = m & 7;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     LaneStats ls;
     ls.zero();
-    int lt = 0;
-    for (int tile = blockIdx.x; tile < A.n_tiles && !aborted_warp(); tile += gridDim.x, ++lt) {
+    int lt = set;
+    for (int64_t tile = (int64_t)blockIdx.x + (int64_t)set * gridDim.x;
+         set < sets && tile < A.n_tiles && !aborted_warp(); tile += (int64_t)gridDim.x * sets, lt += sets) {
       const Tile tl = A.tiles[tile];
+      const Shape shp = shape_of(tl);
+      const int ti = m >> shp.log_nj, tj = m & ((1 << shp.log_nj) - 1);
       const int64_t x = ti < tl.ni ? A.rowid[tl.ibase + ti] : -1;
       const int64_t y = tj < tl.nj ? A.rowid[tl.jbase + tj] : -1;
       bool pv = x >= 0 && y >= 0 && (tl.ibase + ti) > (tl.jbase + tj);
@@ -659,15 +745,6 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
       const float4 fa_y = y >= 0 ? A.F.fa[y] : make_float4(0.f, 0.f, 0.f, 0.f);
       const float4 fa_a = x > y ? fa_x : fa_y, fa_b = x > y ? fa_y : fa_x;
       const float mi = fa_x.x, mj = fa_y.x;  // evaluation order: row i, row j
-      float kks[3];
-      if (KIND == KIND_MUL) {
-        kks[0] = mi * mj;
-        kks[1] = mi * fa_y.y;
-        kks[2] = mj * fa_x.y;
-      } else {
-        kks[0] = kks[1] = 0.f;
-        kks[2] = fabsf(mi - mj);
-      }
       // numerators: one block stays in TMEM until the end; longer sample
       // ranges drain each block into a running FP32 sum kept in TMEM
       // columns [6 NTP, 9 NTP) (added in registers, block by block)
@@ -712,29 +789,29 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
       if (!wait_warp_lazy(&sh.gen_done[p], (lt >> 1) & 1)) break;
       // this warp's copy of the list thresholds (they only rise, so an older
       // copy is still a valid lower bound)
-      for (int t = lane; t < NTP; t += 32) {
-        sh.theta[q][t] = t < A.T ? ld_relaxed(&A.B.theta[A.t0 + t]) : 0.f;
-        sh.ysum[q][t] = t < A.T ? A.ysum32[A.t0 + t] : 0.f;
-      }
+      for (int t = lane; t < NTP; t += 32) sh.theta[ew][t] = t < A.T ? ld_relaxed(&A.B.theta[A.t0 + t]) : 0.f;
       __syncwarp();
-      float st12[6];
+      // the row's S1 and S2: the parts added in order, in place (this lane's
+      // own entries)
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
         float v = sh.hand[p][0][m][i];
 #pragma unroll
         for (int h = 1; h < NPART; ++h) v += sh.hand[p][h][m][i];
-        st12[i] = v;
+        sh.hand[p][0][m][i] = v;
       }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sh.epi_free[p]);
       uint64_t pushed = 0;
-#pragma unroll
+      // (loops over the slots and the targets: one copy of the scoring code;
+      // unrolled, with the generation beside it, warps waited for
+      // instructions 3.9 cycles an issued one)
+#pragma unroll 1
       for (int k = 0; k < 3; ++k) {
-        const int opc = KIND == KIND_MUL ? (k == 0 ? DSE_OP_MUL : k == 1 ? DSE_OP_DIV : DSE_OP_RDIV)
-                                         : (k == 0 ? DSE_OP_ADD : k == 1 ? DSE_OP_SUB : DSE_OP_ABSDIFF);
-        const TcCand tcc = tc_prepare(A, ls, pv, ia, ib, opc, pbase, fa_a, fa_b, kks[k], mi, mj, st12[2 * k],
-                                      st12[2 * k + 1], gamma_gen, gamma_num);
-#pragma unroll(NTP <= 32 ? 2 : 1)
+        const int opc = KIND == KIND_MUL ? DSE_OP_MUL + k : k == 2 ? DSE_OP_ABSDIFF : DSE_OP_ADD + k;
+        const float kk = KIND == KIND_MUL ? (k == 0 ? mi * mj : k == 1 ? mi * fa_y.y : mj * fa_x.y)
+                                          : (k == 2 ? fabsf(mi - mj) : 0.f);
+        const TcCand tcc = tc_prepare(A, ls, pv, ia, ib, opc, pbase, fa_a, fa_b, kk, mi, mj, sh.hand[p][0][m][2 * k],
+                                      sh.hand[p][0][m][2 * k + 1], gamma_gen, gamma_num);
+#pragma unroll 1
         for (int c16 = 0; c16 < NTP; c16 += 16) {
           float v[16];
           if (nblocks == 1) {
@@ -751,7 +828,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
           } else {
             tmem_ld16(tmem + lane_base + (6 + k) * NTP + c16, v);
           }
-          if (tcc.ok) pushed |= tc_targets16(A, tcc, v, c16, gamma_gen, gamma_num, sh.ysum[q], sh.theta[q], sh.sy[q]);
+          pushed |= tc_targets16(A, tcc, v, c16, gamma_gen, gamma_num, sh.ysum, sh.theta[ew]);
         }
       }
       if (nblocks == 1) {
@@ -759,13 +836,10 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.acc_empty[buf_last]);
       }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.epi_free[p]);
       // raise the thresholds of the lists this warp pushed to
-      unsigned lo = (unsigned)pushed, hi = (unsigned)(pushed >> 32);
-      lo = __reduce_or_sync(0xffffffffu, lo);
-      hi = __reduce_or_sync(0xffffffffu, hi);
-      const uint64_t all = (uint64_t)lo | ((uint64_t)hi << 32);
-      for (int t = 0; t < NTP && t < 64; ++t)
-        if (all & (1ull << t)) refresh_theta(A.B, A.t0 + t, A.k);
+      for (uint64_t all = pushed; all; all &= all - 1) refresh_theta(A.B, A.t0 + __ffsll((long long)all) - 1, A.k);
     }
     flush_stats(A, ls);
   }

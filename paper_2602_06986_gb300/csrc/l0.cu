@@ -8,14 +8,17 @@
 // the search is a scan of small Cholesky factorisations over the Gram
 // matrix:
 //   1. columns, centring, b and raw norms (one block per candidate);
-//   2. the Gram matrix G (tiled, FP64; the dense contraction of the step);
+//   2. the Gram matrix G on the tensor cores, error-free up to the slicing
+//      (the dense contraction of the step, see k_l0_gram);
 //   3. the scan: D = 1 thread per candidate, D = 2 thread per pair, D = 3
-//      warp per pair (p_0, p_1) with lanes over p_2 -- an incremental
-//      Cholesky step per subset -- keeping each warp's 32 best (q, subset)
-//      in registers across its lanes, then each block's 32 best;
-//   4. the 32 best of all blocks (one block), then an explicit FP64 refit
-//      of each (coefficients and the RMSE of the explicit residual) whose
-//      order (RMSE, positions) decides.
+//      warp per pair (p_0, p_1) with lanes over p_2 -- an FP32 upper bound of
+//      q, then an incremental Cholesky step in FP64 for the subsets it does
+//      not exclude -- keeping each warp's 32 best (q, subset) in registers
+//      across its lanes, then each block's 32 best;
+//   4. the 64 best of all blocks (one block); their Gram entries and q again
+//      in plain FP64, sample by sample, the 32 best of those, then an
+//      explicit FP64 refit of each (coefficients and the RMSE of the explicit
+//      residual) whose order (RMSE, positions) decides.
 // The rank rule is that of the refits: a pivot of the centred Cholesky at
 // or below 1e-12 of the raw column's norm rejects the subset, with the
 // pivots taken in position order (as a QR of [1, X_p0, X_p1, ...] would).
@@ -28,6 +31,7 @@
 #include "dse_internal.cuh"
 #include "eval64.cuh"
 #include "plan.cuh"
+#include "tcgen05.cuh"
 #include "util.cuh"
 
 namespace dse {
@@ -37,6 +41,7 @@ FeatTable table_of(const dse_space *S);
 namespace {
 
 constexpr int kTop = 32;        // subsets kept per warp / block / search
+constexpr int kMore = 64;       // subsets whose q is taken again in plain FP64
 constexpr int kCol = 128;       // threads per column block
 constexpr double kRank2 = 1e-24;  // (1e-12)^2: squared pivot / squared raw norm
 
@@ -127,51 +132,301 @@ __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, in
   }
 }
 
-// Gram matrix of the centred columns: one 32 x 32 tile (bi <= bj) per block
-// of 256 threads, 2 x 2 outputs per thread, samples staged in 32-sample
-// slices through shared memory; both G[i][j] and G[j][i] are written.
-constexpr int kGT = 32, kGS = 32;
-__global__ void __launch_bounds__(256) k_l0_gram(const double *X, int64_t n, int64_t N, int64_t nt, double *Gm) {
-  __shared__ double xi[kGT][kGS + 1], xj[kGT][kGS + 1];
-  // tile index -> (bi, bj), bi <= bj, over the upper triangle of nt x nt tiles
-  // tile t of the triangle with the diagonal: t = bj (bj + 1) / 2 + bi, bi <= bj
-  const int64_t t = blockIdx.x;
-  uint64_t bj = (uint64_t)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-  while ((bj + 1) * (bj + 2) / 2 <= (uint64_t)t) ++bj;
-  while (bj * (bj + 1) / 2 > (uint64_t)t) --bj;
-  const uint64_t bi = (uint64_t)t - bj * (bj + 1) / 2;
-  const int64_t i0 = (int64_t)bi * kGT, j0 = (int64_t)bj * kGT;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads, 2 x 2 outputs each
-  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-  for (int64_t s0 = 0; s0 < N; s0 += kGS) {
-    for (int e = threadIdx.x; e < kGT * kGS; e += 256) {
-      const int r2 = e / kGS, k = e % kGS;
-      const int64_t s = s0 + k;
-      xi[r2][k] = (i0 + r2 < n && s < N) ? X[(i0 + r2) * N + s] : 0.0;
-      xj[r2][k] = (j0 + r2 < n && s < N) ? X[(j0 + r2) * N + s] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kGS; ++k) {
-      const double a0 = xi[ty * 2][k], a1 = xi[ty * 2 + 1][k];
-      const double b0 = xj[tx * 2][k], b1 = xj[tx * 2 + 1][k];
-      acc[0][0] = fma(a0, b0, acc[0][0]);
-      acc[0][1] = fma(a0, b1, acc[0][1]);
-      acc[1][0] = fma(a1, b0, acc[1][0]);
-      acc[1][1] = fma(a1, b1, acc[1][1]);
-    }
-    __syncthreads();
+// ---------------------------------------------------- Gram matrix, sliced
+//
+// G = X X^T of the centred columns to FP64 accuracy on the tensor cores.  In
+// FP64 instructions the contraction is bound by the FP64 pipe (2 a clock and
+// SM: n = 3000, N = 1000 took 7.69 ms).  Here each column is scaled by a power
+// of two and cut into eight signed 7-bit digits, x = 2^e sum_k d_k 2^-7k + r
+// with |d_k| <= 64 and |r| <= 2^(e-57) (at most 2^-55 of the column's largest
+// value; the FP64 sum of products loses more).  The digits are BF16 numbers,
+// their products integers up to 2^12, and the 36 digit products with
+// i + j <= 7 are added by class s = i + j, at most 8 of them a class, over
+// blocks of 512 samples: every partial sum is an integer up to 2^24, so the
+// FP32 accumulation in tensor memory is exact in any order.  The blocks' sums
+// meet in 64-bit integers; one rounding per entry follows at the end.  (The
+// dropped products, i + j > 7, are below 2^-56 of the product of the columns'
+// largest values a sample.)  36 BF16 contractions cost 1/30 of the FP64 one:
+// 7.69 -> 0.29 ms.
+namespace sliced {
+constexpr int DIG = 8, BITS = 7;
+constexpr int RB = 64;                       // columns of X in an image block
+constexpr int KC = 16;                       // samples of a stage: one MMA deep
+constexpr int TILE = RB * KC * 2;            // bytes of a digit's tile: 2048
+constexpr int CHUNK = DIG * TILE;            // bytes of a block's chunk: 16 KB
+constexpr int KB = 32;                       // chunks of an exact block: 512 samples
+constexpr int STAGE = 3 * CHUNK, NS = 4;     // A: two blocks (128 columns), B: one
+constexpr int EPI = 8, WARPS = 2 + EPI, THREADS = 32 * WARPS;
+constexpr uint32_t LBO = 128, SBO = 256;     // K-major 8 x 8 core matrices, no swizzle
+constexpr uint32_t kWait = 1u << 22;
+struct Shared {
+  uint64_t full[NS], empty[NS], acc_full, acc_empty, drain;
+  uint32_t tmem;
+  int abort;
+};
+constexpr size_t SMEM = 1024 + (size_t)NS * STAGE;
+__device__ __forceinline__ uint64_t desc(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(LBO >> 4) << 16) | ((uint64_t)(SBO >> 4) << 32) |
+         (1ull << 46);
+}
+}  // namespace sliced
+
+// Exponent e of each column: |x| <= 2^(e-1) for every sample (one block per
+// column; 0 and nothing to slice for a zero or non-finite column).
+__global__ void __launch_bounds__(kCol) k_l0_exponents(const double *X, int64_t N, int *ex) {
+  __shared__ unsigned long long sm[kCol / 32];
+  const double *x = X + (int64_t)blockIdx.x * N;
+  unsigned long long m = 0;  // (the bits of |x| order like the values)
+  for (int64_t i = threadIdx.x; i < N; i += kCol) {
+    const unsigned long long v = (unsigned long long)__double_as_longlong(x[i]) & 0x7fffffffffffffffull;
+    m = v > m ? v : m;
   }
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+    m = v > m ? v : m;
+  }
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kCol / 32; ++w) m = sm[w] > m ? sm[w] : m;
+    const int be = (int)(m >> 52);  // biased exponent of the largest value
+    ex[blockIdx.x] = m == 0 || be == 2047 ? INT32_MIN : (be ? be : 1) - 1023 + 2;
+  }
+}
+
+// Digit images of samples [s0, s0 + ns): block rb, chunk c, digit k at
+// ((rb nc + c) DIG + k) TILE, rows (columns of X) x 16 samples in core
+// matrices.  A block of 128 threads takes one image block and chunk: thread t
+// one row and half of its samples.
+__global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *ex, int64_t n, int64_t N, int64_t s0,
+                                                   int64_t ns, int nc, unsigned char *img) {
+  using namespace sliced;
+  const int c = blockIdx.x, rb = blockIdx.y, row = threadIdx.x & 63, h = threadIdx.x >> 6;
+  const int64_t col = (int64_t)rb * RB + row, k0 = (int64_t)c * KC + 8 * h;
+  const int e = col < n ? ex[col] : INT32_MIN;
+  uint32_t d[DIG][4];
 #pragma unroll
-  for (int a = 0; a < 2; ++a)
+  for (int k = 0; k < DIG; ++k) d[k][0] = d[k][1] = d[k][2] = d[k][3] = 0u;
+  if (e != INT32_MIN) {
+    const double *x = X + col * N + s0 + k0;
 #pragma unroll
-    for (int c2 = 0; c2 < 2; ++c2) {
-      const int64_t i = i0 + ty * 2 + a, j = j0 + tx * 2 + c2;
-      if (i < n && j < n) {
-        Gm[i * n + j] = acc[a][c2];
-        Gm[j * n + i] = acc[a][c2];
+    for (int i = 0; i < 8; ++i) {
+      // the digits of x 2^(56 - e), an integer up to 2^55, lowest first
+      long long q = k0 + i < ns ? __double2ll_rn(scalbn(x[i], DIG * BITS - e)) : 0ll;
+#pragma unroll
+      for (int k = DIG - 1; k >= 0; --k) {
+        const int v = k ? (int)((q + 64) & 127) - 64 : (int)q;
+        q = (q - v) >> BITS;
+        const uint32_t bits = __float_as_uint((float)v) >> 16;  // exact: |v| <= 64
+        d[k][i >> 1] |= bits << (16 * (i & 1));
       }
     }
+  }
+  unsigned char *o = img + ((size_t)rb * nc + c) * CHUNK + (row >> 3) * SBO + h * LBO + (row & 7) * 16;
+#pragma unroll
+  for (int k = 0; k < DIG; ++k)
+    *reinterpret_cast<uint4 *>(o + k * TILE) = make_uint4(d[k][0], d[k][1], d[k][2], d[k][3]);
+}
+
+// One tile of 128 x 64 entries (i-block bi of 128 columns, j-block bj of 64, bj >= 2
+// bi) per CTA.  Warp 0: producer; warp 1: tensor memory and the MMAs (36 a
+// chunk, accumulators s = 0..7 of 64 columns each: all of tensor memory);
+// warps 2-9: the block sums into 64-bit integers, 32 entries a lane, then the
+// entries i <= j of the tile, both G[i][j] and G[j][i], and the scale-free
+// FP32 values the scan's bound reads.  `add`: onto an earlier panel's.
+__global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned char *img, const int *ex, int64_t n,
+                                                                int nc, int add, int upper, double *Gm, float *G32,
+                                                                int *err) {
+  using namespace sliced;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  Shared &sh = *reinterpret_cast<Shared *>(smem);
+  unsigned char *stages = smem + 1024;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // tile t: i-block bi has the j-blocks 2 bi .. nb - 1, before it come bi (nb + 1 - bi)
+  const int nb = 2 * (int)((n + 127) / 128);
+  const int64_t t = blockIdx.x;
+  int bi = 0;
+  {
+    const double h = 0.5 * (nb + 1);
+    bi = (int)(h - sqrt(fmax(h * h - (double)t, 0.0)));
+    while (bi > 0 && (int64_t)bi * (nb + 1 - bi) > t) --bi;
+    while ((int64_t)(bi + 1) * (nb - bi) <= t) ++bi;
+  }
+  const int bj = 2 * bi + (int)(t - (int64_t)bi * (nb + 1 - bi));
+  const int nkb = (nc + KB - 1) / KB;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < NS; ++i) {
+      mbar_init(&sh.full[i], 1);
+      mbar_init(&sh.empty[i], 1);
+    }
+    mbar_init(&sh.acc_full, 1);
+    mbar_init(&sh.acc_empty, EPI);
+    mbar_init(&sh.drain, 1);
+    sh.abort = 0;
+    mbar_fence_init();
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)),
+                 "r"(512u)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = sh.tmem;
+  volatile int *abort_flag = &sh.abort;
+  auto wait = [&](uint64_t *bar, uint32_t parity) -> bool {
+    if (mbar_wait_bounded(bar, parity, kWait)) return true;
+    atomicExch(err, DSE_ETIMEOUT);
+    *abort_flag = 1;
+    return false;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int c = 0;
+      const unsigned char *a0 = img + (size_t)(2 * bi) * nc * CHUNK, *a1 = a0 + (size_t)nc * CHUNK,
+                          *b0 = img + (size_t)bj * nc * CHUNK;
+      for (; c < nc && !*abort_flag; ++c) {
+        const int st = c % NS, u = c / NS;
+        if (u >= 1 && !wait(&sh.empty[st], (u - 1) & 1)) break;
+        unsigned char *S = stages + (size_t)st * STAGE;
+        mbar_arrive_expect_tx(&sh.full[st], STAGE);
+        for (int k = 0; k < DIG; ++k) {  // a digit's 128 rows side by side
+          bulk_g2s(S + (2 * k) * TILE, a0 + (size_t)c * CHUNK + k * TILE, TILE, &sh.full[st]);
+          bulk_g2s(S + (2 * k + 1) * TILE, a1 + (size_t)c * CHUNK + k * TILE, TILE, &sh.full[st]);
+        }
+        bulk_g2s(S + 2 * CHUNK, b0 + (size_t)c * CHUNK, CHUNK, &sh.full[st]);
+      }
+      // no copy may still be landing when the CTA exits
+      for (int st = 0; st < NS && st < c; ++st) {
+        const int last = (c - 1 - st) / NS * NS + st;
+        mbar_wait_bounded(&sh.full[st], (last / NS) & 1, kWait);
+      }
+    }
+  } else if (warp == 1) {
+    if (lane == 0) {
+      for (int kb = 0; kb < nkb && !*abort_flag; ++kb) {
+        if (kb >= 1 && !wait(&sh.acc_empty, (kb - 1) & 1)) break;
+        tc::fence_after();
+        const int c1 = min(nc, (kb + 1) * KB);
+        for (int c = kb * KB; c < c1; ++c) {
+          const int st = c % NS;
+          if (!wait(&sh.full[st], (c / NS) & 1)) break;
+          tc::fence_after();
+          const uint32_t A = smem_u32(stages + (size_t)st * STAGE), B = A + 2 * CHUNK;
+          // digit i of A against the digits j <= 7 - i of B: their tiles lie
+          // side by side, as do the accumulators of the classes i + j, so
+          // four of them are one MMA of 256 columns
+          for (int i = 0; i < DIG; ++i) {
+            const uint64_t da = desc(A + 2 * i * TILE);
+            const uint32_t acc = c > kb * KB || i > 0 ? 1u : 0u;
+            for (int j = 0; i + j < DIG; j += 4) {
+              const int w = min(4, DIG - i - j);
+              tc::mma_bf16(tmem + (i + j) * RB, da, desc(B + j * TILE), tc::idesc_bf16(128, w * RB), acc);
+            }
+          }
+          tc::mma_commit(&sh.empty[st]);
+          if (c == c1 - 1) tc::mma_commit(&sh.acc_full);
+        }
+      }
+      tc::mma_commit(&sh.drain);
+      mbar_wait_bounded(&sh.drain, 0, kWait);
+    }
+  } else {
+    const int q = warp & 3, half = (warp - 2) >> 2;
+    const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + half * 32;
+    long long hi[32], lo[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) hi[i] = lo[i] = 0;
+    bool ok = true;
+    for (int kb = 0; kb < nkb && ok; ++kb) {
+      bool done = false;
+      for (uint32_t it = 0; it < kWait && !done; ++it) {
+        done = mbar_try_wait(&sh.acc_full, kb & 1);
+        if (!done) __nanosleep(100);
+      }
+      ok = __all_sync(0xffffffffu, done);
+      if (!ok) {
+        if (lane == 0) {
+          atomicExch(err, DSE_ETIMEOUT);
+          *abort_flag = 1;
+        }
+        break;
+      }
+      tc::fence_after();
+      // hi counts in units of 2^-35, lo of 2^-63 (class s: 2^(-7 (s + 2)))
+#pragma unroll
+      for (int s = 0; s < DIG; ++s) {
+        float v[32];
+        tc::tmem_ld32(at + s * RB, v);
+        const int sh_ = BITS * (3 - (s & 3));
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+          const long long w = (long long)__float2int_rn(v[i]) << sh_;
+          if (s < 4) hi[i] += w;
+          else lo[i] += w;
+        }
+      }
+      tc::fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&sh.acc_empty);
+    }
+    const int64_t i = (int64_t)bi * 128 + q * 32 + lane, j0 = (int64_t)bj * RB + half * 32;
+    const int ei = i < n ? ex[i] : INT32_MIN;
+    if (ok) {
+      // 64-bit integers below 2^51 to doubles: the bits of 1.5 * 2^52 plus the
+      // integer, less 1.5 * 2^52 (exact; one FP64 addition)
+      auto dbl = [](long long v) { return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0; };
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const int64_t j = j0 + k;
+        if (i < n && j < n && i <= j) {
+          const int ej = ex[j];
+          // the value without the columns' scales, then scaled (a zero column has digits 0)
+          const double v = fma(dbl(hi[k]), 2.9103830456733704e-11, dbl(lo[k]) * 1.0842021724855044e-19);
+          const int e = (ei == INT32_MIN ? 0 : ei) + (ej == INT32_MIN ? 0 : ej);
+          double g = e > -1000 && e < 1000 ? v * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(v, e);
+          float f = __ll2float_rn(hi[k]) * 2.9103830456733704e-11f;  // (lo adds less than 2^-40 of it or of N 2^-35)
+          const int64_t at_g = upper ? i * n + j : j * n + i;
+          if (add) {
+            g += Gm[at_g];
+            f += G32[at_g];
+          }
+          Gm[at_g] = g;
+          G32[at_g] = f;
+        }
+      }
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  tc::fence_after();
+  __syncwarp();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512u) : "memory");
+}
+
+// Per candidate, for the scan: the pivot test, its FP64 root L, z = b / L and
+// q = z^2 (valid < 0: the candidate is rejected), and the scale-free FP32
+// forms w = 1 / sqrt(its G32 diagonal) and cr = z / sqrt(Syy).
+struct Cand {
+  const double *L, *z, *q;
+  const float *w, *cr;
+};
+__global__ void k_l0_cands(const double *Gm, const float *G32, const double *b, const double *nrm2, int64_t n,
+                           const double *syy, double *L, double *z, double *q, float *w, float *cr) {
+  const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= n) return;
+  const double g = Gm[p * n + p];
+  const bool ok = g > kRank2 * nrm2[p];
+  const double l = ok ? sqrt(g) : 1.0, zz = ok ? b[p] / l : 0.0;
+  L[p] = l;
+  z[p] = zz;
+  q[p] = ok ? zz * zz : -1.0;
+  w[p] = ok ? rsqrtf(G32[p * n + p]) : 0.f;
+  cr[p] = ok ? (float)(zz / sqrt(*syy)) : 0.f;
 }
 
 // (q, subset) ordering: larger explained q first, then positions ascending
@@ -180,8 +435,11 @@ struct Hit {
   double q;
   uint64_t key;
 };
+// (q >= 0, or -1 for none: the bits as integers order alike, and FP64 compares
+// are slow on this part)
 __device__ __forceinline__ bool better(double qa, uint64_t ka, double qb, uint64_t kb) {
-  return qa > qb || (qa == qb && ka < kb);
+  const long long a = __double_as_longlong(qa), b = __double_as_longlong(qb);
+  return a > b || (a == b && ka < kb);
 }
 __device__ __forceinline__ uint64_t pack3(int64_t p0, int64_t p1, int64_t p2) {
   return ((uint64_t)p0 << 42) | ((uint64_t)p1 << 21) | (uint64_t)p2;
@@ -242,92 +500,151 @@ struct WarpTop {
 
 // Explained sum of squares of the subset, in position order (p0 < p1 < p2):
 // incremental Cholesky of the centred Gram submatrix; -1 if a pivot fails
-// the rank rule.
-__device__ __forceinline__ double explained1(const double *Gm, const double *b, const double *nrm2, int64_t n,
-                                             int64_t p0, double *L11, double *z1) {
-  const double g = Gm[p0 * n + p0];
-  if (!(g > kRank2 * nrm2[p0])) return -1.0;
+// the rank rule.  g..: the subset's Gram entries.
+__device__ __forceinline__ double explained1(double g, double b, double nrm2, double *L11, double *z1) {
+  if (!(g > kRank2 * nrm2)) return -1.0;
   *L11 = sqrt(g);
-  *z1 = b[p0] / *L11;
+  *z1 = b / *L11;
   return *z1 * *z1;
+}
+__device__ __forceinline__ double explained2(double q1, double L11, double z1, double g10, double g11, double b1,
+                                             double nrm2) {
+  const double L21 = g10 / L11;
+  const double d = g11 - L21 * L21;
+  if (!(d > kRank2 * nrm2)) return -1.0;
+  const double z2 = (b1 - L21 * z1) / sqrt(d);
+  return q1 + z2 * z2;
+}
+struct Step2 {  // the state after two pivots
+  double L21, z1, z2, q2, i11, i22;
+};
+__device__ __forceinline__ bool two_pivots(double q1, double L11, double z1, double g10, double g11, double b1,
+                                           double nrm2, Step2 *o) {
+  o->L21 = g10 / L11;
+  const double d2 = g11 - o->L21 * o->L21;
+  if (!(d2 > kRank2 * nrm2)) return false;
+  const double L22 = sqrt(d2);
+  o->z1 = z1;
+  o->z2 = (b1 - o->L21 * z1) / L22;
+  o->q2 = q1 + o->z2 * o->z2;
+  o->i11 = 1.0 / L11;
+  o->i22 = 1.0 / L22;
+  return true;
+}
+__device__ __forceinline__ double explained3(const Step2 &s, double g20, double g21, double g22, double b2,
+                                             double nrm2) {
+  const double L31 = g20 * s.i11;
+  const double L32 = (g21 - L31 * s.L21) * s.i22;
+  const double d3 = g22 - L31 * L31 - L32 * L32;
+  if (!(d3 > kRank2 * nrm2)) return -1.0;
+  const double t = b2 - L31 * s.z1 - L32 * s.z2;
+  return s.q2 + t * t / d3;
 }
 
 // Scan of every D-subset; each block writes its kTop best to out[block].
+// An FP32 bound of q / Syy from the candidates' correlations (G32 w w, within
+// 5e-7) excludes nearly every subset.  Pairs: 1 - r^2 is within 1e-6 and the
+// numerator within 1e-6.  Triples, where 1 - r^2 > 1e-2: its root is within
+// 5e-5, the second row within 6.5e-5, the last pivot within 1.4e-4 and the
+// numerator within 1.3e-4.  The margins below are wider; where a pivot is
+// smaller the bound is not used. The exact evaluation of each (about 12 FP64
+// operations, two divisions and a root) took 0.96 ms for 4.5 M pairs (0.15 now).
+// `floor`: the best 32nd-best q of any warp so far; a subset below it by
+// more than 1e-9 cannot be among the kMore best that matter.
 template <int D>
-__global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const double *b, const double *nrm2, int64_t n,
-                                                 Hit *out) {
+__global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *G32, const double *b,
+                                                 const double *nrm2, const Cand C, const double *syy, int64_t n,
+                                                 unsigned long long *floor_bits, Hit *out) {
   __shared__ Hit sh[8 * 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WarpTop top;
   top.init();
+  // what a bound has to reach, as a share of Syy (one rounding up)
+  const double isyy = *syy > 0.0 ? 1.0 / *syy : 0.0;
+  float need = -1.f;
+  auto renew = [&]() {
+    unsigned long long f = 0;
+    if (lane == 0) {
+      if (top.wq > 0.0) atomicMax(floor_bits, (unsigned long long)__double_as_longlong(top.wq));
+      f = *(volatile unsigned long long *)floor_bits;
+    }
+    f = __shfl_sync(0xffffffffu, f, 0);
+    const double q = fmax(top.wq, __longlong_as_double((long long)f));
+    need = q > 0.0 && isyy > 0.0 ? (float)(q * isyy) * (1.0f - 1e-6f) : -1.f;
+  };
   if (D == 1) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t base0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     for (int64_t base = base0 - lane; base < n; base += stride) {
       const int64_t p = base + lane;
-      double q = -1.0, L, z;
-      if (p < n) q = explained1(Gm, b, nrm2, n, p, &L, &z);
+      const double q = p < n ? C.q[p] : -1.0;
       top.offer(q >= 0.0, q, pack3(p, 0, 0));
     }
   } else if (D == 2) {
     const uint64_t npairs = (uint64_t)n * (uint64_t)(n - 1) / 2;
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t base0 = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x - lane;
+    int turn = 0;
     for (uint64_t base = base0; base < npairs; base += stride) {
       const uint64_t idx = base + lane;
-      double q = -1.0;
-      uint64_t key = ~0ull;
+      if ((++turn & 15) == 0) renew();
+      bool maybe = false;
+      int64_t p0 = 0, p1 = 0;
       if (idx < npairs) {
         uint64_t hi, lo;
         pair_from_index(idx, &hi, &lo);  // lo < hi
-        const int64_t p0 = (int64_t)lo, p1 = (int64_t)hi;
-        double L11, z1;
-        const double q1 = explained1(Gm, b, nrm2, n, p0, &L11, &z1);
-        if (q1 >= 0.0) {
-          const double L21 = Gm[p1 * n + p0] / L11;
-          const double d = Gm[p1 * n + p1] - L21 * L21;
-          if (d > kRank2 * nrm2[p1]) {
-            const double z2 = (b[p1] - L21 * z1) / sqrt(d);
-            q = q1 + z2 * z2;
-            key = pack3(p0, p1, 0);
-          }
-        }
+        p0 = (int64_t)lo, p1 = (int64_t)hi;
+        const float r = G32[p1 * n + p0] * C.w[p0] * C.w[p1], c0 = C.cr[p0];
+        const float d = fmaf(-r, r, 1.0f), x = fabsf(fmaf(-r, c0, C.cr[p1])) + 2e-6f;
+        maybe = !(d > 1e-3f) || fmaf(c0, c0, x * x / (d - 4e-6f)) * (1.0f + 1e-5f) + 1e-6f >= need;
       }
-      top.offer(q >= 0.0, q, key);
+      if (!__any_sync(0xffffffffu, maybe)) continue;
+      double q = -1.0;
+      if (maybe && C.q[p0] >= 0.0)
+        q = explained2(C.q[p0], C.L[p0], C.z[p0], Gm[p1 * n + p0], Gm[p1 * n + p1], b[p1], nrm2[p1]);
+      const double before = top.wq;
+      top.offer(q >= 0.0, q, pack3(p0, p1, 0));
+      if (top.wq != before) renew();
     }
   } else {
     // warp per pair (p0 < p1); lanes over p2 > p1
     const uint64_t npairs = (uint64_t)n * (uint64_t)(n - 1) / 2;
     const uint64_t warps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    int turn = 0;
     for (uint64_t w = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < npairs; w += warps) {
       uint64_t hi, lo;
       pair_from_index(w, &hi, &lo);
       const int64_t p0 = (int64_t)lo, p1 = (int64_t)hi;
-      if (p1 + 1 >= n) continue;
-      double L11, z1;
-      const double q1 = explained1(Gm, b, nrm2, n, p0, &L11, &z1);
-      if (q1 < 0.0) continue;
-      const double L21 = Gm[p1 * n + p0] / L11;
-      const double d2 = Gm[p1 * n + p1] - L21 * L21;
-      if (!(d2 > kRank2 * nrm2[p1])) continue;
-      const double L22 = sqrt(d2);
-      const double z2 = (b[p1] - L21 * z1) / L22;
-      const double q2 = q1 + z2 * z2;
-      const double i11 = 1.0 / L11, i22 = 1.0 / L22;
-      const double *g0 = Gm + p0 * n, *g1 = Gm + p1 * n;
-      for (int64_t base = p1 + 1; base < n; base += 32) {
+      if ((++turn & 7) == 0) renew();
+      if (p1 + 1 >= n || C.q[p0] < 0.0) continue;
+      // the FP32 forms of the two pivots; the exact ones at the first need
+      const float *f0 = G32 + p0 * n, *f1 = G32 + p1 * n;
+      const float w0 = C.w[p0], w1 = C.w[p1], c0 = C.cr[p0];
+      const float r = f0[p1] * w0 * w1, d2 = fmaf(-r, r, 1.0f);
+      const bool fine = d2 > 1e-2f;
+      const float i2 = fine ? rsqrtf(d2) : 0.f, c1 = fmaf(-r, c0, C.cr[p1]) * i2, q2 = fmaf(c0, c0, c1 * c1);
+      bool have = false, bad = false;
+      Step2 st;
+      for (int64_t base = p1 + 1; base < n && !bad; base += 32) {
         const int64_t p2 = base + lane;
-        double q = -1.0;
-        if (p2 < n) {
-          const double L31 = g0[p2] * i11;
-          const double L32 = (g1[p2] - L31 * L21) * i22;
-          const double d3 = Gm[p2 * n + p2] - L31 * L31 - L32 * L32;
-          if (d3 > kRank2 * nrm2[p2]) {
-            const double t = b[p2] - L31 * z1 - L32 * z2;
-            q = q2 + t * t / d3;
-          }
+        bool maybe = p2 < n;
+        if (maybe && fine) {
+          const float w2 = C.w[p2], l1 = f0[p2] * w0 * w2, l2 = fmaf(-l1, r, f1[p2] * w1 * w2) * i2;
+          const float d3 = fmaf(-l2, l2, fmaf(-l1, l1, 1.0f));
+          const float x = fabsf(fmaf(-l2, c1, fmaf(-l1, c0, C.cr[p2]))) + 2e-4f;
+          maybe = !(d3 > 1e-2f) || (q2 + x * x / (d3 - 2e-4f)) * (1.0f + 1e-5f) + 3e-4f >= need;
         }
+        if (!__any_sync(0xffffffffu, maybe)) continue;
+        if (!have) {
+          have = true;
+          bad = !two_pivots(C.q[p0], C.L[p0], C.z[p0], Gm[p0 * n + p1], Gm[p1 * n + p1], b[p1], nrm2[p1], &st);
+          if (bad) break;
+        }
+        double q = -1.0;
+        if (maybe) q = explained3(st, Gm[p0 * n + p2], Gm[p1 * n + p2], Gm[p2 * n + p2], b[p2], nrm2[p2]);
+        const double before = top.wq;
         top.offer(q >= 0.0, q, pack3(p0, p1, p2));
+        if (top.wq != before) renew();
       }
     }
   }
@@ -351,38 +668,85 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const double 
   if (threadIdx.x < kTop) out[(size_t)blockIdx.x * kTop + threadIdx.x] = sh[threadIdx.x];
 }
 
-// The kTop best of all blocks (one block; nb * kTop <= 8192 entries).
-__global__ void __launch_bounds__(1024) k_l0_merge(Hit *in, int64_t m, Hit *best) {
-  extern __shared__ Hit hs[];
-  int64_t M = 1;
-  while (M < m) M <<= 1;
-  for (int64_t i = threadIdx.x; i < M; i += blockDim.x) hs[i] = i < m ? in[i] : Hit{-1.0, ~0ull};
+// The kMore best of all blocks' lists (one block): each warp's 32 best of its
+// share, then a sort of the warps' 1024.  Entries clearly below the floor are
+// passed over.  (A sort of all 8192 entries took 0.43 ms; 0.10.)
+__global__ void __launch_bounds__(1024) k_l0_merge(const Hit *in, int64_t m, const unsigned long long *floor_bits,
+                                                   Hit *best) {
+  __shared__ Hit hs[1024];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double floor_q = __longlong_as_double((long long)*floor_bits) * (1.0 - 1e-9);
+  WarpTop top;
+  top.init();
+  for (int64_t base = (int64_t)warp * 32; base < m; base += 1024) {
+    const Hit h = base + lane < m ? in[base + lane] : Hit{-1.0, ~0ull};
+    top.offer(h.q >= floor_q, h.q, h.key);
+  }
+  hs[threadIdx.x] = Hit{top.q, top.key};
   __syncthreads();
-  for (int64_t size = 2; size <= M; size <<= 1)
-    for (int64_t stride = size >> 1; stride > 0; stride >>= 1) {
-      for (int64_t i = threadIdx.x; i < M; i += blockDim.x) {
-        const int64_t j = i ^ stride;
-        if (j > i) {
-          const bool up = (i & size) == 0;
-          const Hit a = hs[i], c = hs[j];
-          const bool sw = up ? better(c.q, c.key, a.q, a.key) : better(a.q, a.key, c.q, c.key);
-          if (sw) {
-            hs[i] = c;
-            hs[j] = a;
-          }
+  for (int size = 2; size <= 1024; size <<= 1)
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      const int i = threadIdx.x, j = i ^ stride;
+      if (j > i) {
+        const bool up = (i & size) == 0;
+        const Hit a = hs[i], c = hs[j];
+        const bool sw = up ? better(c.q, c.key, a.q, a.key) : better(a.q, a.key, c.q, c.key);
+        if (sw) {
+          hs[i] = c;
+          hs[j] = a;
         }
       }
       __syncthreads();
     }
-  if (threadIdx.x < kTop) best[threadIdx.x] = hs[threadIdx.x];
+  if (threadIdx.x < kMore) best[threadIdx.x] = hs[threadIdx.x];
+}
+
+// The kept subsets' Gram entries (00, 10, 11, 20, 21, 22) in plain FP64, the
+// samples in order, and their q from them (one warp each): what decides and
+// is reported does not depend on the slicing.
+__global__ void __launch_bounds__(32) k_l0_exact(Hit *best, int D, const double *X, const double *b,
+                                                 const double *nrm2, int64_t N, double *ge) {
+  __shared__ double xs[3][64];
+  const int lane = threadIdx.x;
+  const Hit h = best[blockIdx.x];
+  const int64_t p[3] = {(int64_t)((h.key >> 42) & 0x1FFFFF), (int64_t)((h.key >> 21) & 0x1FFFFF),
+                        (int64_t)(h.key & 0x1FFFFF)};
+  if (!(h.q >= 0.0)) return;
+  const int ne = D * (D + 1) / 2, e = lane < ne ? lane : 0;
+  const int r = e == 0 ? 0 : e < 3 ? 1 : 2, c = e == 0 || e == 1 || e == 3 ? 0 : e == 5 ? 2 : 1;
+  double acc = 0.0;
+  for (int64_t s0 = 0; s0 < N; s0 += 64) {
+    __syncwarp();
+    for (int d = 0; d < D; ++d)
+      for (int i = lane; i < 64; i += 32) xs[d][i] = s0 + i < N ? X[p[d] * N + s0 + i] : 0.0;
+    __syncwarp();
+#pragma unroll 8
+    for (int i = 0; i < 64; ++i) acc = fma(xs[c][i], xs[r][i], acc);
+  }
+  double g[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) g[k] = __shfl_sync(0xffffffffu, acc, k);
+  if (lane == 0) {
+    for (int k = 0; k < ne; ++k) ge[(size_t)blockIdx.x * 6 + k] = g[k];
+    double L11, z1;
+    double q = explained1(g[0], b[p[0]], nrm2[p[0]], &L11, &z1);
+    if (q >= 0.0 && D == 2) q = explained2(q, L11, z1, g[1], g[2], b[p[1]], nrm2[p[1]]);
+    if (q >= 0.0 && D == 3) {
+      Step2 st;
+      q = two_pivots(q, L11, z1, g[1], g[2], b[p[1]], nrm2[p[1]], &st)
+              ? explained3(st, g[3], g[4], g[5], b[p[2]], nrm2[p[2]])
+              : -1.0;
+    }
+    best[blockIdx.x].q = q;
+  }
 }
 
 // Explicit FP64 refit of each kept subset (one block each): coefficients
 // from the centred Cholesky, RMSE of the explicit residual.
 __global__ void __launch_bounds__(kCol) k_l0_refit(const Hit *best, int D, const double *X, const double *yc,
-                                                   const double *mean, const double *Gm, const double *b,
-                                                   const double *nrm2, int64_t n, int64_t N, double my,
-                                                   double *rmse, double *coef) {
+                                                   const double *mean, const double *ge, const double *b,
+                                                   const double *nrm2, int64_t N, double my, double *rmse,
+                                                   double *coef) {
   __shared__ double sm[(kCol / 32) * 2];
   const Hit h = best[blockIdx.x];
   int64_t p[3];
@@ -390,11 +754,12 @@ __global__ void __launch_bounds__(kCol) k_l0_refit(const Hit *best, int D, const
   p[1] = (int64_t)((h.key >> 21) & 0x1FFFFF);
   p[2] = (int64_t)(h.key & 0x1FFFFF);
   bool ok = h.q >= 0.0;
+  const double *g = ge + (size_t)blockIdx.x * 6;
   double beta[4] = {0, 0, 0, 0};
   if (ok) {
     double L[3][3] = {}, z[3];
     for (int c = 0; c < D && ok; ++c) {
-      double dsum = Gm[p[c] * n + p[c]];
+      double dsum = g[c * (c + 1) / 2 + c];
       for (int k = 0; k < c; ++k) dsum -= L[c][k] * L[c][k];
       if (!(dsum > kRank2 * nrm2[p[c]])) {
         ok = false;
@@ -402,7 +767,7 @@ __global__ void __launch_bounds__(kCol) k_l0_refit(const Hit *best, int D, const
       }
       L[c][c] = sqrt(dsum);
       for (int r = c + 1; r < D; ++r) {
-        double v = Gm[p[r] * n + p[c]];
+        double v = g[r * (r + 1) / 2 + c];
         for (int k = 0; k < c; ++k) v -= L[r][k] * L[c][k];
         L[r][c] = v / L[c][c];
       }
@@ -451,12 +816,19 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
         set_error("candidate id %llu out of range", (unsigned long long)d->ids[i]);
         return DSE_ERANGE;
       }
-  const int64_t nt = (n + kGT - 1) / kGT;
+  // digit images: panels of samples, 16 n bytes a sample, 2 GB at most
+  const int nblk = 2 * (int)((n + 127) / 128);
+  const int64_t panel = std::min<int64_t>((N + 511) / 512 * 512,
+                                          std::max<int64_t>(512, ((int64_t)2 << 30) / (16 * 64 * (int64_t)nblk) / 512 * 512));
   const int sms = sm_count();
   const int nb = std::min<int64_t>(2 * sms, 8192 / kTop);  // scan blocks (their kTop bests fit the merge)
   // scratch
   double *yd = nullptr, *yc = nullptr, *syy = nullptr, *ym = nullptr, *X = nullptr, *nrm2 = nullptr, *bv = nullptr, *mean = nullptr,
-         *Gm = nullptr, *rm = nullptr, *cf = nullptr;
+         *Gm = nullptr, *rm = nullptr, *cf = nullptr, *cL = nullptr, *cz = nullptr, *cq = nullptr, *ge = nullptr;
+  float *G32 = nullptr, *cw = nullptr, *cc = nullptr;
+  int *ex = nullptr, *err = nullptr;
+  unsigned char *img = nullptr;
+  unsigned long long *floor_bits = nullptr;
   uint64_t *ids = nullptr;
   Hit *part = nullptr, *best = nullptr;
   Scratch sc;
@@ -471,9 +843,19 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
   sc.add(&mean, (size_t)n);
   sc.add(&Gm, (size_t)n * n);
   sc.add(&part, (size_t)nb * kTop);
-  sc.add(&best, kTop);
-  sc.add(&rm, kTop);
-  sc.add(&cf, (size_t)kTop * 4);
+  sc.add(&best, kMore);
+  sc.add(&G32, (size_t)n * n);
+  sc.add(&ex, (size_t)n);
+  sc.add(&img, (size_t)nblk * (size_t)(panel / sliced::KC) * sliced::CHUNK);
+  sc.add(&cL, (size_t)n);
+  sc.add(&cz, (size_t)n);
+  sc.add(&cq, (size_t)n);
+  sc.add(&cw, (size_t)n);
+  sc.add(&cc, (size_t)n);
+  sc.add(&ge, (size_t)kMore * 6);
+  sc.add(&floor_bits, 2);
+  sc.add(&rm, kMore);
+  sc.add(&cf, (size_t)kMore * 4);
   void *base = nullptr;
   size_t bytes = 0;
   DSE_TRY(sc.alloc(&base, &bytes));
@@ -492,54 +874,76 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
     idp = ids;
   }
   const FeatTable F = table_of(sp);
-  note_launches(6);
+  err = reinterpret_cast<int *>(floor_bits + 1);
+  DSE_CUDA(cudaMemsetAsync(floor_bits, 0, 16, st));
+  static bool attr[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!attr[dev & 63]) {
+    DSE_CUDA(cudaFuncSetAttribute(k_l0_gram, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sliced::SMEM));
+    attr[dev & 63] = true;
+  }
+  note_launches(8);
   k_l0_target<<<1, kCol, 0, st>>>(y, N, yc, syy, ym);
   k_l0_columns<<<(unsigned)n, kCol, 0, st>>>(F, sp->geom, sp->n, idp, n, yc, X, nrm2, bv, mean);
-  k_l0_gram<<<(unsigned)(nt * (nt + 1) / 2), 256, 0, st>>>(X, n, N, nt, Gm);
-  if (D == 1) k_l0_scan<1><<<nb, 256, 0, st>>>(Gm, bv, nrm2, n, part);
-  else if (D == 2) k_l0_scan<2><<<nb, 256, 0, st>>>(Gm, bv, nrm2, n, part);
-  else k_l0_scan<3><<<nb, 256, 0, st>>>(Gm, bv, nrm2, n, part);
-  {
-    int64_t M = 1;
-    while (M < (int64_t)nb * kTop) M <<= 1;
-    const size_t sm = (size_t)M * sizeof(Hit);
-    static bool attr = false;
-    if (!attr) {
-      DSE_CUDA(cudaFuncSetAttribute(k_l0_merge, cudaFuncAttributeMaxDynamicSharedMemorySize, 8192 * (int)sizeof(Hit)));
-      attr = true;
-    }
-    k_l0_merge<<<1, 1024, sm, st>>>(part, (int64_t)nb * kTop, best);
+  k_l0_exponents<<<(unsigned)n, kCol, 0, st>>>(X, N, ex);
+  const int64_t hb2 = nblk / 2, tiles = hb2 * (nblk + 1 - hb2);  // i-blocks 0..nblk/2 - 1 (see k_l0_gram)
+  for (int64_t s0 = 0; s0 < N; s0 += panel) {
+    const int64_t ns = std::min(panel, N - s0);
+    const int nc = (int)((ns + sliced::KC - 1) / sliced::KC);
+    note_launches(2);
+    k_l0_slices<<<dim3((unsigned)nc, (unsigned)nblk), 128, 0, st>>>(X, ex, n, N, s0, ns, nc, img);
+    k_l0_gram<<<(unsigned)tiles, sliced::THREADS, sliced::SMEM, st>>>(img, ex, n, nc, s0 > 0 ? 1 : 0, D == 3 ? 1 : 0, Gm, G32, err);
   }
-  k_l0_refit<<<kTop, kCol, 0, st>>>(best, D, X, yc, mean, Gm, bv, nrm2, n, N, 0.0, rm, cf);
+  k_l0_cands<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(Gm, G32, bv, nrm2, n, syy, cL, cz, cq, cw, cc);
+  const Cand cands{cL, cz, cq, cw, cc};
+  if (D == 1) k_l0_scan<1><<<nb, 256, 0, st>>>(Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  else if (D == 2) k_l0_scan<2><<<nb, 256, 0, st>>>(Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  else k_l0_scan<3><<<nb, 256, 0, st>>>(Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  k_l0_merge<<<1, 1024, 0, st>>>(part, (int64_t)nb * kTop, floor_bits, best);
+  k_l0_exact<<<kMore, 32, 0, st>>>(best, D, X, bv, nrm2, N, ge);
+  k_l0_refit<<<kMore, kCol, 0, st>>>(best, D, X, yc, mean, ge, bv, nrm2, N, 0.0, rm, cf);
   DSE_CUDA(cudaGetLastError());
   // reports: RMSEs, coefficients (intercept without the target's mean), the
   // subsets and the target's mean, one wait
-  double *hs = static_cast<double *>(pinned_staging(8 * (kTop * 5 + 1) + sizeof(Hit) * kTop));
+  double *hs = static_cast<double *>(pinned_staging(8 * (kMore * 5 + 2) + sizeof(Hit) * kMore));
   if (!hs) return DSE_ENOMEM;
-  Hit *hb = reinterpret_cast<Hit *>(hs + kTop * 5 + 1);
-  DSE_CUDA(cudaMemcpyAsync(hs, rm, 8 * kTop, cudaMemcpyDeviceToHost, st));
-  DSE_CUDA(cudaMemcpyAsync(hs + kTop, cf, 8 * kTop * 4, cudaMemcpyDeviceToHost, st));
-  DSE_CUDA(cudaMemcpyAsync(hs + kTop * 5, ym, 8, cudaMemcpyDeviceToHost, st));
-  DSE_CUDA(cudaMemcpyAsync(hb, best, sizeof(Hit) * kTop, cudaMemcpyDeviceToHost, st));
+  Hit *hb = reinterpret_cast<Hit *>(hs + kMore * 5 + 2);
+  DSE_CUDA(cudaMemcpyAsync(hs, rm, 8 * kMore, cudaMemcpyDeviceToHost, st));
+  DSE_CUDA(cudaMemcpyAsync(hs + kMore, cf, 8 * kMore * 4, cudaMemcpyDeviceToHost, st));
+  DSE_CUDA(cudaMemcpyAsync(hs + kMore * 5, ym, 8, cudaMemcpyDeviceToHost, st));
+  DSE_CUDA(cudaMemcpyAsync(hs + kMore * 5 + 1, err, sizeof(int), cudaMemcpyDeviceToHost, st));
+  DSE_CUDA(cudaMemcpyAsync(hb, best, sizeof(Hit) * kMore, cudaMemcpyDeviceToHost, st));
   DSE_CUDA(cudaStreamSynchronize(st));
-  const double my = hs[kTop * 5];
+  if (*reinterpret_cast<const int *>(hs + kMore * 5 + 1)) {
+    set_error("a bounded device wait timed out");
+    return DSE_ETIMEOUT;
+  }
+  const double my = hs[kMore * 5];
   struct Row {
-    double rmse;
+    double q, rmse;
+    uint64_t key;
     int64_t p[3];
     double c[4];
   };
   std::vector<Row> rows;
-  for (int i = 0; i < kTop; ++i) {
-    if (!(hb[i].q >= 0.0) || !(hs[i] < INFINITY)) continue;
+  for (int i = 0; i < kMore; ++i) {
+    if (!(hb[i].q >= 0.0)) continue;
     Row r;
+    r.q = hb[i].q;
     r.rmse = hs[i];
+    r.key = hb[i].key;
     r.p[0] = (int64_t)((hb[i].key >> 42) & 0x1FFFFF);
     r.p[1] = (int64_t)((hb[i].key >> 21) & 0x1FFFFF);
     r.p[2] = (int64_t)(hb[i].key & 0x1FFFFF);
-    for (int c = 0; c < 4; ++c) r.c[c] = hs[kTop + i * 4 + c];
+    for (int c = 0; c < 4; ++c) r.c[c] = hs[kMore + i * 4 + c];
     r.c[0] += my;
     rows.push_back(r);
   }
+  // the kTop of largest q; of those the full-rank fits, by RMSE
+  std::sort(rows.begin(), rows.end(), [](const Row &a, const Row &c) { return a.q > c.q || (a.q == c.q && a.key < c.key); });
+  if (rows.size() > (size_t)kTop) rows.resize(kTop);
+  rows.erase(std::remove_if(rows.begin(), rows.end(), [](const Row &r) { return !(r.rmse < INFINITY); }), rows.end());
   std::sort(rows.begin(), rows.end(), [&](const Row &a, const Row &c) {
     if (a.rmse != c.rmse) return a.rmse < c.rmse;
     for (int k = 0; k < D; ++k)

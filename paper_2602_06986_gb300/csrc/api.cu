@@ -295,6 +295,7 @@ uint64_t count_slots_mod(uint64_t x, int nb, const std::vector<int> &posset) {
 // statistics and re-score job counts (n_jobs[0..2)).
 __global__ void k_screen_reset(unsigned *count, unsigned *hist, unsigned *hist_hi, unsigned *hist_c, int nl,
                                unsigned *esc_count, unsigned long long *stats, unsigned *n_jobs) {
+  pdl_enter();
   const int64_t nh = (int64_t)nl * kNumBins, nc = (int64_t)nl * kCoarse;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nh; e += (int64_t)gridDim.x * blockDim.x) {
     hist[e] = 0u;
@@ -319,8 +320,7 @@ static dse_status run_screen(dse_result *R, const ScreenPlan &plan, void *scr_ti
   const int64_t launches0 = launches_so_far();
   // the screen's counters and histograms, zeroed by one kernel
   note_launches(1);
-  k_screen_reset<<<std::max(1, std::min(sms, (int)((nl * kNumBins + 255) / 256))), 256, 0, st>>>(
-      A.B.count, A.B.hist, A.B.hist_hi, A.B.hist_c, nl, A.esc_count, A.stats, S.n_jobs);
+  launch_k(k_screen_reset, std::max(1, std::min(sms, (int)((nl * kNumBins + 255) / 256))), 256, 0, st, A.B.count, A.B.hist, A.B.hist_hi, A.B.hist_c, nl, A.esc_count, A.stats, S.n_jobs);
   // per-candidate reasons: -1 until a kernel decides the candidate
   if (A.why) DSE_CUDA(cudaMemsetAsync(A.why, 0xff, (size_t)(A.id_end - A.id_begin), st));
   // intervals: NaN (all bits set) until a kernel writes one
@@ -947,6 +947,7 @@ constexpr int kSmall = ST_COUNT + 5;  // per iteration: counters, overflow, buff
 __global__ void k_loop_snapshot(const unsigned long long *stats, const unsigned *overflow, const unsigned *buf_count,
                                 const int64_t *out_n, const double *max_eps, int *err, const uint64_t *out_id,
                                 int64_t k, unsigned long long *small, uint64_t *ids, float *theta, int n_lists) {
+  pdl_enter();
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (t < ST_COUNT) small[t] = stats[t];
   if (t == 0) {
@@ -1042,8 +1043,7 @@ static dse_status residual_loop_impl(dse_space *sp, const dse_loop_desc *d, dse_
 
   auto snapshot = [&](int it) -> dse_status {
     note_launches(1);
-    k_loop_snapshot<<<(unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (k + 255) / 256)), 256, 0, st>>>(
-        R->stats, R->overflow, R->buf_count, R->out_n, R->max_eps, R->err, R->out_id, k,
+    launch_k(k_loop_snapshot, (unsigned)std::max<int64_t>(1, std::min<int64_t>(64, (k + 255) / 256)), 256, 0, st, R->stats, R->overflow, R->buf_count, R->out_n, R->max_eps, R->err, R->out_id, k,
         small + (size_t)it * kSmall, ids + (size_t)it * k, kp->A.B.theta, R->n_lists);
     return DSE_OK;
   };

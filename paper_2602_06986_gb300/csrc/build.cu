@@ -25,6 +25,7 @@ namespace dse {
 
 __global__ void k_gather_rows(const double *X, int64_t ldx, const int64_t *idx, int64_t n0, int64_t N, int64_t ld,
                               double *out) {
+  pdl_enter();
   int64_t total = n0 * ld;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     int64_t f = e / ld, s = e % ld;
@@ -73,6 +74,7 @@ __global__ void __launch_bounds__(kSumThreads) k_summaries(double *v64, int64_t 
                                                            double *max64, double *minabs64, double *maxabs64,
                                                            double *minabsnz64, double fmin_std_rel, uint8_t *ok,
                                                            const unsigned long long *n_dev) {
+  pdl_enter();
   __shared__ double smd[kSumThreads / 32];
   // the partials of the merged reductions: per warp {sum, min|x|} after the
   // first pass, then {min, max, max|x|, min nonzero |x|, finite, sxx, s2, rs}
@@ -219,6 +221,7 @@ __global__ void __launch_bounds__(kSumThreads) k_summaries(double *v64, int64_t 
 // scratch rows: one block per slot, one evaluation per sample.
 __global__ void __launch_bounds__(kSumThreads) k_eval_rows(FeatTable F, RungGeom g, const uint64_t *list, uint64_t cap,
                                                            const unsigned long long *n_dev, double *rows) {
+  pdl_enter();
   const uint64_t w = blockIdx.x;
   if (w >= cap || w >= *n_dev) return;
   int op;
@@ -260,6 +263,7 @@ __global__ void __launch_bounds__(kSumThreads) k_take_eval(FeatTable F, RungGeom
                                                            int64_t *ca_out, int64_t *cb_out, int32_t *cplx_out,
                                                            int32_t *units_out, uint64_t *used_out,
                                                            uint64_t *dmask_out) {
+  pdl_enter();
   const uint64_t w = blockIdx.x;
   if (w >= n_keep) return;
   const uint64_t p = pos[w];
@@ -293,6 +297,7 @@ __global__ void __launch_bounds__(kSumThreads) k_take_eval(FeatTable F, RungGeom
 
 // A-priori reason of every flat slot of rung r.
 __global__ void k_apriori_rung(FeatTable F, RungGeom g, AprioriParams P, uint8_t *why, int *bad) {
+  pdl_enter();
   for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < g.slots;
        p += (uint64_t)gridDim.x * blockDim.x) {
     int op;
@@ -313,6 +318,7 @@ __global__ void k_take_rows(const int64_t *keep, int64_t nk, int64_t ld, const d
                             const double *maxabs64, const double *minabsnz64, double *o_v64, double *o_mean64,
                             double *o_rmean64, double *o_min64, double *o_max64, double *o_minabs64,
                             double *o_maxabs64, double *o_minabsnz64) {
+  pdl_enter();
   const int64_t f = blockIdx.x;
   if (f >= nk) return;
   const int64_t p = keep[f];
@@ -339,6 +345,7 @@ __global__ void __launch_bounds__(kPrepThreads)
                 const double *mean64, const double *rmean64, const double *min64, const double *max64,
                 const double *minabs64, const double *maxabs64, const double *minabsnz64, const int32_t *units,
                 double exp_arg_max, float4 *fa, float2 *fr, uint32_t *flags, uint64_t *ukey, float *fnorm) {
+  pdl_enter();
   __shared__ double red[kPrepThreads / 32];
   const int lane = threadIdx.x & 31;
   for (int64_t f = blockIdx.x; f < n; f += gridDim.x) {
@@ -450,6 +457,7 @@ constexpr int64_t kClassStage = 2048;
 
 __global__ void k_class_rows(const uint64_t *ukey, int64_t n, int one_class, int32_t *class_rows,
                              int32_t *rowid_ident) {
+  pdl_enter();
   extern __shared__ uint64_t sk[];
   const bool staged = n <= kClassStage;
   if (staged && !one_class) {
@@ -485,6 +493,7 @@ struct CopySegs {
 };
 
 __global__ void k_copy_segments(const CopySegs c) {
+  pdl_enter();
   const int k = blockIdx.y;
   if (k >= c.n) return;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < c.words[k];
@@ -519,7 +528,7 @@ static dse_status table_copy(TableArrays &dst, const TableArrays &src, int64_t n
   add(dst.dmask, src.dmask, 8 * n);
   const uint64_t big = (uint64_t)2 * n * ld;  // the rows are the longest copy
   note_launches(1);
-  k_copy_segments<<<dim3((unsigned)std::min<uint64_t>(1024, (big + 255) / 256), (unsigned)c.n), 256, 0, s>>>(c);
+  launch_k(k_copy_segments, dim3((unsigned)std::min<uint64_t>(1024, (big + 255) / 256), (unsigned)c.n), 256, 0, s, c);
   DSE_CUDA(cudaGetLastError());
   return DSE_OK;
 }
@@ -620,10 +629,10 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
   }
   TableArrays T0;
   DSE_TRY(table_alloc(T0, n0, ld, false));
-  k_gather_rows<<<grid_for(n0 * ld, 256), 256, 0, st>>>(Xd, ldx, idx_d, n0, N, ld, T0.v64);
+  launch_k(k_gather_rows, grid_for(n0 * ld, 256), 256, 0, st, Xd, ldx, idx_d, n0, N, ld, T0.v64);
   uint8_t *ok = nullptr;
   DSE_TRY(dalloc(&ok, n0, "primary flags"));
-  k_summaries<<<(unsigned)n0, kSumThreads, 0, st>>>(T0.v64, ld, N, 0, n0, T0.mean64, T0.rmean64, T0.min64,
+  launch_k(k_summaries, (unsigned)n0, kSumThreads, 0, st, T0.v64, ld, N, 0, n0, T0.mean64, T0.rmean64, T0.min64,
                                                        T0.max64, T0.minabs64, T0.maxabs64, T0.minabsnz64,
                                                        S->fmin_std_rel, ok, nullptr);
   std::vector<uint8_t> hok(n0);
@@ -695,7 +704,7 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
     };
     DSE_CUDA(up(keep_d, keep.data(), 8 * nk));
     note_launches(1);
-    k_take_rows<<<(unsigned)nk, 128, 0, st>>>(keep_d, nk, ld, T0.v64, T0.mean64, T0.rmean64, T0.min64, T0.max64,
+    launch_k(k_take_rows, (unsigned)nk, 128, 0, st, keep_d, nk, ld, T0.v64, T0.mean64, T0.rmean64, T0.min64, T0.max64,
                                               T0.minabs64, T0.maxabs64, T0.minabsnz64, T.v64, T.mean64, T.rmean64,
                                               T.min64, T.max64, T.minabs64, T.maxabs64, T.minabsnz64);
     dfree(keep_d);
@@ -740,7 +749,7 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
     DSE_TRY(dalloc(&vlist, g.slots, "valid list"));
     DSE_CUDA(cudaMemsetAsync(meta, 0, 10 * sizeof(unsigned long long), st));
     note_launches(1);
-    if (g.slots) k_apriori_rung<<<grid_for(g.slots, 256), 256, 0, st>>>(F, g, P, why, (int *)(meta + 8));
+    if (g.slots) launch_k(k_apriori_rung, grid_for(g.slots, 256), 256, 0, st, F, g, P, why, (int *)(meta + 8));
     launch_count_reasons(why, g.slots, meta, st);
     DSE_TRY(compact_bytes_dev(why, g.slots, DSE_VALID, list, meta + 6, st));
     dfree(why);
@@ -764,8 +773,8 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
     DSE_CUDA(cudaMemsetAsync(rw, 0, g.slots, st));
     note_launches(2);
     if (cap_rows) {
-      k_eval_rows<<<(unsigned)cap_rows, kSumThreads, 0, st>>>(F, g, list, cap_rows, meta + 6, rows);
-      k_summaries<<<(unsigned)cap_rows, kSumThreads, 0, st>>>(rows, ld, N, 0, (int64_t)cap_rows, rsum.mean64,
+      launch_k(k_eval_rows, (unsigned)cap_rows, kSumThreads, 0, st, F, g, list, cap_rows, meta + 6, rows);
+      launch_k(k_summaries, (unsigned)cap_rows, kSumThreads, 0, st, rows, ld, N, 0, (int64_t)cap_rows, rsum.mean64,
                                                              rsum.rmean64, rsum.min64, rsum.max64, rsum.minabs64,
                                                              rsum.maxabs64, rsum.minabsnz64, S->fmin_std_rel, rw,
                                                              meta + 6);
@@ -807,7 +816,7 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
     RowSummaries dsum{T2.mean64, T2.rmean64, T2.min64, T2.max64, T2.minabs64, T2.maxabs64, T2.minabsnz64};
     note_launches(1);
     if (n_new)
-      k_take_eval<<<(unsigned)n_new, kSumThreads, 0, st>>>(Fold, g, P, list, vlist, n_new, n, rows, rsum, T2.v64, dsum,
+      launch_k(k_take_eval, (unsigned)n_new, kSumThreads, 0, st, Fold, g, P, list, vlist, n_new, n, rows, rsum, T2.v64, dsum,
                                                            T2.op, T2.ca, T2.cb, T2.cplx, T2.units, T2.used, T2.dmask);
     drop_scratch();
     // stream-ordered frees: the old table and the scratch stay valid for
@@ -843,7 +852,7 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
   DSE_TRY(dalloc(&S->fnorm, n, "helpers"));
   DSE_TRY(dalloc(&S->flags, n, "flags"));
   DSE_TRY(dalloc(&S->ukey, 2 * n, "unit keys"));
-  k_fp32_prep<<<(unsigned)std::min<int64_t>(std::max<int64_t>(n, 1), 65535), kPrepThreads, 0, st>>>(n, N, ld, S->D, T.v64, S->v32, S->v32lo, T.mean64, T.rmean64, T.min64,
+  launch_k(k_fp32_prep, (unsigned)std::min<int64_t>(std::max<int64_t>(n, 1), 65535), kPrepThreads, 0, st, n, N, ld, S->D, T.v64, S->v32, S->v32lo, T.mean64, T.rmean64, T.min64,
                                                      T.max64, T.minabs64, T.maxabs64, T.minabsnz64, T.units,
                                                      S->exp_arg_max, S->fa, S->fr, S->flags, S->ukey, S->fnorm);
   dfree(T.minabsnz64);
@@ -893,7 +902,7 @@ static dse_status build_impl(const dse_space_desc *d, dse_space *S) {
     // would synchronise the stream; the rank count is O(n^2))
     note_launches(1);
     const size_t shm = n <= kClassStage && !one_class ? (size_t)16 * n : 0;
-    k_class_rows<<<(unsigned)((n + 7) / 8), 256, shm, st>>>(S->ukey, n, one_class ? 1 : 0, S->class_rows,
+    launch_k(k_class_rows, (unsigned)((n + 7) / 8), 256, shm, st, S->ukey, n, one_class ? 1 : 0, S->class_rows,
                                                            S->rowid_ident);
   } else {
     std::vector<int32_t> ident(n);
@@ -969,6 +978,7 @@ FeatTable table_of(const dse_space *S) {
 
 // A-priori reason counts of rung max_rung (no evaluation).
 __global__ void k_count_apriori(FeatTable F, RungGeom g, AprioriParams P, unsigned long long *counts) {
+  pdl_enter();
   __shared__ unsigned int c[6];
   if (threadIdx.x < 6) c[threadIdx.x] = 0;
   __syncthreads();
@@ -993,7 +1003,7 @@ dse_status count_last_rung(dse_space *S, cudaStream_t st) {
   DSE_CUDA(cudaMemsetAsync(cnt, 0, 6 * sizeof(unsigned long long), st));
   AprioriParams P{S->D, S->unit_check_addsub, S->explog_dimensionless, S->max_complexity, S->fmax_max,
                   S->exp_arg_max};
-  if (S->geom.slots) k_count_apriori<<<grid_for(S->geom.slots, 256, 152 * 32), 256, 0, st>>>(table_of(S), S->geom, P, cnt);
+  if (S->geom.slots) launch_k(k_count_apriori, grid_for(S->geom.slots, 256, 152 * 32), 256, 0, st, table_of(S), S->geom, P, cnt);
   unsigned long long hc[6];
   DSE_CUDA(cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, st));
   DSE_CUDA(cudaStreamSynchronize(st));

@@ -57,6 +57,7 @@ __device__ __forceinline__ double block_sum128(double v, double *sm) {
 __global__ void __launch_bounds__(kUnitThreads) k_dedup_unit(FeatTable F, RungGeom G, int64_t n_stored,
                                                              const uint64_t *ids, const int64_t *n_list, int64_t kk,
                                                              int l0, double *z) {
+  pdl_enter();
   __shared__ double sm[kUnitThreads / 32];
   const int l = l0 + (int)blockIdx.y;
   const int64_t i = blockIdx.x;
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(kFlagThreads) k_dedup_flags(const uint64_t *id
                                                               const int64_t *n_list, const double *max_eps,
                                                               int64_t kk, int l0, int64_t N, const double *z,
                                                               double tau, double w_tau, uint8_t *red) {
+  pdl_enter();
   __shared__ int found;
   const int l = l0 + (int)blockIdx.y;
   const int64_t i = blockIdx.x, n = n_list[l];
@@ -138,6 +140,7 @@ __global__ void k_dedup_compact(const uint64_t *ids, const double *score, const 
                                 const double *max_eps, int64_t kk, int64_t k, int full, double w_tau,
                                 const uint8_t *red, uint64_t *o_id, double *o_score, double *o_eps, int64_t *o_n,
                                 double *o_max_eps, int *undecided, int64_t *n_red) {
+  pdl_enter();
   const int l = blockIdx.x;
   const int lane = threadIdx.x;
   const int64_t n = n_list[l];
@@ -202,8 +205,8 @@ dse_status dedup_result(dse_result *R, int64_t k, double tau, bool full, bool *u
     const int nl = std::min(chunk, L - l0);
     const dim3 grid((unsigned)kk, (unsigned)nl);
     note_launches(2);
-    k_dedup_unit<<<grid, kUnitThreads, 0, st>>>(F, sp->geom, sp->n, R->out_id, R->out_n, kk, l0, z);
-    k_dedup_flags<<<grid, kFlagThreads, 0, st>>>(R->out_id, R->out_score, R->out_n, R->max_eps, kk, l0, N, z, tau,
+    launch_k(k_dedup_unit, grid, kUnitThreads, 0, st, F, sp->geom, sp->n, R->out_id, R->out_n, kk, l0, z);
+    launch_k(k_dedup_flags, grid, kFlagThreads, 0, st, R->out_id, R->out_score, R->out_n, R->max_eps, kk, l0, N, z, tau,
                                                  w_tau, red);
   }
   // new lists: ids, scores, bounds [L][k], lengths, bounds, flags, counts
@@ -220,7 +223,7 @@ dse_status dedup_result(dse_result *R, int64_t k, double tau, bool full, bool *u
   int *o_un = reinterpret_cast<int *>(buf + off_un);
   int64_t *o_nr = reinterpret_cast<int64_t *>(buf + off_nr);
   note_launches(1);
-  k_dedup_compact<<<(unsigned)L, 32, 0, st>>>(R->out_id, R->out_score, R->out_eps, R->out_n, R->max_eps, kk, k,
+  launch_k(k_dedup_compact, (unsigned)L, 32, 0, st, R->out_id, R->out_score, R->out_eps, R->out_n, R->max_eps, kk, k,
                                               full ? 1 : 0, w_tau, red, o_id, o_sc, o_ep, o_n, o_me, o_un, o_nr);
   dfree(z);
   dfree(red);

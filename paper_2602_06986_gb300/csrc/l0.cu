@@ -80,6 +80,7 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double *sm) {
 // Centred target and Syy (one block).
 __global__ void __launch_bounds__(kCol) k_l0_target(const double *y, int64_t N, double *yc, double *syy,
                                                     double *ymean) {
+  pdl_enter();
   __shared__ double sm[(kCol / 32) * 2];
   double s[1] = {0.0};
   for (int64_t i = threadIdx.x; i < N; i += kCol) s[0] += y[i];
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(kCol) k_l0_target(const double *y, int64_t N, 
 __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, int64_t n_stored, const uint64_t *ids,
                                                      int64_t n, const double *yc, double *X, double *nrm2, double *b,
                                                      double *mean) {
+  pdl_enter();
   __shared__ double sm[(kCol / 32) * 2];
   const int64_t c = blockIdx.x;
   if (c >= n) return;
@@ -174,6 +176,7 @@ __device__ __forceinline__ uint64_t desc(uint32_t saddr) {
 // Exponent e of each column: |x| <= 2^(e-1) for every sample (one block per
 // column; 0 and nothing to slice for a zero or non-finite column).
 __global__ void __launch_bounds__(kCol) k_l0_exponents(const double *X, int64_t N, int *ex) {
+  pdl_enter();
   __shared__ unsigned long long sm[kCol / 32];
   const double *x = X + (int64_t)blockIdx.x * N;
   unsigned long long m = 0;  // (the bits of |x| order like the values)
@@ -200,6 +203,7 @@ __global__ void __launch_bounds__(kCol) k_l0_exponents(const double *X, int64_t 
 // one row and half of its samples.
 __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *ex, int64_t n, int64_t N, int64_t s0,
                                                    int64_t ns, int nc, unsigned char *img) {
+  pdl_enter();
   using namespace sliced;
   const int c = blockIdx.x, rb = blockIdx.y, row = threadIdx.x & 63, h = threadIdx.x >> 6;
   const int64_t col = (int64_t)rb * RB + row, k0 = (int64_t)c * KC + 8 * h;
@@ -237,6 +241,7 @@ __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *e
 __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned char *img, const int *ex, int64_t n,
                                                                 int nc, int add, int upper, double *Gm, float *G32,
                                                                 int *err) {
+  pdl_enter();
   using namespace sliced;
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared &sh = *reinterpret_cast<Shared *>(smem);
@@ -417,6 +422,7 @@ struct Cand {
 };
 __global__ void k_l0_cands(const double *Gm, const float *G32, const double *b, const double *nrm2, int64_t n,
                            const double *syy, double *L, double *z, double *q, float *w, float *cr) {
+  pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n) return;
   const double g = Gm[p * n + p];
@@ -555,6 +561,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *G32, const double *b,
                                                  const double *nrm2, const Cand C, const double *syy, int64_t n,
                                                  unsigned long long *floor_bits, Hit *out) {
+  pdl_enter();
   __shared__ Hit sh[8 * 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   WarpTop top;
@@ -673,6 +680,7 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
 // passed over.  (A sort of all 8192 entries took 0.43 ms; 0.10.)
 __global__ void __launch_bounds__(1024) k_l0_merge(const Hit *in, int64_t m, const unsigned long long *floor_bits,
                                                    Hit *best) {
+  pdl_enter();
   __shared__ Hit hs[1024];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const double floor_q = __longlong_as_double((long long)*floor_bits) * (1.0 - 1e-9);
@@ -706,6 +714,7 @@ __global__ void __launch_bounds__(1024) k_l0_merge(const Hit *in, int64_t m, con
 // is reported does not depend on the slicing.
 __global__ void __launch_bounds__(32) k_l0_exact(Hit *best, int D, const double *X, const double *b,
                                                  const double *nrm2, int64_t N, double *ge) {
+  pdl_enter();
   __shared__ double xs[3][64];
   const int lane = threadIdx.x;
   const Hit h = best[blockIdx.x];
@@ -747,6 +756,7 @@ __global__ void __launch_bounds__(kCol) k_l0_refit(const Hit *best, int D, const
                                                    const double *mean, const double *ge, const double *b,
                                                    const double *nrm2, int64_t N, double my, double *rmse,
                                                    double *coef) {
+  pdl_enter();
   __shared__ double sm[(kCol / 32) * 2];
   const Hit h = best[blockIdx.x];
   int64_t p[3];
@@ -884,25 +894,25 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
     attr[dev & 63] = true;
   }
   note_launches(8);
-  k_l0_target<<<1, kCol, 0, st>>>(y, N, yc, syy, ym);
-  k_l0_columns<<<(unsigned)n, kCol, 0, st>>>(F, sp->geom, sp->n, idp, n, yc, X, nrm2, bv, mean);
-  k_l0_exponents<<<(unsigned)n, kCol, 0, st>>>(X, N, ex);
+  launch_k(k_l0_target, 1, kCol, 0, st, y, N, yc, syy, ym);
+  launch_k(k_l0_columns, (unsigned)n, kCol, 0, st, F, sp->geom, sp->n, idp, n, yc, X, nrm2, bv, mean);
+  launch_k(k_l0_exponents, (unsigned)n, kCol, 0, st, X, N, ex);
   const int64_t hb2 = nblk / 2, tiles = hb2 * (nblk + 1 - hb2);  // i-blocks 0..nblk/2 - 1 (see k_l0_gram)
   for (int64_t s0 = 0; s0 < N; s0 += panel) {
     const int64_t ns = std::min(panel, N - s0);
     const int nc = (int)((ns + sliced::KC - 1) / sliced::KC);
     note_launches(2);
-    k_l0_slices<<<dim3((unsigned)nc, (unsigned)nblk), 128, 0, st>>>(X, ex, n, N, s0, ns, nc, img);
-    k_l0_gram<<<(unsigned)tiles, sliced::THREADS, sliced::SMEM, st>>>(img, ex, n, nc, s0 > 0 ? 1 : 0, D == 3 ? 1 : 0, Gm, G32, err);
+    launch_k(k_l0_slices, dim3((unsigned)nc, (unsigned)nblk), 128, 0, st, X, ex, n, N, s0, ns, nc, img);
+    launch_k(k_l0_gram, (unsigned)tiles, sliced::THREADS, sliced::SMEM, st, img, ex, n, nc, s0 > 0 ? 1 : 0, D == 3 ? 1 : 0, Gm, G32, err);
   }
-  k_l0_cands<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(Gm, G32, bv, nrm2, n, syy, cL, cz, cq, cw, cc);
+  launch_k(k_l0_cands, (unsigned)((n + 127) / 128), 128, 0, st, Gm, G32, bv, nrm2, n, syy, cL, cz, cq, cw, cc);
   const Cand cands{cL, cz, cq, cw, cc};
-  if (D == 1) k_l0_scan<1><<<nb, 256, 0, st>>>(Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
-  else if (D == 2) k_l0_scan<2><<<nb, 256, 0, st>>>(Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
-  else k_l0_scan<3><<<nb, 256, 0, st>>>(Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
-  k_l0_merge<<<1, 1024, 0, st>>>(part, (int64_t)nb * kTop, floor_bits, best);
-  k_l0_exact<<<kMore, 32, 0, st>>>(best, D, X, bv, nrm2, N, ge);
-  k_l0_refit<<<kMore, kCol, 0, st>>>(best, D, X, yc, mean, ge, bv, nrm2, N, 0.0, rm, cf);
+  if (D == 1) launch_k(k_l0_scan<1>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  else if (D == 2) launch_k(k_l0_scan<2>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  else launch_k(k_l0_scan<3>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  launch_k(k_l0_merge, 1, 1024, 0, st, part, (int64_t)nb * kTop, floor_bits, best);
+  launch_k(k_l0_exact, kMore, 32, 0, st, best, D, X, bv, nrm2, N, ge);
+  launch_k(k_l0_refit, kMore, kCol, 0, st, best, D, X, yc, mean, ge, bv, nrm2, N, 0.0, rm, cf);
   DSE_CUDA(cudaGetLastError());
   // reports: RMSEs, coefficients (intercept without the target's mean), the
   // subsets and the target's mean, one wait

@@ -41,6 +41,7 @@ __device__ __forceinline__ void decode_any(const RungGeom &G, int64_t n_stored, 
 // Columns of the given ids into out[c][N]: block c (any block size),
 // threads over samples, so that the FP64 evaluations of a column overlap.
 __global__ void k_columns(FeatTable F, RungGeom G, int64_t n_stored, const uint64_t *ids, int n, double *out) {
+  pdl_enter();
   const int w = blockIdx.x;
   if (w >= n) return;
   if (ids[w] >= (uint64_t)n_stored + G.slots) {  // no such candidate (a failed step of a chained loop)
@@ -60,6 +61,7 @@ constexpr int kMaxP = 4;  // fixed columns + candidate
 __global__ void k_refit(FeatTable F, RungGeom G, int64_t n_stored, const double *y, const double *fixed_cols, int nf,
                         const uint64_t *fixed_ids, const uint64_t *cand, int64_t n_cand, double *rmse_out,
                         double *beta_out) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w >= n_cand) return;
@@ -230,6 +232,7 @@ constexpr int kPrep = kWide;  // threads of the (one-block) prep
 template <int NF>
 __global__ void __launch_bounds__(kPrep) k_refit_prep(const double *y, const double *fixed_cols, int64_t N,
                                                       double *fcc, double *ycc, double *rc, double *pre) {
+  pdl_enter();
   constexpr int nf = NF;
   __shared__ double sm[(kPrep / 32) * (kMaxP * kMaxP + 3 * kMaxP)];
   __shared__ double s_beta[kMaxP + 1];
@@ -358,6 +361,7 @@ __global__ void __launch_bounds__(kColThreads) k_refit_fill(FeatTable F, RungGeo
                                                             const int64_t *n_dev, const double *rc,
                                                             const double *fcc, const float2 *xdf, const int *xexp,
                                                             double *out_x, unsigned long long *minkey) {
+  pdl_enter();
   __shared__ ColShared sh;
   const int64_t w = blockIdx.x;
   if (w == 0 && threadIdx.x == 0) *minkey = ~0ull;  // the smallest RSS + err of this fit (below)
@@ -396,6 +400,7 @@ __global__ void __launch_bounds__(kColThreads) k_refit_fill(FeatTable F, RungGeo
 template <int NF>
 __global__ void k_refit_split(const double *rc, const double *fcc, const double *pre, int64_t N, float2 *xdf,
                               int *xexp) {
+  pdl_enter();
   const int64_t total = (int64_t)(1 + NF) * N;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
     const int m = (int)(i / N);
@@ -434,6 +439,7 @@ __global__ void k_refit_solve(const double *out_x, const uint64_t *cand, int64_t
                               const uint64_t *fixed_ids, const double *pre, int64_t N, double *rmse_out,
                               double *beta_out, uint8_t *explicit_flag, double *err_out,
                               unsigned long long *minkey) {
+  pdl_enter();
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= n_cand || (n_dev && w >= *n_dev)) return;
   constexpr int nf = NF;
@@ -532,6 +538,7 @@ __global__ void __launch_bounds__(kWide) k_refit_wide(FeatTable F, RungGeom G, i
                                                       const int64_t *n_dev, double *rmse_out, double *beta_out,
                                                       const uint8_t *only, double *err_out,
                                                       unsigned long long *minkey, bool near) {
+  pdl_enter();
   constexpr int nf = NF;
   __shared__ double sm[(kWide / 32) * 20];
   __shared__ double s_bc[kMaxP + 2];
@@ -716,9 +723,9 @@ static RefitBufs carve(void *scratch, int64_t N, int64_t cap) {
 
 template <int NF>
 static void prep_nf(const dse_space *S, const double *y, const RefitBufs &b, cudaStream_t st) {
-  k_refit_prep<NF><<<1, kPrep, 0, st>>>(y, b.fc, S->N, b.fcc, b.ycc, b.rc, b.pre);
+  launch_k(k_refit_prep<NF>, 1, kPrep, 0, st, y, b.fc, S->N, b.fcc, b.ycc, b.rc, b.pre);
   const int64_t total = (int64_t)(1 + NF) * S->N;
-  k_refit_split<NF><<<(unsigned)std::min<int64_t>(256, (total + 255) / 256), 256, 0, st>>>(b.rc, b.fcc, b.pre, S->N,
+  launch_k(k_refit_split<NF>, (unsigned)std::min<int64_t>(256, (total + 255) / 256), 256, 0, st, b.rc, b.fcc, b.pre, S->N,
                                                                                          b.xdf, b.xexp);
 }
 
@@ -728,16 +735,15 @@ template <int NF>
 static void fit_nf(const FeatTable &F, const dse_space *S, const uint64_t *fid, const uint64_t *cand, int64_t cap,
                    const int64_t *n_dev, const RefitBufs &b, cudaStream_t st) {
   const int64_t N = S->N;
-  k_refit_fill<NF><<<(unsigned)cap, kColThreads, 0, st>>>(F, S->geom, S->n, cand, cap, n_dev, b.rc, b.fcc, b.xdf,
+  launch_k(k_refit_fill<NF>, (unsigned)cap, kColThreads, 0, st, F, S->geom, S->n, cand, cap, n_dev, b.rc, b.fcc, b.xdf,
                                                           b.xexp, b.outx, b.minkey);
-  k_refit_solve<NF><<<(unsigned)((cap + 127) / 128), 128, 0, st>>>(b.outx, cand, cap, n_dev, fid, b.pre, N, b.rm,
+  launch_k(k_refit_solve<NF>, (unsigned)((cap + 127) / 128), 128, 0, st, b.outx, cand, cap, n_dev, fid, b.pre, N, b.rm,
                                                                     b.beta, b.flag, b.err, b.minkey);
   auto wide = [&](const uint8_t *only, bool near) {
     if (N <= kRefitCacheMax)
-      k_refit_wide<true, NF><<<(unsigned)cap, kWide, (size_t)N * sizeof(double), st>>>(
-          F, S->geom, S->n, b.fcc, b.ycc, b.pre, fid, cand, cap, n_dev, b.rm, b.beta, only, b.err, b.minkey, near);
+      launch_k(k_refit_wide<true, NF>, (unsigned)cap, kWide, (size_t)N * sizeof(double), st, F, S->geom, S->n, b.fcc, b.ycc, b.pre, fid, cand, cap, n_dev, b.rm, b.beta, only, b.err, b.minkey, near);
     else
-      k_refit_wide<false, NF><<<(unsigned)cap, kWide, 0, st>>>(F, S->geom, S->n, b.fcc, b.ycc, b.pre, fid, cand, cap,
+      launch_k(k_refit_wide<false, NF>, (unsigned)cap, kWide, 0, st, F, S->geom, S->n, b.fcc, b.ycc, b.pre, fid, cand, cap,
                                                                 n_dev, b.rm, b.beta, only, b.err, b.minkey, near);
   };
   // in FP64: the fits the sums cannot resolve (near-perfect ones) and every
@@ -752,7 +758,7 @@ void refit_chain_prep(dse_space *S, const double *y, const uint64_t *fid, int nf
   const RefitBufs b = carve(scratch, S->N, cap);
   const FeatTable F = table_of(S);
   note_launches(2 + (nf ? 1 : 0));
-  if (nf) k_columns<<<(unsigned)nf, 256, 0, st>>>(F, S->geom, S->n, fid, nf, b.fc);
+  if (nf) launch_k(k_columns, (unsigned)nf, 256, 0, st, F, S->geom, S->n, fid, nf, b.fc);
   switch (nf) {
     case 0: prep_nf<0>(S, y, b, st); break;
     case 1: prep_nf<1>(S, y, b, st); break;
@@ -793,8 +799,8 @@ void refit_chain_fit(dse_space *S, const double *y, const uint64_t *fid, int nf,
     case 2: fit_nf<2>(F, S, fid, cand, cap, n_dev, b, st); break;
     default: fit_nf<3>(F, S, fid, cand, cap, n_dev, b, st); break;
   }
-  k_argmin<<<1, 1024, 0, st>>>(b.rm, cand, cap, b.best, b.beta, report, n_dev, chosen);
-  k_residual<<<64, 256, 0, st>>>(F, S->geom, S->n, y, b.fc, nf, cand, b.best, b.beta, res);
+  launch_k(k_argmin, 1, 1024, 0, st, b.rm, cand, cap, b.best, b.beta, report, n_dev, chosen);
+  launch_k(k_residual, 64, 256, 0, st, F, S->geom, S->n, y, b.fc, nf, cand, b.best, b.beta, res);
 }
 
 // Index of the smallest RMSE (ties: lower id); one block.  report (when not
@@ -804,6 +810,7 @@ void refit_chain_fit(dse_space *S, const double *y, const uint64_t *fid, int nf,
 // null) gets the winner's id (2^64-1 if none), for fits chained on the device.
 __global__ void k_argmin(const double *rmse, const uint64_t *cand, int64_t n, int64_t *best, const double *beta,
                          double *report, const int64_t *n_dev, uint64_t *chosen) {
+  pdl_enter();
   if (n_dev && *n_dev < n) n = *n_dev;
   // comparisons on order-preserving integer keys of the RMSEs (the integer
   // pipe instead of the slow FP64 one); a NaN ranks with +inf
@@ -859,6 +866,7 @@ __global__ void k_argmin(const double *rmse, const uint64_t *cand, int64_t n, in
 // Residual y - fit of the chosen candidate.
 __global__ void k_residual(FeatTable F, RungGeom G, int64_t n_stored, const double *y, const double *fixed_cols,
                            int nf, const uint64_t *cand, const int64_t *best, const double *beta_all, double *res) {
+  pdl_enter();
   const int64_t bi = *best;
   if (bi < 0) return;
   const double *beta = beta_all + bi * (kMaxP + 1);

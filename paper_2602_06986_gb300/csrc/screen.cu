@@ -96,6 +96,7 @@ __device__ void target_prep(const double *y, int64_t N, int32_t ldy, double *y64
 // One block per target.
 __global__ void k_targets(const double *Y, int64_t ldY, int T, int64_t N, int32_t ldy, double *y64, float *y32,
                           float2 *ydf, float *ysum32, int *err) {
+  pdl_enter();
   const int t = blockIdx.x;
   if (t >= T) return;
   target_prep(Y + (int64_t)t * ldY, N, ldy, y64 + (int64_t)t * ldy, y32 + (int64_t)t * ldy,
@@ -106,6 +107,7 @@ __global__ void k_targets(const double *Y, int64_t ldY, int T, int64_t N, int32_
 // problem's own sample count, into row p.
 __global__ void k_targets_batched(const double *Y, const int64_t *yoff, const ScreenArgs *args, int n,
                                   int32_t ldy, double *y64, float *y32, float *ysum32, int *err) {
+  pdl_enter();
   const int p = blockIdx.x;
   if (p >= n) return;
   target_prep(Y + yoff[p], args[p].N, ldy, y64 + (int64_t)p * ldy, y32 + (int64_t)p * ldy, nullptr, ysum32 + p, err);
@@ -376,6 +378,7 @@ __device__ __forceinline__ void load_ysum(const ScreenArgs &A, R (&ysum)[NT]) {
 template <typename R, int NT>
 __global__ void __launch_bounds__(256) k_feature(const ScreenArgs A, uint64_t id0, uint64_t id1, uint64_t p0,
                                                  uint64_t p1, float gamma_lane) {
+  pdl_enter();
   const uint64_t nid = id1 - id0, ncand = nid + (p1 - p0);
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
   R ysum[NT];
@@ -412,6 +415,7 @@ __device__ __forceinline__ void cp_async4(void *dst, const void *src, bool valid
 template <int CW>
 __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64_t id0, uint64_t id1, uint64_t p0,
                                                       uint64_t p1, float gamma_lane) {
+  pdl_enter();
   constexpr int NT = 16, TH = kF16Half, KS = kF16Chunk, WARPS = 8, NC = WARPS * CW;
   extern __shared__ __align__(16) float f16sm[];
   float(*ys)[KS][TH] = reinterpret_cast<float(*)[KS][TH]>(f16sm);                  // [2][KS][TH]
@@ -632,6 +636,7 @@ __device__ __forceinline__ bool next_job(unsigned int *counter, int n_jobs, int 
 template <typename R>
 __global__ void __launch_bounds__(256) k_feature_batched(const ScreenArgs *args, const Job *jobs, int n_jobs,
                                                          unsigned int *counter) {
+  pdl_enter();
   int j;
   while (next_job(counter, n_jobs, &j)) {
     const Job jb = jobs[j];
@@ -806,6 +811,7 @@ struct PairRing {
 template <typename R, int KIND, int NT, int MI, int MJ, bool BATCH>
 __global__ void __launch_bounds__(256, (sizeof(R) == 4 && NT == 1) ? 2 : 1)
     k_pair(const ScreenArgs A0, const ScreenArgs *batch, int block_len0) {
+  pdl_enter();
   using C = PairCfg<R, KIND, NT, MI, MJ>;
   using V2 = typename Vec2<R>::T;
   constexpr int NS = C::NS, WARPS = 8;
@@ -1208,6 +1214,7 @@ struct PairSums {
 template <int KIND, int NT, int MI, bool BATCH>
 __global__ void __launch_bounds__(PackedPairCfg<NT, MI>::THREADS, PackedPairCfg<NT, MI>::MIN_CTAS)
     k_pair_packed(const ScreenArgs A0, const ScreenArgs *batch, int block_len0) {
+  pdl_enter();
   using C = PackedPairCfg<NT, MI>;
   constexpr int MJ = 2;
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -1399,6 +1406,7 @@ constexpr int k64Chunk = 32;
 
 template <int KIND, int T>
 __global__ void __launch_bounds__(T *T) k_pair64(const ScreenArgs A) {
+  pdl_enter();
   constexpr int ROWS = 2 * T, STR = ROWS + 1;  // sample-major, odd stride: neither loads nor stores conflict
   __shared__ double xs[k64Chunk * STR], zs[k64Chunk * STR], ys[k64Chunk];
   const int tid = threadIdx.x, ti = tid / T, tj = tid % T;
@@ -1571,6 +1579,7 @@ __device__ __forceinline__ void pairlist_one(const ScreenArgs &A, int64_t ia, in
 template <typename R, int NT>
 __global__ void __launch_bounds__(256) k_pairlist(const ScreenArgs A, const int2 *pairs, int64_t n_pairs,
                                                   float gamma_lane) {
+  pdl_enter();
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
   R ysum[NT];
   load_ysum<R, NT>(A, ysum);
@@ -1588,6 +1597,7 @@ __global__ void __launch_bounds__(256) k_pairlist(const ScreenArgs A, const int2
 template <typename R>
 __global__ void __launch_bounds__(256) k_pairlist_batched(const ScreenArgs *args, const int2 *pairs,
                                                           const Job *jobs, int n_jobs, unsigned int *counter) {
+  pdl_enter();
   int j;
   while (next_job(counter, n_jobs, &j)) {
     const Job jb = jobs[j];
@@ -1734,6 +1744,7 @@ __device__ __forceinline__ void esc_pass1(const double *xa, const double *xb, co
 
 // batch != nullptr: entries of a batched screen, each with its problem.
 __global__ void __launch_bounds__(kEsc) k_escalate(const ScreenArgs A0, const ScreenArgs *batch) {
+  pdl_enter();
   __shared__ double sm[(kEsc / 32) * 16];
   const unsigned n = min(*A0.esc_count, (unsigned)A0.esc_cap);
   for (unsigned w = blockIdx.x; w < n; w += gridDim.x) {
@@ -1819,6 +1830,7 @@ constexpr int64_t kEscStashMax = 40960;  // samples kept in shared memory (160 K
 constexpr int kEscS = 512;                // threads per candidate (FP64 latency wants many warps)
 
 __global__ void __launch_bounds__(kEscS, 2) k_escalate_stash(const ScreenArgs A) {
+  pdl_enter();
   extern __shared__ float wsm[];
   __shared__ double sm[(kEscS / 32) * 16];
   const unsigned n = min(*A.esc_count, (unsigned)A.esc_cap);
@@ -1933,6 +1945,7 @@ __global__ void __launch_bounds__(kEscS, 2) k_escalate_stash(const ScreenArgs A)
 // x * (1/x), other operators, operands outside the FP32-safe range) go to
 // the undecided list that the FP64 kernels then take.
 __global__ void __launch_bounds__(256, 2) k_escalate32(const ScreenArgs A) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const unsigned n = min(*A.esc_count, (unsigned)A.esc_cap);
   const unsigned warps = (gridDim.x * blockDim.x) >> 5;
@@ -2000,6 +2013,7 @@ __global__ void __launch_bounds__(256, 2) k_escalate32(const ScreenArgs A) {
 // follows from the shifted sums, sum (v - vbar) y = sum (v - c) y -
 // (vbar - c) sum y, with sum y accumulated alongside.
 __global__ void __launch_bounds__(kEsc) k_escalate1(const ScreenArgs A0, const ScreenArgs *batch) {
+  pdl_enter();
   __shared__ double sm[(kEsc / 32) * 6];
   const unsigned n = min(*A0.esc_count, (unsigned)A0.esc_cap);
   for (unsigned w = blockIdx.x; w < n; w += gridDim.x) {
@@ -2048,6 +2062,7 @@ __global__ void __launch_bounds__(kEsc) k_escalate1(const ScreenArgs A0, const S
 // entry of the range was written by the kernel that decided it; an entry
 // still at -1 afterwards would be a candidate no kernel looked at.
 __global__ void k_why_fixup(const ScreenArgs A) {
+  pdl_enter();
   const uint64_t n = A.id_end - A.id_begin;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     if (A.why[i] != -1) continue;
@@ -2069,7 +2084,7 @@ void launch_why_fixup(const ScreenArgs &A, int sms, cudaStream_t st) {
   uint64_t blocks = (n + 255) / 256;
   if (blocks > (uint64_t)sms * 8) blocks = (uint64_t)sms * 8;
   note_launches(1);
-  k_why_fixup<<<(unsigned)blocks, 256, 0, st>>>(A);
+  launch_k(k_why_fixup, (unsigned)blocks, 256, 0, st, A);
 }
 
 // ------------------------------------------------------------ launchers
@@ -2096,10 +2111,10 @@ void launch_feature_t(const ScreenArgs &A, uint64_t id0, uint64_t id1, uint64_t 
       cudaFuncSetAttribute(k_feature16<kF16CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF16Smem);
       attr[dev & 63] = true;
     }
-    k_feature16<kF16CW><<<(unsigned)tiles, 256, kF16Smem, st>>>(B, id0, id1, p0, p1, gamma);
+    launch_k(k_feature16<kF16CW>, (unsigned)tiles, 256, kF16Smem, st, B, id0, id1, p0, p1, gamma);
     return;
   }
-  k_feature<R, NT><<<(unsigned)blocks, 256, 0, st>>>(B, id0, id1, p0, p1, gamma);
+  launch_k(k_feature<R, NT>, (unsigned)blocks, 256, 0, st, B, id0, id1, p0, p1, gamma);
 }
 
 template <typename R, int KIND, int NT, int MI, int MJ, bool BATCH = false>
@@ -2125,7 +2140,7 @@ dse_status launch_pair_t(const ScreenArgs &A, int block_len, int sms, cudaStream
   note_launches(1);
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
-  k_pair<R, KIND, NT, MI, MJ, BATCH><<<grid, 256, C::SMEM, st>>>(B, batch, block_len);
+  launch_k(k_pair<R, KIND, NT, MI, MJ, BATCH>, grid, 256, C::SMEM, st, B, batch, block_len);
   return DSE_OK;
 }
 
@@ -2146,7 +2161,7 @@ dse_status launch_pair_packed(const ScreenArgs &A, int block_len, cudaStream_t s
   note_launches(1);
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
-  k_pair_packed<KIND, NT, MI, BATCH><<<A.n_tiles, C::THREADS, C::SMEM, st>>>(B, batch, block_len);
+  launch_k(k_pair_packed<KIND, NT, MI, BATCH>, A.n_tiles, C::THREADS, C::SMEM, st, B, batch, block_len);
   return DSE_OK;
 }
 
@@ -2183,8 +2198,8 @@ static dse_status launch_pair64(const ScreenArgs &A, int tile, cudaStream_t st) 
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
   note_launches(1);
-  if (tile == 16) k_pair64<KIND, 16><<<A.n_tiles, 256, 0, st>>>(B);
-  else k_pair64<KIND, 8><<<A.n_tiles, 64, 0, st>>>(B);
+  if (tile == 16) launch_k(k_pair64<KIND, 16>, A.n_tiles, 256, 0, st, B);
+  else launch_k(k_pair64<KIND, 8>, A.n_tiles, 64, 0, st, B);
   return DSE_OK;
 }
 
@@ -2218,11 +2233,11 @@ void launch_pairlist(int prec64, int nt, const ScreenArgs &A, const int2 *pairs,
   ScreenArgs B = A;
   B.group = 2;
   if (prec64) {
-    if (nt == 1) k_pairlist<double, 1><<<(unsigned)blocks, 256, 0, st>>>(B, pairs, n_pairs, gamma);
-    else k_pairlist<double, 16><<<(unsigned)blocks, 256, 0, st>>>(B, pairs, n_pairs, gamma);
+    if (nt == 1) launch_k(k_pairlist<double, 1>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
+    else launch_k(k_pairlist<double, 16>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
   } else {
-    if (nt == 1) k_pairlist<float, 1><<<(unsigned)blocks, 256, 0, st>>>(B, pairs, n_pairs, gamma);
-    else k_pairlist<float, 16><<<(unsigned)blocks, 256, 0, st>>>(B, pairs, n_pairs, gamma);
+    if (nt == 1) launch_k(k_pairlist<float, 1>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
+    else launch_k(k_pairlist<float, 16>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
   }
 }
 
@@ -2232,7 +2247,7 @@ void launch_targets_batched(const double *Y, const int64_t *yoff, const ScreenAr
                             double *y64, float *y32, float *ysum32, int *err, cudaStream_t st) {
   if (n <= 0) return;
   note_launches(1);
-  k_targets_batched<<<n, 256, 0, st>>>(Y, yoff, args, n, ldy, y64, y32, ysum32, err);
+  launch_k(k_targets_batched, n, 256, 0, st, Y, yoff, args, n, ldy, y64, y32, ysum32, err);
 }
 
 void launch_feature_batched(int prec64, const ScreenArgs *args, const Job *jobs, int n_jobs, unsigned int *counter,
@@ -2240,8 +2255,8 @@ void launch_feature_batched(int prec64, const ScreenArgs *args, const Job *jobs,
   if (n_jobs <= 0) return;
   const int blocks = std::min(sms * 8, (n_jobs + 7) / 8);
   note_launches(1);
-  if (prec64) k_feature_batched<double><<<blocks, 256, 0, st>>>(args, jobs, n_jobs, counter);
-  else k_feature_batched<float><<<blocks, 256, 0, st>>>(args, jobs, n_jobs, counter);
+  if (prec64) launch_k(k_feature_batched<double>, blocks, 256, 0, st, args, jobs, n_jobs, counter);
+  else launch_k(k_feature_batched<float>, blocks, 256, 0, st, args, jobs, n_jobs, counter);
 }
 
 dse_status launch_pair_batched(int prec64, int kind, const ScreenArgs &A0, const ScreenArgs *args, int sms,
@@ -2258,8 +2273,8 @@ void launch_pairlist_batched(int prec64, const ScreenArgs *args, const int2 *pai
   if (n_jobs <= 0) return;
   const int blocks = std::min(sms * 8, (n_jobs + 7) / 8);
   note_launches(1);
-  if (prec64) k_pairlist_batched<double><<<blocks, 256, 0, st>>>(args, pairs, jobs, n_jobs, counter);
-  else k_pairlist_batched<float><<<blocks, 256, 0, st>>>(args, pairs, jobs, n_jobs, counter);
+  if (prec64) launch_k(k_pairlist_batched<double>, blocks, 256, 0, st, args, pairs, jobs, n_jobs, counter);
+  else launch_k(k_pairlist_batched<float>, blocks, 256, 0, st, args, pairs, jobs, n_jobs, counter);
 }
 
 void launch_escalate(const ScreenArgs &A0, int sms, cudaStream_t st, const ScreenArgs *batch) {
@@ -2271,7 +2286,7 @@ void launch_escalate(const ScreenArgs &A0, int sms, cudaStream_t st, const Scree
     // candidates costs less than the stage's extra launches)
     if (cudaMemsetAsync(A.esc2_count, 0, sizeof(unsigned), st) == cudaSuccess) {
       note_launches(1);
-      k_escalate32<<<sms * 4, 256, 0, st>>>(A0);
+      launch_k(k_escalate32, sms * 4, 256, 0, st, A0);
       A.esc_id = A.esc2_id;
       A.esc_count = A.esc2_count;
     } else {
@@ -2280,7 +2295,7 @@ void launch_escalate(const ScreenArgs &A0, int sms, cudaStream_t st, const Scree
   }
   note_launches(1);
   if (batch || A.T == 1) {
-    k_escalate1<<<sms * 8, kEsc, 0, st>>>(A, batch);
+    launch_k(k_escalate1, sms * 8, kEsc, 0, st, A, batch);
   } else if (A.N >= 8192 && A.N <= kEscStashMax) {
     // (below 8192 samples the 128-thread blocks of k_escalate keep more
     // candidates in flight and win)
@@ -2292,16 +2307,16 @@ void launch_escalate(const ScreenArgs &A0, int sms, cudaStream_t st, const Scree
                            (int)(kEscStashMax * sizeof(float)));
       attr[dev & 63] = true;
     }
-    k_escalate_stash<<<sms * 2, kEscS, (size_t)A.N * sizeof(float), st>>>(A);
+    launch_k(k_escalate_stash, sms * 2, kEscS, (size_t)A.N * sizeof(float), st, A);
   } else {
-    k_escalate<<<sms * 8, kEsc, 0, st>>>(A, batch);
+    launch_k(k_escalate, sms * 8, kEsc, 0, st, A, batch);
   }
 }
 
 void launch_targets(const double *Y, int64_t ldY, int T, int64_t N, int32_t ldy, double *y64, float *y32,
                     float2 *ydf, float *ysum32, int *err, cudaStream_t st) {
   note_launches(1);
-  k_targets<<<T, 256, 0, st>>>(Y, ldY, T, N, ldy, y64, y32, ydf, ysum32, err);
+  launch_k(k_targets, T, 256, 0, st, Y, ldY, T, N, ldy, y64, y32, ydf, ysum32, err);
 }
 
 }  // namespace dse

@@ -128,6 +128,7 @@ struct GmtTgt {
 // Space part, one block per feature slot f of the a-blocks (slots past n
 // write zero rows): the a-image rows p, p^2 of x and the feature's sums.
 __global__ void __launch_bounds__(128) k_gmt_space(FeatTable F, int nchunks, unsigned char *aimg, GramFeat *gf) {
+  pdl_enter();
   __shared__ double sm[4 * 10];
   const int64_t f = blockIdx.x;
   const bool real = f < F.n;
@@ -206,6 +207,7 @@ size_t gmt_part_count(int64_t n, int64_t N) {
 // zero rows after the last b-feature's.
 __global__ void __launch_bounds__(256) k_gmt_brows(FeatTable F, int nchunks, const float *y32, int64_t ldy, int T,
                                                    const GramFeat *gf, unsigned char *bimg, GmtPart *part) {
+  pdl_enter();
   using namespace gmt;
   constexpr int KC = tc::KC;
   // double-buffered per-chunk values: [g][family][sample], [target][sample]
@@ -333,6 +335,7 @@ __global__ void __launch_bounds__(256) k_gmt_brows(FeatTable F, int nchunks, con
 // merged in FP32 (compensated), the sums of squares added in FP64.
 __global__ void __launch_bounds__(64) k_gmt_tsum(int64_t n, int ncb, const GmtPart *part, int64_t groups,
                                                  GmtTgt *gt) {
+  pdl_enter();
   using namespace gmt;
   const int64_t f = blockIdx.x;
   const int x = threadIdx.x;  // family x NTP + target
@@ -797,6 +800,7 @@ __device__ __forceinline__ void gmt_epilogue(const ScreenArgs &A, const GmtArgs 
 // the empty barriers of both CTAs).  CL = 1: one CTA per tile.
 template <int CL>
 __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A, const GmtArgs GA) {
+  pdl_enter();
   using namespace gmt;
   using namespace tc;
   static_assert(CL == 1 || CL == 2, "clusters of one or two CTAs");
@@ -977,7 +981,7 @@ void gmt_build_space(const FeatTable &F, void *buf, cudaStream_t st) {
   unsigned char *aimg = static_cast<unsigned char *>(buf);
   GramFeat *gf = reinterpret_cast<GramFeat *>(aimg + (size_t)gmt_na(n) * nchunks * gmt::A_IMG);
   note_launches(1);
-  k_gmt_space<<<(unsigned)(gmt_na(n) * gmt::FA), 128, 0, st>>>(F, nchunks, aimg, gf);
+  launch_k(k_gmt_space, (unsigned)(gmt_na(n) * gmt::FA), 128, 0, st, F, nchunks, aimg, gf);
 }
 
 // One screen's b-images and target sums into `scr` (gmt_screen_bytes):
@@ -993,9 +997,9 @@ void launch_gmt_brows(const ScreenArgs &A, const void *space_buf, void *scr, cud
   GmtPart *part = reinterpret_cast<GmtPart *>(reinterpret_cast<unsigned char *>(gt) +
                                               ((size_t)n * sizeof(GmtTgt) + 255) / 256 * 256);
   note_launches(2);
-  k_gmt_brows<<<dim3((unsigned)gmt_nb(n), (unsigned)ncb), 256, 0, st>>>(A.F, nchunks, A.y32 + (int64_t)A.t0 * A.ldy,
+  launch_k(k_gmt_brows, dim3((unsigned)gmt_nb(n), (unsigned)ncb), 256, 0, st, A.F, nchunks, A.y32 + (int64_t)A.t0 * A.ldy,
                                                                       A.ldy, A.T, gf, bimg, part);
-  k_gmt_tsum<<<(unsigned)n, 64, 0, st>>>(n, ncb, part, (int64_t)nchunks * (tc::KC / 8), gt);
+  launch_k(k_gmt_tsum, (unsigned)n, 64, 0, st, n, ncb, part, (int64_t)nchunks * (tc::KC / 8), gt);
 }
 
 // The tiles (a-block, b-block) holding an ordered pair (i, j), i != j, of a
@@ -1121,7 +1125,7 @@ dse_status launch_pair_gmt(const ScreenArgs &A, const void *space_buf, void *scr
     return DSE_OK;
   }
   const int grid = sms < n_tiles ? sms : n_tiles;
-  k_pair_gmt<1><<<grid, gmt::THREADS, gmt::smem_total(), st>>>(B, GA);
+  launch_k(k_pair_gmt<1>, grid, gmt::THREADS, gmt::smem_total(), st, B, GA);
   return DSE_OK;
 }
 

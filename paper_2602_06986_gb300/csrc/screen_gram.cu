@@ -120,6 +120,7 @@ static_assert(smem_total() <= 227 * 1024, "shared memory of one CTA");
 // and of 1/x) and the sums of GramFeat.  Images are zero-initialised by the
 // caller (unused rows, samples past N).
 __global__ void __launch_bounds__(128) k_gram_space(FeatTable F, int nchunks, unsigned char *bimg, GramFeat *gf) {
+  pdl_enter();
   __shared__ double sm[4 * 10];
   const int64_t f = blockIdx.x;
   if (f >= F.n) return;
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(128) k_gram_space(FeatTable F, int nchunks, un
 // p y of x and of 1/x, y the FP32 target) and the target sums.
 __global__ void __launch_bounds__(128) k_gram_arows(FeatTable F, int nchunks, const float *y32, const GramFeat *gf,
                                                     unsigned char *aimg, GramTgt *gt) {
+  pdl_enter();
   __shared__ double sm[4 * 4];
   const int64_t f = blockIdx.x;
   if (f >= F.n) return;
@@ -232,6 +234,7 @@ struct GramArgs {
 };
 
 __global__ void __launch_bounds__(gram::THREADS, 1) k_pair_gram(const ScreenArgs A, const GramArgs GA) {
+  pdl_enter();
   using namespace gram;
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -553,7 +556,7 @@ void gram_build_space(const FeatTable &F, void *buf, cudaStream_t st) {
   GramFeat *gf = reinterpret_cast<GramFeat *>(bimg + (size_t)nb * nchunks * gram::B_IMG);
   cudaMemsetAsync(bimg, 0, (size_t)nb * nchunks * gram::B_IMG, st);
   note_launches(1);
-  k_gram_space<<<(unsigned)n, 128, 0, st>>>(F, nchunks, bimg, gf);
+  launch_k(k_gram_space, (unsigned)n, 128, 0, st, F, nchunks, bimg, gf);
 }
 
 // The tiles (a-block, b-block) holding a pair of the binary block of rung k
@@ -602,7 +605,7 @@ void launch_gram_arows(const ScreenArgs &A, const void *space_buf, void *scr, cu
   // (every row the epilogue reads is written for every chunk; the unused
   // rows only feed TMEM lanes that are never read)
   note_launches(1);
-  k_gram_arows<<<(unsigned)n, 128, 0, st>>>(A.F, nchunks, A.y32 + (int64_t)A.t0 * A.ldy, gf, aimg, gt);
+  launch_k(k_gram_arows, (unsigned)n, 128, 0, st, A.F, nchunks, A.y32 + (int64_t)A.t0 * A.ldy, gf, aimg, gt);
 }
 
 // One screen's product/quotient slots: the kernel over `tiles` (device,
@@ -629,7 +632,7 @@ dse_status launch_pair_gram(const ScreenArgs &A, const void *space_buf, void *sc
   ScreenArgs B = A;
   B.group = 1;
   const int grid = sms < n_tiles ? sms : n_tiles;
-  k_pair_gram<<<grid, gram::THREADS, gram::smem_total(), st>>>(B, GA);
+  launch_k(k_pair_gram, grid, gram::THREADS, gram::smem_total(), st, B, GA);
   return DSE_OK;
 }
 

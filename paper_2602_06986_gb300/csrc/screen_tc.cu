@@ -173,6 +173,7 @@ __host__ __device__ constexpr size_t run_bytes(int ntp) { return tmem_a(ntp) ? (
 // layout (targets beyond T and samples beyond N are zero).
 __global__ void k_tc_targets(const float *y32, int32_t ldy, int t0, int T, int N, int ntp, int nchunks,
                              unsigned char *out) {
+  pdl_enter();
   const int64_t total = (int64_t)nchunks * ntp * tc::KC;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int c = (int)(e / ((int64_t)ntp * tc::KC));
@@ -445,6 +446,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
                                                              const __grid_constant__ CUtensorMap rows_map,
                                                              const __grid_constant__ CUtensorMap rcp_map,
                                                              float gamma_gen, float gamma_num, int gen_blk) {
+  pdl_enter();
   using namespace tc;
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared &sh = *reinterpret_cast<Shared *>(smem);
@@ -908,13 +910,14 @@ static dse_status launch_tc_t(const ScreenArgs &A, const unsigned char *bsplit, 
   note_launches(1);
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
-  k_pair_tc<KIND, NTP><<<grid, tc::THREADS, smem, st>>>(B, bsplit, map, rmap, gamma_gen, gamma_num, gen_blk);
+  launch_k(k_pair_tc<KIND, NTP>, grid, tc::THREADS, smem, st, B, bsplit, map, rmap, gamma_gen, gamma_num, gen_blk);
   return DSE_OK;
 }
 
 // Reciprocal rows of the stored FP32 rows (the rcp.approx the error model
 // assumes), read by the product/quotient kernel next to the rows.
 __global__ void k_rcp_rows(const float *v32, int64_t count, float *out) {
+  pdl_enter();
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x)
     out[e] = rcp_approx(v32[e]);
 }
@@ -924,13 +927,14 @@ void launch_rcp_rows(const float *v32, int64_t count, float *out, int sms, cudaS
   if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
   if (blocks < 1) return;
   note_launches(1);
-  k_rcp_rows<<<(unsigned)blocks, 256, 0, st>>>(v32, count, out);
+  launch_k(k_rcp_rows, (unsigned)blocks, 256, 0, st, v32, count, out);
 }
 
 // Rows in the order of a row list (the unit-class order of the additive
 // tiles): out[p] = v32[rows[p]], so that a tile's rows are consecutive for
 // the 2-D copies.
 __global__ void k_gather_rows(const float *v32, int64_t ld, const int32_t *rows, int64_t n, float *out) {
+  pdl_enter();
   const int64_t total = n * ld;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x)
     out[e] = v32[(int64_t)rows[e / ld] * ld + e % ld];
@@ -942,7 +946,7 @@ void launch_gather_rows(const float *v32, int64_t ld, const int32_t *rows, int64
   if (blocks > (int64_t)sms * 16) blocks = (int64_t)sms * 16;
   if (blocks < 1) return;
   note_launches(1);
-  k_gather_rows<<<(unsigned)blocks, 256, 0, st>>>(v32, ld, rows, n, out);
+  launch_k(k_gather_rows, (unsigned)blocks, 256, 0, st, v32, ld, rows, n, out);
 }
 
 // Samples of each chunk one generation thread sums (the blocked FP32 sums
@@ -971,7 +975,7 @@ void launch_tc_targets(const float *y32, int32_t ldy, int t0, int T, int N, int 
   int64_t blocks = (total + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   note_launches(1);
-  k_tc_targets<<<(unsigned)blocks, 256, 0, st>>>(y32, ldy, t0, T, N, ntp, nchunks, out);
+  launch_k(k_tc_targets, (unsigned)blocks, 256, 0, st, y32, ldy, t0, T, N, ntp, nchunks, out);
 }
 
 dse_status launch_pair_tc(int kind, int ntp, const ScreenArgs &A, const unsigned char *bsplit, const float *rows,

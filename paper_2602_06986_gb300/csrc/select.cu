@@ -82,6 +82,7 @@ __device__ int suffix_bin(const unsigned *h, unsigned long long k, unsigned long
 
 // 1) per list: entry count, overflow flag, bins and in-bin ranks of L and H.
 __global__ void __launch_bounds__(1024) k_sel_bins(const SelectArgs S) {
+  pdl_enter();
   __shared__ unsigned long long rankL, rankH;
   const int l = blockIdx.x;
   const unsigned cnt = S.B.count[l];
@@ -107,6 +108,7 @@ __global__ void __launch_bounds__(1024) k_sel_bins(const SelectArgs S) {
 
 // 2) entries of the L bin and of the H bin, per list (all blocks, 2-D grid).
 __global__ void k_sel_collect(const SelectArgs S) {
+  pdl_enter();
   const int l = blockIdx.y;
   const SelState st = S.state[l];
   if (st.all_in) return;
@@ -190,6 +192,7 @@ __device__ float kth_largest(const float *v, unsigned n, unsigned r, unsigned *h
 
 // 3) exact L and H from their bins (one block per list).
 __global__ void __launch_bounds__(1024) k_sel_exact(const SelectArgs S) {
+  pdl_enter();
   __shared__ unsigned hist[256];
   const int l = blockIdx.x;
   SelState st = S.state[l];
@@ -210,6 +213,7 @@ __device__ __forceinline__ uint64_t score_key(double s) { return (uint64_t)__dou
 
 // 4) classification into the retained set and the FP64 job list (all blocks).
 __global__ void k_sel_classify(const SelectArgs S) {
+  pdl_enter();
   const int l = blockIdx.y;
   const SelState st = S.state[l];
   const size_t base = (size_t)l * S.B.cap;
@@ -256,6 +260,7 @@ constexpr int kRes = 128;
 // compile-time count keeps the accumulators in registers.
 template <int NT>
 __global__ void __launch_bounds__(kRes) k_rescore(const SelectArgs S, const ScreenArgs A0, const ScreenArgs *batch) {
+  pdl_enter();
   __shared__ double red[kRes / 32][2 + NT];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const unsigned nj = *S.n_jobs;
@@ -327,6 +332,7 @@ __global__ void __launch_bounds__(kRes) k_rescore(const SelectArgs S, const Scre
 // job would spend its time in barriers and reductions.
 template <int NT>
 __global__ void __launch_bounds__(256) k_rescore_warp(const SelectArgs S, const ScreenArgs A) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const unsigned nj = *S.n_jobs;
   const unsigned warps = (gridDim.x * blockDim.x) >> 5;
@@ -396,6 +402,7 @@ __global__ void __launch_bounds__(256) k_rescore_warp(const SelectArgs S, const 
 // bound.  Entries it cannot take (other operators, operands outside the
 // FP32-safe range, a wider bound) join the pair re-score's jobs.
 __global__ void __launch_bounds__(256, 3) k_rescore32(const SelectArgs S, const ScreenArgs A) {
+  pdl_enter();
   const int lane = threadIdx.x & 31;
   const unsigned nj = S.n_jobs[1];
   const unsigned warps = (gridDim.x * blockDim.x) >> 5;
@@ -455,6 +462,7 @@ __global__ void __launch_bounds__(256, 3) k_rescore32(const SelectArgs S, const 
 template <bool ONE>
 __global__ void __launch_bounds__(kColThreads, ONE ? 6 : 1) k_rescore1(const SelectArgs S, const ScreenArgs A0,
                                                           const ScreenArgs *batch) {
+  pdl_enter();
   __shared__ ColShared sh;
   const unsigned nj = *S.n_jobs;
   for (unsigned w = blockIdx.x; w < nj; w += gridDim.x) {
@@ -528,6 +536,7 @@ constexpr int kRankTile = 2048, kRankPer = 8, kRankGroup = 8 * kRankPer;
 // entries' keys in registers and its lanes run over the tile, so that every
 // key read from shared memory serves 8 comparisons.
 __global__ void __launch_bounds__(256) k_rank(const SelectArgs S) {
+  pdl_enter();
   __shared__ uint64_t tk[kRankTile], ti[kRankTile];
   const int l = blockIdx.y;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -575,6 +584,7 @@ __global__ void __launch_bounds__(256) k_rank(const SelectArgs S) {
 // largest returned bound (bounds are non-negative: their bit patterns order
 // like the values).
 __global__ void k_rank_write(const SelectArgs S) {
+  pdl_enter();
   const int l = blockIdx.y;
   const int64_t rn = S.r_count[l];
   const size_t base = (size_t)l * S.B.cap;
@@ -610,27 +620,27 @@ dse_status launch_select(const SelectArgs &S0, const ScreenArgs &A, int sms, cud
   SelectArgs S = S0;
   S.rescore32 = !batch && !S.all64 && S.nx == 0 && !S.r_x && S.job32 && S.job32_list && A.F.v32 && A.y32 &&
                 A.ysum32 && (A.mode != DSE_MODE_AGGREGATED || A.T == 1);
-  k_sel_bins<<<S.n_lists, 1024, 0, st>>>(S);
+  launch_k(k_sel_bins, S.n_lists, 1024, 0, st, S);
   const unsigned bx = (unsigned)std::max(1, std::min(256, (sms * 4 + S.n_lists - 1) / S.n_lists));
   dim3 g(bx, S.n_lists);
-  k_sel_collect<<<g, 256, 0, st>>>(S);
-  k_sel_exact<<<S.n_lists, 1024, 0, st>>>(S);
-  k_sel_classify<<<g, 256, 0, st>>>(S);
+  launch_k(k_sel_collect, g, 256, 0, st, S);
+  launch_k(k_sel_exact, S.n_lists, 1024, 0, st, S);
+  launch_k(k_sel_classify, g, 256, 0, st, S);
   const bool one = batch || A.mode != DSE_MODE_AGGREGATED || A.T == 1;
   if (S.rescore32) {
     note_launches(1);
-    k_rescore32<<<sms * 8, 256, 0, st>>>(S, A);
+    launch_k(k_rescore32, sms * 8, 256, 0, st, S, A);
   }
   if (one && !batch && S.nx == 0)
-    k_rescore1<true><<<sms * 16, kColThreads, 0, st>>>(S, A, batch);
+    launch_k(k_rescore1<true>, sms * 16, kColThreads, 0, st, S, A, batch);
   else if (one)
-    k_rescore1<false><<<sms * 8, kColThreads, 0, st>>>(S, A, batch);
-  else if (A.N <= 4096) k_rescore_warp<16><<<sms * 8, 256, 0, st>>>(S, A);
-  else k_rescore<16><<<sms * 8, kRes, 0, st>>>(S, A, batch);
+    launch_k(k_rescore1<false>, sms * 8, kColThreads, 0, st, S, A, batch);
+  else if (A.N <= 4096) launch_k(k_rescore_warp<16>, sms * 8, 256, 0, st, S, A);
+  else launch_k(k_rescore<16>, sms * 8, kRes, 0, st, S, A, batch);
   const dim3 gr((unsigned)std::max(1, std::min(1024, (sms * 2 + S.n_lists - 1) / S.n_lists)), S.n_lists);
-  k_rank<<<gr, 256, 0, st>>>(S);
+  launch_k(k_rank, gr, 256, 0, st, S);
   const dim3 gw((unsigned)std::max(1, std::min(64, (sms + S.n_lists - 1) / S.n_lists)), S.n_lists);
-  k_rank_write<<<gw, 256, 0, st>>>(S);
+  launch_k(k_rank_write, gw, 256, 0, st, S);
   return DSE_OK;
 }
 

@@ -148,6 +148,7 @@ constexpr int kCompactPer = 16;  // elements per thread
 constexpr int kCompactTile = kCompactThreads * kCompactPer;
 
 __global__ void k_compact_count(const uint8_t *flags, uint64_t n, uint8_t want, unsigned int *block_counts) {
+  pdl_enter();
   __shared__ unsigned int red[kCompactThreads / 32];
   uint64_t base = (uint64_t)blockIdx.x * kCompactTile + (uint64_t)threadIdx.x * kCompactPer;
   unsigned int c = 0;
@@ -168,6 +169,7 @@ __global__ void k_compact_count(const uint8_t *flags, uint64_t n, uint8_t want, 
 // Exclusive scan of block counts by one block (loops over chunks).
 __global__ void k_compact_scan(const unsigned int *block_counts, uint64_t nb, unsigned long long *offsets,
                                unsigned long long *total) {
+  pdl_enter();
   __shared__ unsigned long long part[1024];
   __shared__ unsigned long long carry;
   if (threadIdx.x == 0) carry = 0;
@@ -193,6 +195,7 @@ __global__ void k_compact_scan(const unsigned int *block_counts, uint64_t nb, un
 
 __global__ void k_compact_write(const uint8_t *flags, uint64_t n, uint8_t want,
                                 const unsigned long long *offsets, uint64_t *out) {
+  pdl_enter();
   __shared__ unsigned int sc[kCompactThreads];
   uint64_t base = (uint64_t)blockIdx.x * kCompactTile + (uint64_t)threadIdx.x * kCompactPer;
   unsigned int c = 0;
@@ -231,9 +234,9 @@ dse_status compact_bytes_dev(const uint8_t *flags, uint64_t n, uint8_t want, uin
     return st;
   }
   note_launches(3);
-  k_compact_count<<<(unsigned)nb, kCompactThreads, 0, s>>>(flags, n, want, bc);
-  k_compact_scan<<<1, 1024, 0, s>>>(bc, nb, off, count_dev);
-  k_compact_write<<<(unsigned)nb, kCompactThreads, 0, s>>>(flags, n, want, off, out);
+  launch_k(k_compact_count, (unsigned)nb, kCompactThreads, 0, s, flags, n, want, bc);
+  launch_k(k_compact_scan, 1, 1024, 0, s, bc, nb, off, count_dev);
+  launch_k(k_compact_write, (unsigned)nb, kCompactThreads, 0, s, flags, n, want, off, out);
   dfree(bc);
   dfree(off);
   DSE_CUDA(cudaGetLastError());
@@ -254,9 +257,9 @@ dse_status compact_bytes(const uint8_t *flags, uint64_t n, uint8_t want, uint64_
     return st;
   }
   note_launches(3);
-  k_compact_count<<<(unsigned)nb, kCompactThreads, 0, s>>>(flags, n, want, bc);
-  k_compact_scan<<<1, 1024, 0, s>>>(bc, nb, off, off + nb);
-  k_compact_write<<<(unsigned)nb, kCompactThreads, 0, s>>>(flags, n, want, off, out);
+  launch_k(k_compact_count, (unsigned)nb, kCompactThreads, 0, s, flags, n, want, bc);
+  launch_k(k_compact_scan, 1, 1024, 0, s, bc, nb, off, off + nb);
+  launch_k(k_compact_write, (unsigned)nb, kCompactThreads, 0, s, flags, n, want, off, out);
   unsigned long long tot = 0;
   cudaError_t e = cudaMemcpyAsync(&tot, off + nb, sizeof(tot), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
@@ -268,6 +271,7 @@ dse_status compact_bytes(const uint8_t *flags, uint64_t n, uint8_t want, uint64_
 }
 
 __global__ void k_count_reasons(const uint8_t *flags, uint64_t n, unsigned long long *counts) {
+  pdl_enter();
   __shared__ unsigned int c[6];
   if (threadIdx.x < 6) c[threadIdx.x] = 0;
   __syncthreads();
@@ -284,7 +288,7 @@ void launch_count_reasons(const uint8_t *flags, uint64_t n, unsigned long long *
   uint64_t blocks = (n + 255) / 256;
   if (blocks > 4096) blocks = 4096;
   note_launches(1);
-  k_count_reasons<<<(unsigned)blocks, 256, 0, s>>>(flags, n, counts);
+  launch_k(k_count_reasons, (unsigned)blocks, 256, 0, s, flags, n, counts);
 }
 
 }  // namespace dse

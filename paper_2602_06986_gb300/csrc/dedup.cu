@@ -132,52 +132,68 @@ __global__ void __launch_bounds__(kFlagThreads) k_dedup_flags(const uint64_t *id
   if (threadIdx.x == 0) red[(int64_t)l * kk + i] = (uint8_t)found;
 }
 
-// Warp per list: the first k non-redundant entries in rank order into the
+// Block per list (one warp, a chain of loads every 32 entries, took 44 us for
+// 800): the first k non-redundant entries in rank order into the
 // output lists; undecided[l] = 1 if an entry examined before the k-th kept
 // one is kept while its score lies within W of the list's last score and
 // the list may be incomplete; n_red[l] = redundant entries examined.
-__global__ void k_dedup_compact(const uint64_t *ids, const double *score, const double *eps, const int64_t *n_list,
+constexpr int kCompactThreads = 1024;
+__global__ void __launch_bounds__(kCompactThreads) k_dedup_compact(const uint64_t *ids, const double *score, const double *eps, const int64_t *n_list,
                                 const double *max_eps, int64_t kk, int64_t k, int full, double w_tau,
                                 const uint8_t *red, uint64_t *o_id, double *o_score, double *o_eps, int64_t *o_n,
                                 double *o_max_eps, int *undecided, int64_t *n_red) {
   pdl_enter();
+  __shared__ int s_kept[32], s_und;
+  __shared__ unsigned long long s_nr, s_me;
   const int l = blockIdx.x;
-  const int lane = threadIdx.x;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t n = n_list[l];
   const int64_t base = (int64_t)l * kk;
   const double W = w_tau + 2.0 * max_eps[l];
   const double s_last = n > 0 ? score[base + n - 1] : 0.0;
   const bool may_miss = full && n == kk;
-  int64_t kept = 0, nr = 0;
-  int und = 0;
-  double me = 0.0;
-  for (int64_t c = 0; c < n && kept < k; c += 32) {
-    const int64_t i = c + lane;
+  if (threadIdx.x == 0) {
+    s_und = 0;
+    s_nr = s_me = 0ull;
+  }
+  int64_t kept = 0;
+  for (int64_t c = 0; c < n && kept < k; c += kCompactThreads) {
+    const int64_t i = c + threadIdx.x;
     const bool in = i < n;
     const bool r = in ? red[base + i] != 0 : true;
+    const double sc = in ? score[base + i] : 0.0, ep = in ? eps[base + i] : 0.0;
+    const uint64_t id = in ? ids[base + i] : 0ull;
     const unsigned km = __ballot_sync(0xffffffffu, in && !r);
-    const int before = __popc(km & ((1u << lane) - 1u));
+    __syncthreads();  // (the counts of the chunk before are read)
+    if (lane == 0) s_kept[warp] = __popc(km);
+    __syncthreads();
+    int before = __popc(km & ((1u << lane) - 1u)), all = 0;
+    for (int q = 0; q < kCompactThreads / 32; ++q) {
+      before += q < warp ? s_kept[q] : 0;
+      all += s_kept[q];
+    }
     const bool examined = in && (kept + before < k);
     // a redundant entry is settled by its partner; a kept one needs the
     // whole window in the list
-    if (examined && !r && may_miss && !(score[base + i] - W > s_last)) und = 1;
+    if (examined && !r && may_miss && !(sc - W > s_last)) s_und = 1;
     if (examined && !r) {
       const int64_t pos = kept + before;
-      o_id[(int64_t)l * k + pos] = ids[base + i];
-      o_score[(int64_t)l * k + pos] = score[base + i];
-      o_eps[(int64_t)l * k + pos] = eps[base + i];
-      me = fmax(me, eps[base + i]);
+      o_id[(int64_t)l * k + pos] = id;
+      o_score[(int64_t)l * k + pos] = sc;
+      o_eps[(int64_t)l * k + pos] = ep;
+      // (bounds are non-negative: their bits order like the values)
+      atomicMax(&s_me, (unsigned long long)__double_as_longlong(ep));
     }
-    nr += __popc(__ballot_sync(0xffffffffu, examined && r));
-    kept += __popc(km);
+    const unsigned rm = __ballot_sync(0xffffffffu, examined && r);
+    if (lane == 0 && rm) atomicAdd(&s_nr, (unsigned long long)__popc(rm));
+    kept += all;
   }
-  und = __any_sync(0xffffffffu, und);
-  me = warp_max64(me);
-  if (lane == 0) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
     o_n[l] = kept < k ? kept : k;
-    o_max_eps[l] = me;
-    undecided[l] = und;
-    n_red[l] = nr;
+    o_max_eps[l] = __longlong_as_double((long long)s_me);
+    undecided[l] = s_und;
+    n_red[l] = (int64_t)s_nr;
   }
 }
 
@@ -223,7 +239,7 @@ dse_status dedup_result(dse_result *R, int64_t k, double tau, bool full, bool *u
   int *o_un = reinterpret_cast<int *>(buf + off_un);
   int64_t *o_nr = reinterpret_cast<int64_t *>(buf + off_nr);
   note_launches(1);
-  launch_k(k_dedup_compact, (unsigned)L, 32, 0, st, R->out_id, R->out_score, R->out_eps, R->out_n, R->max_eps, kk, k,
+  launch_k(k_dedup_compact, (unsigned)L, kCompactThreads, 0, st, R->out_id, R->out_score, R->out_eps, R->out_n, R->max_eps, kk, k,
                                               full ? 1 : 0, w_tau, red, o_id, o_sc, o_ep, o_n, o_me, o_un, o_nr);
   dfree(z);
   dfree(red);

@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64
         ract[warp * CW + k] = act[k] ? 1 : 0;
       }
     }
-    for (int half = 0; half < 2; ++half) {
+    for (int half = 0; half < (T > TH ? 2 : 1); ++half) {  // (up to 8 targets: one pass)
       const int th0 = half * TH;
       const bool first = half == 0;
       float S1[CW], S2[CW], o1[CW], o2[CW], Sy[CW][TH], oy[CW][TH];
@@ -1576,6 +1576,98 @@ __device__ __forceinline__ void pairlist_one(const ScreenArgs &A, int64_t ia, in
   refresh_pushed<NT>(A, pushed);
 }
 
+// The same for a short list over many samples: a block of 8 warps per pair.
+// A lane of pairlist_one sums its samples in blocks of 16 (512 samples a
+// warp) and adds the blocks in order; here the warps take the blocks in turn
+// and the first warp adds their sums in that order, so every sum keeps its
+// bits.  (One warp a pair leaves the GPU to the latency of a few warps: 22
+// blocks of pairs over 20000 samples and 16 targets took 703 us, now 193.)
+template <int NT>
+__global__ void __launch_bounds__(256) k_pairlist_split(const ScreenArgs A, const int2 *pairs, float gamma_lane) {
+  pdl_enter();
+  constexpr int NV = 3 * (2 + NT), WARPS = 8, SEG = 512;
+  extern __shared__ float seg_sums[];  // [WARPS][NV][32]
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int2 pr = pairs[blockIdx.x];
+  const int64_t ia = pr.x, ib = pr.y;
+  const int64_t Ns = A.N, ldy = A.ldy;
+  const int T = A.T, t0 = A.t0;
+  const float4 fa_a = A.F.fa[ia], fa_b = A.F.fa[ib];
+  const float mi = fa_a.x, mj = fa_b.x;
+  const float cabs = mi - mj < 0.f ? mj - mi : mi - mj;
+  const float *xa = A.F.v32 + ia * A.F.ld, *xb = A.F.v32 + ib * A.F.ld;
+  float tot[NV];
+#pragma unroll
+  for (int v = 0; v < NV; ++v) tot[v] = 0.f;
+  constexpr int U = NT == 1 ? 8 : NT <= 4 ? 4 : 2;
+  for (int64_t r0 = 0; r0 < Ns; r0 += (int64_t)WARPS * SEG) {
+    float acc[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) acc[v] = 0.f;
+    const int64_t b0 = r0 + (int64_t)warp * SEG, b1 = b0 + SEG < Ns ? b0 + SEG : Ns;
+    for (int64_t s0 = b0 + lane; s0 < b1; s0 += 32 * U) {
+      float av[U], bv[U], yv[U][NT];
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        const int64_t s = s0 + 32 * q;
+        const bool in = s < b1;
+        av[q] = in ? xa[s] : 0.f;
+        bv[q] = in ? xb[s] : 0.f;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) yv[q][t] = in && t < T ? A.y32[(int64_t)(t0 + t) * ldy + s] : 0.f;
+      }
+#pragma unroll
+      for (int q = 0; q < U; ++q) {
+        if (s0 + 32 * q >= b1) break;
+        const float ac = av[q] - mi, bc = bv[q] - mj, d = av[q] - bv[q];
+        const float w3[3] = {ac + bc, ac - bc, (d < 0.f ? -d : d) - cabs};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          acc[k * (2 + NT)] += w3[k];
+          acc[k * (2 + NT) + 1] = fmaf(w3[k], w3[k], acc[k * (2 + NT) + 1]);
+#pragma unroll
+          for (int t = 0; t < NT; ++t) acc[k * (2 + NT) + 2 + t] = fmaf(w3[k], yv[q][t], acc[k * (2 + NT) + 2 + t]);
+        }
+      }
+    }
+    __syncthreads();  // (the sums of the round before are read)
+#pragma unroll
+    for (int v = 0; v < NV; ++v) seg_sums[(warp * NV + v) * 32 + lane] = acc[v];
+    __syncthreads();
+    if (warp == 0)
+      for (int g = 0; g < WARPS && r0 + (int64_t)g * SEG < Ns; ++g)
+#pragma unroll
+        for (int v = 0; v < NV; ++v) tot[v] += seg_sums[(g * NV + v) * 32 + lane];
+  }
+  if (warp != 0) return;
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    float x = tot[v];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    tot[v] = x;
+  }
+  const float u = 5.9604644775390625e-8f;
+  const float N = (float)Ns, invN = (float)A.invN, sqrtN = sqrtf(N);
+  const uint64_t pbase = A.G.um + (tri((uint64_t)ia) + (uint64_t)ib - A.G.tri_o) * (uint64_t)A.G.nb;
+  float ysum[NT];
+  load_ysum<float, NT>(A, ysum);
+  LaneStats ls;
+  ls.zero();
+  unsigned pushed = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int opc = k == 0 ? DSE_OP_ADD : k == 1 ? DSE_OP_SUB : DSE_OP_ABSDIFF;
+    float Sy[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) Sy[t] = tot[k * (2 + NT) + 2 + t];
+    pushed |= binary_candidate<float, NT>(A, ls, lane == 0, true, ia, ib, opc, pbase, fa_a, fa_b, cabs, mi, mj,
+                                          tot[k * (2 + NT)], tot[k * (2 + NT) + 1], Sy, N, invN, sqrtN, gamma_lane, u,
+                                          (float)A.fmin_std_rel64, ysum);
+  }
+  refresh_pushed<NT>(A, pushed);
+  flush_stats(A, ls);
+}
+
 template <typename R, int NT>
 __global__ void __launch_bounds__(256) k_pairlist(const ScreenArgs A, const int2 *pairs, int64_t n_pairs,
                                                   float gamma_lane) {
@@ -2224,6 +2316,20 @@ dse_status launch_pair(int prec64, int kind, int nt, int tile_rows, const Screen
                           : launch_pair_t<float, KIND_ADD, 16, 1, 1>(A, block_len, sms, st);
 }
 
+template <int NT>
+static void launch_pairlist_split(const ScreenArgs &A, const int2 *pairs, int64_t n_pairs, float gamma,
+                                  cudaStream_t st) {
+  const size_t smem = (size_t)8 * 3 * (2 + NT) * 32 * sizeof(float);
+  static bool attr[64] = {false};
+  int dev = 0;
+  cudaGetDevice(&dev);
+  if (!attr[dev & 63]) {
+    cudaFuncSetAttribute(k_pairlist_split<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    attr[dev & 63] = true;
+  }
+  launch_k(k_pairlist_split<NT>, (unsigned)n_pairs, 256, smem, st, A, pairs, gamma);
+}
+
 void launch_pairlist(int prec64, int nt, const ScreenArgs &A, const int2 *pairs, int64_t n_pairs, float gamma,
                      int sms, cudaStream_t st) {
   if (n_pairs <= 0) return;
@@ -2232,6 +2338,15 @@ void launch_pairlist(int prec64, int nt, const ScreenArgs &A, const int2 *pairs,
   note_launches(1);
   ScreenArgs B = A;
   B.group = 2;
+  if (!prec64 && A.N > 512 && n_pairs <= (int64_t)sms * 16) {
+    // (a block a pair is within twice what the SMs hold at once; up to 512
+    // samples there is one block of sums and nothing to share out)
+    if (nt == 1) launch_pairlist_split<1>(B, pairs, n_pairs, gamma, st);
+    else if (A.T <= 4) launch_pairlist_split<4>(B, pairs, n_pairs, gamma, st);
+    else if (A.T <= 8) launch_pairlist_split<8>(B, pairs, n_pairs, gamma, st);
+    else launch_pairlist_split<16>(B, pairs, n_pairs, gamma, st);
+    return;
+  }
   if (prec64) {
     if (nt == 1) launch_k(k_pairlist<double, 1>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
     else launch_k(k_pairlist<double, 16>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);

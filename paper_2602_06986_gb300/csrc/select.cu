@@ -626,17 +626,29 @@ dse_status launch_select(const SelectArgs &S0, const ScreenArgs &A, int sms, cud
   launch_k(k_sel_collect, g, 256, 0, st, S);
   launch_k(k_sel_exact, S.n_lists, 1024, 0, st, S);
   launch_k(k_sel_classify, g, 256, 0, st, S);
+  // blocks for the jobs that lists of k retain (a few more than k each; the
+  // kernels loop): a short list's re-score does not start thousands of blocks
+  const int64_t jobs = (S.k + S.k / 2 + 64) * S.n_lists;
   const bool one = batch || A.mode != DSE_MODE_AGGREGATED || A.T == 1;
   if (S.rescore32) {
     note_launches(1);
-    launch_k(k_rescore32, sms * 8, 256, 0, st, S, A);
+    launch_k(k_rescore32, (unsigned)std::min<int64_t>(sms * 8, jobs / 8 + 1), 256, 0, st, S, A);
   }
   if (one && !batch && S.nx == 0)
-    launch_k(k_rescore1<true>, sms * 16, kColThreads, 0, st, S, A, batch);
+    launch_k(k_rescore1<true>, (unsigned)std::min<int64_t>(sms * 16, jobs), kColThreads, 0, st, S, A, batch);
   else if (one)
     launch_k(k_rescore1<false>, sms * 8, kColThreads, 0, st, S, A, batch);
-  else if (A.N <= 4096) launch_k(k_rescore_warp<16>, sms * 8, 256, 0, st, S, A);
-  else launch_k(k_rescore<16>, sms * 8, kRes, 0, st, S, A, batch);
+  // (aggregated lists: as many sums as there are targets; FP64 instructions
+  // that are predicated off still take their turn)
+  else if (A.N <= 4096) {
+    if (A.T <= 4) launch_k(k_rescore_warp<4>, sms * 8, 256, 0, st, S, A);
+    else if (A.T <= 8) launch_k(k_rescore_warp<8>, sms * 8, 256, 0, st, S, A);
+    else launch_k(k_rescore_warp<16>, sms * 8, 256, 0, st, S, A);
+  } else {
+    if (A.T <= 4) launch_k(k_rescore<4>, sms * 8, kRes, 0, st, S, A, batch);
+    else if (A.T <= 8) launch_k(k_rescore<8>, sms * 8, kRes, 0, st, S, A, batch);
+    else launch_k(k_rescore<16>, sms * 8, kRes, 0, st, S, A, batch);
+  }
   const dim3 gr((unsigned)std::max(1, std::min(1024, (sms * 2 + S.n_lists - 1) / S.n_lists)), S.n_lists);
   launch_k(k_rank, gr, 256, 0, st, S);
   const dim3 gw((unsigned)std::max(1, std::min(64, (sms + S.n_lists - 1) / S.n_lists)), S.n_lists);

@@ -154,14 +154,36 @@ static void tc_tiles(int64_t ia, int64_t ja, int64_t ib, int64_t jb, std::vector
 // group.  A wave of one CTA per SM then covers a compact block of the
 // triangle (e.g. 8 i-blocks x 19 j-blocks) whose rows stay in L2, instead of
 // one i-block against hundreds of j-blocks.
+// (The list comes i-block by i-block, each with rising j-blocks: a group is a
+// merge of its runs.  Sorted instead, the 66 k tiles of a 40 M id block took
+// most of the 5 ms in which the GPU waited for the plan.)
 void group_tiles(std::vector<Tile> &t, int64_t ia, int BI, int G) {
   const int64_t span = (int64_t)BI * G;
-  std::stable_sort(t.begin(), t.end(), [&](const Tile &a, const Tile &b) {
-    const int64_t ga = (a.ibase - ia) / span, gb = (b.ibase - ia) / span;
-    if (ga != gb) return ga < gb;
-    if (a.jbase != b.jbase) return a.jbase < b.jbase;
-    return a.ibase < b.ibase;
-  });
+  std::vector<Tile> out;
+  out.reserve(t.size());
+  std::vector<std::pair<size_t, size_t>> runs;
+  for (size_t pos = 0; pos < t.size();) {
+    const int64_t g = (t[pos].ibase - ia) / span;
+    runs.clear();
+    while (pos < t.size() && (t[pos].ibase - ia) / span == g) {
+      const size_t first = pos;
+      while (pos < t.size() && t[pos].ibase == t[first].ibase) ++pos;
+      runs.push_back({first, pos});
+    }
+    for (;;) {
+      int32_t j = INT32_MAX;
+      bool any = false;
+      for (const auto &r : runs)
+        if (r.first < r.second) {
+          any = true;
+          j = std::min(j, t[r.first].jbase);
+        }
+      if (!any) break;
+      for (auto &r : runs)
+        while (r.first < r.second && t[r.first].jbase == j) out.push_back(t[r.first++]);
+    }
+  }
+  t.swap(out);
 }
 
 // ------------------------------------------------------------- screening
@@ -760,7 +782,8 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
                               : plan.use_tc && !plan.mul_tiles.empty()   ? DSE_PATH_TENSOR
                               : !plan.mul_tiles.empty()                  ? DSE_PATH_CUDA_CORE
                                                                          : 0;
-  Keep *keep = new (std::nothrow) Keep{plan, A, S, tmul, tadd};
+  R->add_total = plan.add_total;
+  Keep *keep = new (std::nothrow) Keep{std::move(plan), A, S, tmul, tadd};  // (the tile lists can be megabytes)
   if (!keep) return fail(DSE_ENOMEM);
   R->keep = keep;
   R->keep_free = [](void *p) { delete reinterpret_cast<Keep *>(p); };
@@ -768,7 +791,6 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
     Keep *k = reinterpret_cast<Keep *>(r->keep);
     return run_screen(r, k->plan, k->tmul, k->tadd, k->A, k->S);
   };
-  R->add_total = plan.add_total;
   R->buf_count = A.B.count;
   *out = R;
   return DSE_OK;
@@ -874,6 +896,18 @@ static dse_status finish(dse_result *R) {
   }
 }
 
+
+// A list's ids, scores and bounds into a caller's device arrays (either may be
+// absent).
+__global__ void k_fetch(const uint64_t *id, const double *score, const double *eps, int64_t n, uint64_t *o_id,
+                        double *o_score, double *o_eps) {
+  pdl_enter();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    if (o_id) o_id[i] = id[i];
+    if (o_score) o_score[i] = score[i];
+    if (o_eps) o_eps[i] = eps[i];
+  }
+}
 
 // ------------------------------------------------- redundancy removal
 
@@ -1380,6 +1414,25 @@ dse_status dse_topk_fetch(dse_result *r, int32_t list, uint64_t *idx, double *sc
   int64_t m = std::min(n, cap);
   if (m == 0) return DSE_OK;
   const size_t off = (size_t)list * r->k;
+  // into this device's memory: one kernel for the three arrays
+  int dev = -1;
+  cudaGetDevice(&dev);
+  auto here = [&](const void *p) {
+    cudaPointerAttributes at;
+    if (!p) return true;
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    return at.type == cudaMemoryTypeDevice && at.device == dev;
+  };
+  if (r->space->device == dev && here(idx) && here(score) && here(err_bound)) {
+    note_launches(1);
+    launch_k(k_fetch, (unsigned)std::min<int64_t>(64, (m + 255) / 256), 256, 0, r->stream, r->out_id + off,
+             r->out_score + off, r->out_eps + off, m, idx, score, err_bound);
+    DSE_CUDA(cudaGetLastError());
+    return DSE_OK;
+  }
   // copies on the result's stream; wait only when one lands in host memory
   bool host = false;
   auto cp = [&](void *dst, const void *src, size_t bytes) {

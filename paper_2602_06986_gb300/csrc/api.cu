@@ -228,9 +228,9 @@ dse_status launch_pair_gram(const ScreenArgs &A, const void *space_buf, void *sc
 
 bool gmt_eligible(int T, int64_t N);
 size_t gmt_space_bytes(int64_t n, int64_t N);
-size_t gmt_screen_bytes(int64_t n, int64_t N);
+size_t gmt_screen_bytes(int64_t n, int64_t N, int T);
 void gmt_build_space(const FeatTable &F, void *buf, cudaStream_t st);
-void gmt_tiles(const dse_space *sp, uint64_t id_begin, uint64_t id_end, std::vector<int2> &out);
+void gmt_tiles(const dse_space *sp, uint64_t id_begin, uint64_t id_end, int T, std::vector<int2> &out);
 void launch_gmt_brows(const ScreenArgs &A, const void *space_buf, void *scr, cudaStream_t st);
 dse_status launch_pair_gmt(const ScreenArgs &A, const void *space_buf, void *scr, const int2 *tiles, int n_tiles,
                            int sms, cudaStream_t st);
@@ -528,7 +528,7 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
     if (plan.use_gram) {
       gram_tiles(sp, id_begin, id_end, plan.gram_tiles);
     } else if (plan.use_gmt) {
-      gmt_tiles(sp, id_begin, id_end, plan.gmt_tiles);
+      gmt_tiles(sp, id_begin, id_end, d->n_targets, plan.gmt_tiles);
     } else if (any_mul) {
       if (plan.use_tc)
         tc_tiles((int64_t)ia, (int64_t)ja, (int64_t)ib2, (int64_t)jb, plan.mul_tiles);
@@ -677,7 +677,7 @@ static dse_status screen_impl(dse_space *sp, const dse_screen_desc *d, dse_resul
   sc.add(&gram_scr, plan.use_gram ? gram_screen_bytes(sp->n, N) : 1);
   unsigned char *gmt_scr = nullptr;
   sc.add(&plan.gmt_tiles_dev, plan.gmt_tiles.size());
-  sc.add(&gmt_scr, plan.use_gmt ? gmt_screen_bytes(sp->n, N) : 1);
+  sc.add(&gmt_scr, plan.use_gmt ? gmt_screen_bytes(sp->n, N, d->n_targets) : 1);
   dse_status s = sc.alloc(&R->scratch, &R->scratch_bytes);
   plan.gram_scr = gram_scr;
   plan.gmt_scr = gmt_scr;

@@ -253,6 +253,22 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
+// One lane of a converged warp.  Warp roles that issue tensor-core products
+// and bulk copies choose their thread with it: the operands of these
+// instructions are uniform registers, and only here does the compiler know
+// that a single thread is active; under a test of the lane number it wraps
+// every one of them in a loop over the active lanes.  One
+// product issued that way took 190 cycles whatever its shape, elected 115 to
+// 160, against 130 of tensor work for M = 128, N = 256, K = 16.  With the
+// constant descriptor offsets of tcgen05.cuh: k_pair_tc (64 targets, 40 M
+// candidates, N = 500) 14.4 -> 12.9 ms, k_pair_gmt (16 targets, N = 20000)
+// 23.1 -> 22.4 ms, k_l0_gram (3000 columns, N = 1000) 294 -> 286 us.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
 }

@@ -167,10 +167,7 @@ struct Shared {
   int abort;
 };
 constexpr size_t SMEM = 1024 + (size_t)NS * STAGE;
-__device__ __forceinline__ uint64_t desc(uint32_t saddr) {
-  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(LBO >> 4) << 16) | ((uint64_t)(SBO >> 4) << 32) |
-         (1ull << 46);
-}
+static_assert(LBO == tc::LBO, "tc::desc_lo");
 }  // namespace sliced
 
 // Exponent e of each column: |x| <= 2^(e-1) for every sample (one block per
@@ -289,7 +286,7 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    if (elect_one()) {
       int c = 0;
       const unsigned char *a0 = img + (size_t)(2 * bi) * nc * CHUNK, *a1 = a0 + (size_t)nc * CHUNK,
                           *b0 = img + (size_t)bj * nc * CHUNK;
@@ -311,7 +308,7 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    if (elect_one()) {
       for (int kb = 0; kb < nkb && !*abort_flag; ++kb) {
         if (kb >= 1 && !wait(&sh.acc_empty, (kb - 1) & 1)) break;
         tc::fence_after();
@@ -320,16 +317,19 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
           const int st = c % NS;
           if (!wait(&sh.full[st], (c / NS) & 1)) break;
           tc::fence_after();
-          const uint32_t A = smem_u32(stages + (size_t)st * STAGE), B = A + 2 * CHUNK;
+          // operand images as lower descriptor words (offsets in 16 bytes)
+          const uint32_t A = tc::desc_lo(smem_u32(stages + (size_t)st * STAGE)), B = A + 2 * CHUNK / 16;
           // digit i of A against the digits j <= 7 - i of B: their tiles lie
           // side by side, as do the accumulators of the classes i + j, so
           // four of them are one MMA of 256 columns
+#pragma unroll
           for (int i = 0; i < DIG; ++i) {
-            const uint64_t da = desc(A + 2 * i * TILE);
             const uint32_t acc = c > kb * KB || i > 0 ? 1u : 0u;
+#pragma unroll
             for (int j = 0; i + j < DIG; j += 4) {
-              const int w = min(4, DIG - i - j);
-              tc::mma_bf16(tmem + (i + j) * RB, da, desc(B + j * TILE), tc::idesc_bf16(128, w * RB), acc);
+              const int w = i + j + 4 <= DIG ? 4 : DIG - i - j;
+              tc::mma_bf16<tc::desc_hi(SBO)>(tmem + (i + j) * RB, A + 2 * i * TILE / 16, B + j * TILE / 16,
+                                             tc::idesc_bf16(128, w * RB), acc);
             }
           }
           tc::mma_commit(&sh.empty[st]);

@@ -21,10 +21,11 @@
 // of the pair (j, i) when i < j, so the full square of ordered pairs gives
 // every quotient once; a*b, a+b and a-b are taken from the entries with
 // i > j (a+b and a-b need only G11 of the x family and the target sums).
-// A tile is 128 a-features x 6 to 15 b-features, contracted in 32-sample chunks (BF16x3: hi*hi + hi*lo + lo*hi, FP32 accumulation in
-// tensor memory).  Long sample ranges are accumulated in blocks of 16
-// chunks (512 samples) into one of two TMEM column sets and drained by the
-// epilogue into FP32 running sums in registers, so that the accumulation
+// A tile is 128 a-features x 6 to 15 b-features, contracted in 32-sample
+// chunks (BF16x3: hi*hi + hi*lo + lo*hi, FP32 accumulation in tensor
+// memory).  Long sample ranges are accumulated in blocks of 16 chunks (512
+// samples) into one of two TMEM column sets and drained by the epilogue
+// into FP32 running sums in registers, so that the accumulation
 // bound stays that of one block (the same model as the multi-target
 // tensor-core kernel) and the drain overlaps the next block's MMAs.
 //
@@ -884,7 +885,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       int lt = 0;
       uint32_t issued = 0;
       for (int tile = blockIdx.x; tile < GA.n_tiles && !*abort_flag; tile += gridDim.x, ++lt) {
@@ -918,7 +919,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
     }
   } else if (warp == 1) {
     // ----------------------------------------------------------------- MMA
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t IDESC1 = idesc_bf16(128, N1), IDESC2 = idesc_bf16(128, NG);
       int lt = 0;
       bool ok = true;
@@ -939,19 +940,20 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
               break;
             }
             fence_after();
-            const uint32_t S = smem_u32(stages + (size_t)st * STAGE);
-            const uint32_t ph = S, p2h = S + A_PART, pl = S + 2 * A_PART, p2l = S + 3 * A_PART;
-            const uint32_t bh = S + A_IMG, bl = bh + B_PART;
+            // operand images as lower descriptor words (offsets in 16 bytes)
+            const uint32_t ph = desc_lo(smem_u32(stages + (size_t)st * STAGE));
+            const uint32_t p2h = ph + A_PART / 16, pl = ph + 2 * A_PART / 16, p2l = ph + 3 * A_PART / 16;
+            const uint32_t bh = ph + A_IMG / 16, bl = bh + B_PART / 16;
 #pragma unroll
             for (int kk = 0; kk < KC / 16; ++kk) {
-              const uint32_t koff = kk * 2 * LBO;
+              const uint32_t koff = kk * 2 * LBO / 16;
               const uint32_t acc = (c == c0 && kk == 0) ? 0u : 1u;
-              mma_bf16(d, smem_desc(ph + koff), smem_desc(bh + koff), IDESC1, acc);
-              mma_bf16(d + N1, smem_desc(p2h + koff), smem_desc(bh + G_OFF + koff), IDESC2, acc);
-              mma_bf16(d, smem_desc(ph + koff), smem_desc(bl + koff), IDESC1, 1u);
-              mma_bf16(d + N1, smem_desc(p2h + koff), smem_desc(bl + G_OFF + koff), IDESC2, 1u);
-              mma_bf16(d, smem_desc(pl + koff), smem_desc(bh + koff), IDESC1, 1u);
-              mma_bf16(d + N1, smem_desc(p2l + koff), smem_desc(bh + G_OFF + koff), IDESC2, 1u);
+              mma_bf16(d, ph + koff, bh + koff, IDESC1, acc);
+              mma_bf16(d + N1, p2h + koff, bh + G_OFF / 16 + koff, IDESC2, acc);
+              mma_bf16(d, ph + koff, bl + koff, IDESC1, 1u);
+              mma_bf16(d + N1, p2h + koff, bl + G_OFF / 16 + koff, IDESC2, 1u);
+              mma_bf16(d, pl + koff, bh + koff, IDESC1, 1u);
+              mma_bf16(d + N1, p2l + koff, bh + G_OFF / 16 + koff, IDESC2, 1u);
             }
             if (CL == 2)
               mma_commit_mc(&sh.empty[st], (uint16_t)3);

@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(gram::THREADS, 1) k_pair_gram(const ScreenArgs
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
-    if (lane == 0) {
+    if (elect_one()) {
       int lt = 0;
       uint32_t issued = 0;
       for (int tile = blockIdx.x; tile < GA.n_tiles && !*abort_flag; tile += gridDim.x, ++lt) {
@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(gram::THREADS, 1) k_pair_gram(const ScreenArgs
     }
   } else if (warp == 1) {
     // ----------------------------------------------------------------- MMA
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t IDESC = idesc_bf16(M, NCOL);
       int lt = 0;
       for (int tile = blockIdx.x; tile < GA.n_tiles && !*abort_flag; tile += gridDim.x, ++lt) {
@@ -332,15 +332,16 @@ __global__ void __launch_bounds__(gram::THREADS, 1) k_pair_gram(const ScreenArgs
             break;
           }
           fence_after();
-          const uint32_t ah = smem_u32(stages + (size_t)st * STAGE), al = ah + A_HALF;
-          const uint32_t bh = ah + A_IMG, bl = bh + B_HALF;
+          // operand images as lower descriptor words (offsets in 16 bytes)
+          const uint32_t ah = desc_lo(smem_u32(stages + (size_t)st * STAGE)), al = ah + A_HALF / 16;
+          const uint32_t bh = ah + A_IMG / 16, bl = bh + B_HALF / 16;
 #pragma unroll
           for (int kk = 0; kk < KC / 16; ++kk) {
-            const uint32_t koff = kk * 2 * LBO;
+            const uint32_t koff = kk * 2 * LBO / 16;
             const uint32_t acc = (c == 0 && kk == 0) ? 0u : 1u;
-            mma_bf16(d, smem_desc(ah + koff), smem_desc(bh + koff), IDESC, acc);
-            mma_bf16(d, smem_desc(ah + koff), smem_desc(bl + koff), IDESC, 1u);
-            mma_bf16(d, smem_desc(al + koff), smem_desc(bh + koff), IDESC, 1u);
+            mma_bf16(d, ah + koff, bh + koff, IDESC, acc);
+            mma_bf16(d, ah + koff, bl + koff, IDESC, 1u);
+            mma_bf16(d, al + koff, bh + koff, IDESC, 1u);
           }
           mma_commit(&sh.empty[st]);
           if (c == nchunks - 1) mma_commit(&sh.acc_full[buf]);

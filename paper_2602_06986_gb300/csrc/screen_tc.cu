@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
           break;
         }
         unsigned char *S = stages + (size_t)st * SB;
-        if (lane == 0) {
+        if (elect_one()) {
           mbar_arrive_expect_tx(&sh.full_rows[st],
                                 (KIND == KIND_MUL ? 2u : 1u) * 1024u * (uint32_t)shp.boxes + b_bytes(NTP));
           const int x = c * KC;
@@ -585,7 +585,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
       }
   } else if (warp == 1) {
     // ----------------------------------------------------------------- MMA
-    if (lane == 0) {
+    if (elect_one()) {
       constexpr uint32_t IDESC = idesc_bf16(M, NTP);
       int lt = 0;
       for (int tile = blockIdx.x; tile < A.n_tiles && !*abort_flag; tile += gridDim.x, ++lt) {
@@ -599,25 +599,26 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
             const uint32_t sa = gc % NS, ua = gc / NS;
             if (!wait(&sh.full_rows[st], u & 1) || !wait(&sh.full_a[sa], ua & 1)) break;
             fence_after();
-            const uint32_t sbase = smem_u32(stages + (size_t)st * SB);
-            const uint32_t bh = sbase + B_OFF, bl = bh + (uint32_t)NTP * KC * 2;
+            // operand images as lower descriptor words (offsets in 16 bytes)
+            const uint32_t sbase = desc_lo(smem_u32(stages + (size_t)st * SB));
+            const uint32_t bh = sbase + B_OFF / 16, bl = bh + (uint32_t)NTP * KC * 2 / 16;
             constexpr uint32_t IDESC2 = idesc_bf16(M, 2 * NTP);  // wh against [yh; yl]
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
               const uint32_t d = tmem + (buf * 3 + k) * ACW;
-              const uint32_t ah = sbase + A_OFF + (2 * k) * A_TILE, al = ah + A_TILE;
+              const uint32_t ah = sbase + (A_OFF + (2 * k) * A_TILE) / 16, al = ah + A_TILE / 16;
               const uint32_t tah = tmem + ACOL + sa * A_STAGE_COLS + k * KC, tal = tah + KC / 2;
 #pragma unroll
               for (int kk = 0; kk < KC / 16; ++kk) {
-                const uint32_t koff = kk * 2 * LBO;
+                const uint32_t koff = kk * 2 * LBO / 16;
                 const uint32_t acc = (c == b * KB && kk == 0) ? 0u : 1u;
                 if (TA) {
-                  mma_bf16_ta(d, tah + kk * 8, smem_desc(bh + koff), IDESC2, acc);
-                  mma_bf16_ta(d, tal + kk * 8, smem_desc(bh + koff), IDESC, 1u);
+                  mma_bf16_ta(d, tah + kk * 8, bh + koff, IDESC2, acc);
+                  mma_bf16_ta(d, tal + kk * 8, bh + koff, IDESC, 1u);
                 } else {
-                  mma_bf16(d, smem_desc(ah + koff), smem_desc(bh + koff), IDESC, acc);
-                  mma_bf16(d, smem_desc(ah + koff), smem_desc(bl + koff), IDESC, 1u);
-                  mma_bf16(d, smem_desc(al + koff), smem_desc(bh + koff), IDESC, 1u);
+                  mma_bf16(d, ah + koff, bh + koff, IDESC, acc);
+                  mma_bf16(d, ah + koff, bl + koff, IDESC, 1u);
+                  mma_bf16(d, al + koff, bh + koff, IDESC, 1u);
                 }
               }
             }

@@ -9,14 +9,17 @@
 //   k_feature  one warp per candidate, lanes over samples, warp-shuffle
 //              reduction: the stored features themselves and the unary block
 //              of rung k;
-//   k_pair     the binary block of rung k: a CTA owns a tile of 16*MI x 16*MJ
-//              operand rows, streams their samples through shared memory in
-//              chunks with 1-D bulk async copies (double-buffered on
-//              mbarriers), and every lane owns MI x MJ pairs (all three slots
-//              of its kind) for the whole sample range, so no cross-lane
-//              reduction is needed;  KIND_MUL covers a*b, a/b, b/a over every
-//              pair, KIND_ADD covers a+b, a-b, |a-b| over pairs of equal
-//              units only (tiles built per unit class);
+//   k_pair_packed, k_pair64, k_pair
+//              the binary block of rung k, every lane one to four pairs (all
+//              three slots of its kind) for the whole sample range, so no
+//              cross-lane reduction is needed;  KIND_MUL covers a*b, a/b, b/a
+//              over every pair, KIND_ADD covers a+b, a-b, |a-b| over pairs of
+//              equal units only (tiles built per unit class).  k_pair_packed:
+//              FP32, up to 8 target slots, packed FMAs; k_pair64: FP64 of one
+//              screen; k_pair: 16 target slots and the batched FP64 screens,
+//              operand rows streamed through shared memory with 1-D bulk
+//              async copies (double-buffered on mbarriers).  Short lists of
+//              equal-unit pairs go to k_pairlist;
 //   k_escalate FP64 evaluation of candidates whose FP32 realised test could
 //              not be decided, or whose operands are outside the FP32-safe
 //              range.
@@ -393,10 +396,15 @@ __global__ void __launch_bounds__(256) k_feature(const ScreenArgs A, uint64_t id
 // Stored and unary candidates against 16 targets in FP32.  One warp per
 // candidate would read all 16 target rows from L2 for every candidate; here
 // a warp scores CW candidates at once and the block's 8 warps move through
-// the samples together: each 256-sample chunk of the targets (sample-major,
-// [s][8], read with 16-byte loads) and of the block's 32 operand rows is
-// staged in shared memory by asynchronous copies (cp.async, zero-filled past
-// N), double-buffered, so the scoring loop reads shared memory only.  The
+// the samples together: each 256-sample chunk of the targets and of the
+// block's 32 operand rows is staged in shared memory by asynchronous 16-byte
+// copies (cp.async, zero-filled past N), double-buffered, so the scoring loop
+// reads shared memory only, 32 consecutive words a load.  A lane takes four
+// samples of a whole chunk at a time: one switch over the operator for four
+// independent evaluations, each target value read once for the four
+// candidates.  (4-byte copies, the targets sample-major and one sample at a
+// time before: 17500 candidates, 16 targets, N = 20000: 2.43 -> 1.17 ms;
+// 5500 candidates, 7 targets, N = 1531: 112 -> 93 us.)  The
 // samples are taken twice, for targets 0..7 (with S1 and S2) and 8..15, so
 // that the running sums of one half fit in registers at two blocks per SM
 // (one pass over all 16 needed 233 registers: one block, 8 warps per SM);
@@ -406,10 +414,28 @@ __global__ void __launch_bounds__(256) k_feature(const ScreenArgs A, uint64_t id
 // k_feature<float, 16>.
 constexpr int kF16Chunk = 256, kF16CW = 4, kF16Half = 8;
 
-__device__ __forceinline__ void cp_async4(void *dst, const void *src, bool valid) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(smem_u32(dst)), "l"(src),
-               "r"(valid ? 4 : 0)
-               : "memory");
+// 16 bytes, of which the first `bytes` are read and the rest zeros.
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, int bytes) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(bytes) : "memory");
+}
+
+// J values of unary_eval<float> under one switch.
+template <int OP, int J>
+__device__ __forceinline__ void unary_eval_j(const float (&a)[J], float c, float (&v)[J]) {
+#pragma unroll
+  for (int j = 0; j < J; ++j) v[j] = unary_eval<float>(OP, a[j], c);
+}
+template <int J>
+__device__ __forceinline__ void unary_evals(int op, const float (&a)[J], float c, float (&v)[J]) {
+  switch (op) {
+    case DSE_OP_SQUARE: unary_eval_j<DSE_OP_SQUARE>(a, c, v); break;
+    case DSE_OP_CUBE: unary_eval_j<DSE_OP_CUBE>(a, c, v); break;
+    case DSE_OP_INV: unary_eval_j<DSE_OP_INV>(a, c, v); break;
+    case DSE_OP_SQRT: unary_eval_j<DSE_OP_SQRT>(a, c, v); break;
+    case DSE_OP_EXP: unary_eval_j<DSE_OP_EXP>(a, c, v); break;
+    case DSE_OP_LOG: unary_eval_j<DSE_OP_LOG>(a, c, v); break;
+    default: unary_eval_j<DSE_OP_PRIMARY>(a, c, v);
+  }
 }
 
 template <int CW>
@@ -418,7 +444,7 @@ __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64
   pdl_enter();
   constexpr int NT = 16, TH = kF16Half, KS = kF16Chunk, WARPS = 8, NC = WARPS * CW;
   extern __shared__ __align__(16) float f16sm[];
-  float(*ys)[KS][TH] = reinterpret_cast<float(*)[KS][TH]>(f16sm);                  // [2][KS][TH]
+  float(*ys)[TH][KS] = reinterpret_cast<float(*)[TH][KS]>(f16sm);                  // [2][TH][KS]
   float(*xs)[NC][KS] = reinterpret_cast<float(*)[NC][KS]>(f16sm + 2 * KS * TH);     // [2][NC][KS]
   __shared__ const float *rows[NC];
   __shared__ int ract[NC];
@@ -438,19 +464,23 @@ __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64
   LaneStats ls;
   ls.zero();
   const int nchunk = (int)((Ns + KS - 1) / KS);
-  // thread i stages sample i of a chunk: the half's 8 targets and the 32 rows
+  // thread i stages samples 4 (i % 64) .. + 3 of every fourth row of a chunk:
+  // the half's 8 targets and the 32 operand rows (row strides are multiples
+  // of 4 samples, so every piece is aligned)
+  static_assert(KS == 256 && TH % 4 == 0 && NC % 4 == 0, "64 pieces a row, four rows at a time");
   auto stage = [&](int ch, int buf, int th0) {
-    const int64_t s = (int64_t)ch * KS + threadIdx.x;
-    const bool in = s < Ns;
+    const int x = (threadIdx.x & 63) * 4, r0 = threadIdx.x >> 6;
+    const int64_t s = (int64_t)ch * KS + x;
+    const int in = s < Ns ? (int)min((int64_t)16, 4 * (Ns - s)) : 0;
 #pragma unroll
-    for (int t = 0; t < TH; ++t) {
-      const bool v = in && th0 + t < T;
-      cp_async4(&ys[buf][threadIdx.x][t], A.y32 + (v ? (int64_t)(t0 + th0 + t) * ldy + s : 0), v);
+    for (int r = 0; r < TH; r += 4) {
+      const int t = r + r0, bytes = th0 + t < T ? in : 0;
+      cp_async16(&ys[buf][t][x], A.y32 + (bytes ? (int64_t)(t0 + th0 + t) * ldy + s : 0), bytes);
     }
-#pragma unroll 8
-    for (int k = 0; k < NC; ++k) {
-      const bool v = in && ract[k];
-      cp_async4(&xs[buf][k][threadIdx.x], rows[k] + (v ? s : 0), v);
+#pragma unroll
+    for (int r = 0; r < NC; r += 4) {
+      const int k = r + r0, bytes = ract[k] ? in : 0;
+      cp_async16(&xs[buf][k][x], rows[k] + (bytes ? s : 0), bytes);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -504,7 +534,39 @@ __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64
 #pragma unroll
         for (int t = 0; t < TH; ++t) Sy[k][t] = oy[k][t] = 0.f;
       }
-      int blk = 0;
+      // J samples of this lane from offset x of a staged chunk on
+      auto take = [&](auto J_, int buf, int x) {
+        constexpr int J = decltype(J_)::value;
+        float v[CW][J];
+#pragma unroll
+        for (int k = 0; k < CW; ++k) {
+          float a[J];
+#pragma unroll
+          for (int j = 0; j < J; ++j) a[j] = xs[buf][warp * CW + k][x + 32 * j];
+          if (act[k]) unary_evals(op[k], a, c[k], v[k]);
+          else
+#pragma unroll
+            for (int j = 0; j < J; ++j) v[k][j] = 0.f;
+          if (first) {
+#pragma unroll
+            for (int j = 0; j < J; ++j) {
+              S1[k] += v[k][j];
+              S2[k] = fmaf(v[k][j], v[k][j], S2[k]);
+            }
+          }
+        }
+#pragma unroll
+        for (int t = 0; t < TH; ++t) {
+          if (th0 + t >= T) break;
+          float y[J];
+#pragma unroll
+          for (int j = 0; j < J; ++j) y[j] = ys[buf][t][x + 32 * j];
+#pragma unroll
+          for (int k = 0; k < CW; ++k)
+#pragma unroll
+            for (int j = 0; j < J; ++j) Sy[k][t] = fmaf(v[k][j], y[j], Sy[k][t]);
+        }
+      };
       __syncthreads();  // (rows of this tile; the previous pass's last chunk is no longer read)
       stage(0, 0, th0);
       for (int ch = 0; ch < nchunk; ++ch) {
@@ -516,45 +578,26 @@ __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64
           asm volatile("cp.async.wait_group 0;" ::: "memory");
         }
         __syncthreads();
+        const int64_t left = Ns - (int64_t)ch * KS;
+        if (left >= KS) {
 #pragma unroll 1
-        for (int j = 0; j < KS / 32; ++j) {
-          const int64_t s = (int64_t)ch * KS + lane + 32 * j;
-          if (s >= Ns) break;
-          float xv[CW];
-#pragma unroll
-          for (int k = 0; k < CW; ++k) xv[k] = xs[buf][warp * CW + k][lane + 32 * j];
-          float yv[TH];
-          const float4 *yp = reinterpret_cast<const float4 *>(&ys[buf][lane + 32 * j][0]);
-#pragma unroll
-          for (int q = 0; q < TH / 4; ++q) {
-            const float4 y4 = yp[q];
-            yv[4 * q] = y4.x, yv[4 * q + 1] = y4.y, yv[4 * q + 2] = y4.z, yv[4 * q + 3] = y4.w;
-          }
+          for (int j = 0; j < KS / 32; j += 4) take(std::integral_constant<int, 4>(), buf, lane + 32 * j);
+        } else {
+#pragma unroll 1
+          for (int x = lane; x < (int)left; x += 32) take(std::integral_constant<int, 1>(), buf, x);
+        }
+        static_assert(KS / 32 * 2 == 16, "blocks of 16 samples a lane: two chunks");
+        if (ch & 1) {
 #pragma unroll
           for (int k = 0; k < CW; ++k) {
-            if (!act[k]) continue;
-            const float v = unary_eval<float>(op[k], xv[k], c[k]);
-            if (first) {
-              S1[k] += v;
-              S2[k] = fmaf(v, v, S2[k]);
-            }
+            o1[k] += S1[k];
+            o2[k] += S2[k];
+            S1[k] = 0.f;
+            S2[k] = 0.f;
 #pragma unroll
-            for (int t = 0; t < TH; ++t)
-              if (th0 + t < T) Sy[k][t] = fmaf(v, yv[t], Sy[k][t]);
-          }
-          if (++blk == 16) {
-            blk = 0;
-#pragma unroll
-            for (int k = 0; k < CW; ++k) {
-              o1[k] += S1[k];
-              o2[k] += S2[k];
-              S1[k] = 0.f;
-              S2[k] = 0.f;
-#pragma unroll
-              for (int t = 0; t < TH; ++t) {
-                oy[k][t] += Sy[k][t];
-                Sy[k][t] = 0.f;
-              }
+            for (int t = 0; t < TH; ++t) {
+              oy[k][t] += Sy[k][t];
+              Sy[k][t] = 0.f;
             }
           }
         }

@@ -628,37 +628,40 @@ __global__ void __launch_bounds__(256, 2) k_feature16(const ScreenArgs A, uint64
       }
       __syncwarp();
     }
-#pragma unroll 1
-    for (int k = 0; k < CW; ++k) {
-      if (!act[k]) continue;  // (warp-uniform)
-      const float *r = sres[warp * CW + k];
-      const float s1 = r[0], s2 = r[1];
-      float sy[NT];
+    // lane k scores candidate k of the warp (a serial walk over the four, each on
+    // one lane: 5500 candidates, 7 targets, N = 1531 took 93 us, now 57 us)
+    uint64_t id = 0;
+    float cl = 0.f;
+    EvalErr<float> el{0.f, 0.f};
+    bool want = false;
 #pragma unroll
-      for (int t = 0; t < NT; ++t) sy[t] = r[2 + t];
-      const CandInterval<float> ci = cand_interval<float>(s1, s2, N, invN, sqrtN, c[k], ee[k], gamma, u, fmin);
+    for (int k = 0; k < CW; ++k)
+      if (lane == k) id = gid[k], cl = c[k], el = ee[k], want = act[k];
+    const float *r = sres[warp * CW + (lane < CW ? lane : 0)];
+    const float s1 = r[0];
+    float sy[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) sy[t] = r[2 + t];
+    CandInterval<float> ci{};
+    if (want) {
+      ci = cand_interval<float>(s1, r[1], N, invN, sqrtN, cl, el, gamma, u, fmin);
       if (ci.realised == 0) {
-        if (lane == 0) {
-          ls.r[DSE_R_REALISED]++;
-          note_why(A, gid[k], DSE_R_REALISED);
-        }
-        continue;
-      }
-      if (ci.realised == 2) {
-        if (lane == 0) {
-          escalate(A, gid[k]);
-          ls.escalated++;
-        }
-        continue;
-      }
-      if (lane == 0) {
+        ls.r[DSE_R_REALISED]++;
+        note_why(A, id, DSE_R_REALISED);
+        want = false;
+      } else if (ci.realised == 2) {
+        escalate(A, id);
+        ls.escalated++;
+        want = false;
+      } else {
         ls.r[DSE_VALID]++;
         ls.evaluated++;
-        note_why(A, gid[k], DSE_VALID);
+        note_why(A, id, DSE_VALID);
       }
-      const unsigned pushed = score_and_push<float, NT>(A, lane == 0, gid[k], ci, s1, sy, invN, gamma, u, ysum);
-      refresh_pushed<NT>(A, pushed);
     }
+    if (!__any_sync(0xffffffffu, want)) continue;
+    const unsigned pushed = score_and_push<float, NT>(A, want, id, ci, s1, sy, invN, gamma, u, ysum);
+    refresh_pushed<NT>(A, pushed);
   }
   flush_stats(A, ls);
 }

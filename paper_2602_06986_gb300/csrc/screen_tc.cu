@@ -814,6 +814,7 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
                                           : (k == 2 ? fabsf(mi - mj) : 0.f);
         const TcCand tcc = tc_prepare(A, ls, pv, ia, ib, opc, pbase, fa_a, fa_b, kk, mi, mj, sh.hand[p][0][m][2 * k],
                                       sh.hand[p][0][m][2 * k + 1], gamma_gen, gamma_num);
+        uint64_t due = 0;
 #pragma unroll 1
         for (int c16 = 0; c16 < NTP; c16 += 16) {
           float v[16];
@@ -831,8 +832,19 @@ __global__ void __launch_bounds__(tc::THREADS, 1) k_pair_tc(const ScreenArgs A, 
           } else {
             tmem_ld16(tmem + lane_base + (6 + k) * NTP + c16, v);
           }
-          pushed |= tc_targets16(A, tcc, v, c16, gamma_gen, gamma_num, sh.ysum, sh.theta[ew]);
+          due |= tc_targets16(A, tcc, v, c16, gamma_gen, gamma_num, sh.ysum, sh.theta[ew]);
         }
+        // a list without a threshold gets one now, not after the tile: two
+        // tiles a CTA are in flight, and all their candidates (117 k a list
+        // over 152 CTAs) nearly filled the buffers of 132 k; a block of 2^30
+        // candidates then ran twice
+        for (uint64_t all = due; all; all &= all - 1) {
+          const int t = __ffsll((long long)all) - 1;
+          if (sh.theta[ew][t] != 0.f) continue;
+          refresh_theta(A.B, A.t0 + t, A.k);
+          due &= ~(1ull << t);
+        }
+        pushed |= due;
       }
       if (nblocks == 1) {
         fence_before();

@@ -49,3 +49,22 @@ def test_row_blocks(env, rows, cut):
     for t in range(len(Y)):
         ids, sc, eb = res.fetch(t)
         ge._check_topk(ids, sc, eb, oids[t], osc[t], orc, Y, t)
+
+
+def test_first_tiles_leave_room():
+    """20 M candidates in full tiles: the tiles scored before the first thresholds exist must not fill the buffers
+    (a list that overflows is screened a second time)."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    ge.build()
+    from paper_2602_06986_gb300 import dse
+    from paper_2602_06986_gb300 import workloads as W
+
+    w = W.precision(seed=0)
+    X, Y = np.ascontiguousarray(w["X"][:, :64]), np.ascontiguousarray(w["Y"][:, :64])
+    sp = dse.Space(torch.from_numpy(X).cuda(), w["units"], w["op_mask"], 3)
+    begin = sp.n_stored + 6 * sp.n_stored + w["block_seed"]
+    st = sp.screen(torch.from_numpy(Y).cuda(), 1000, precision=dse.PREC_BF16X3, id_begin=begin,
+                   id_end=begin + 20_000_000).stats()
+    assert st["binary_path"] == dse.PATH_TENSOR and st["screened"] == 20_000_000 and st["reruns"] == 0

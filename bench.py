@@ -298,7 +298,7 @@ def bench_batched(args):
     lane_ops = sum(s["evaluated"] * len(t) for s, t in zip(st, targets)) * OPS_PER_EVAL
     pk, pk_src = alu_peak(dse)
     ach = lane_ops / (res["graph"]["ms_per_step"] * 1e-3) / 1e12
-    roofline = {"bound": "alu", "kernel": "the whole batched screen (k_feature_batched, k_pair<float,..,BATCH>, "
+    roofline = {"bound": "alu", "kernel": "the whole batched screen (k_feature_batched, k_pair_packed<..,BATCH>, "
                                           "k_pairlist_batched, selection)",
                 "achieved": ach, "peak": pk, "unit": "T fp32-lane-ops/s", "frac": ach / pk, "traffic": None,
                 "peak_source": pk_src, "ops_per_candidate_sample": OPS_PER_EVAL,
@@ -1036,7 +1036,7 @@ def bench_medium(args):
     else:
         peak, alu_src = alu_peak(dse)  # T lane-ops/s
         achieved = mul_valid * N * OPS_PER_EVAL / (mul_ms * 1e-3) / 1e12 if mul_ms > 0 else None
-        roofline = {"bound": "alu", "kernel": "k_pair<float,MUL,1,2,2> (a*b, a/b, b/a slots)",
+        roofline = {"bound": "alu", "kernel": "k_pair_packed<MUL,1,2> (a*b, a/b, b/a slots)",
                     "achieved": achieved, "peak": peak, "unit": "T fp32-lane-ops/s",
                     "frac": (achieved / peak) if achieved else None, "traffic": None,
                     "peak_source": alu_src,

@@ -434,7 +434,8 @@ dse_status dse_residual_loop(dse_space *space, const dse_loop_desc *desc, dse_lo
    top_pos[n_top][dim] positions into ids (ascending within a subset),
    top_rmse[n_top], top_coefs[n_top][dim+1] (intercept first; may be NULL),
    host arrays; n_found = how many (fewer if fewer subsets have full rank).
-   Limits: dim 1..3, n_ids <= 65536 (the Gram matrix takes 8 n_ids^2 bytes),
+   Limits: dim 1..3, n_ids <= 65536 (the Gram matrix and its FP32 copy take 12
+   n_ids^2 bytes),
    n_top <= 32.  Synchronises. */
 typedef struct {
   const double *y;        /* N values, host or device                       */

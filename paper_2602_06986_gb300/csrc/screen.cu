@@ -39,6 +39,8 @@
 
 namespace dse {
 
+int sm_count();  // api.cu
+
 constexpr uint32_t kWaitLimit = 1u << 22;
 
 // ----------------------------------------------------------- target prep
@@ -2249,10 +2251,10 @@ void launch_feature_t(const ScreenArgs &A, uint64_t id0, uint64_t id1, uint64_t 
       cudaFuncSetAttribute(k_feature16<kF16CW>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF16Smem);
       attr[dev & 63] = true;
     }
-    launch_k(k_feature16<kF16CW>, (unsigned)tiles, 256, kF16Smem, st, B, id0, id1, p0, p1, gamma);
+    launch_spread(k_feature16<kF16CW>, (unsigned)tiles, 256, kF16Smem, st, B, id0, id1, p0, p1, gamma);
     return;
   }
-  launch_k(k_feature<R, NT>, (unsigned)blocks, 256, 0, st, B, id0, id1, p0, p1, gamma);
+  launch_k<sizeof(R) == 4>(k_feature<R, NT>, (unsigned)blocks, 256, 0, st, B, id0, id1, p0, p1, gamma);
 }
 
 template <typename R, int KIND, int NT, int MI, int MJ, bool BATCH = false>
@@ -2278,7 +2280,7 @@ dse_status launch_pair_t(const ScreenArgs &A, int block_len, int sms, cudaStream
   note_launches(1);
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
-  launch_k(k_pair<R, KIND, NT, MI, MJ, BATCH>, grid, 256, C::SMEM, st, B, batch, block_len);
+  launch_k<sizeof(R) == 4>(k_pair<R, KIND, NT, MI, MJ, BATCH>, grid, 256, C::SMEM, st, B, batch, block_len);
   return DSE_OK;
 }
 
@@ -2299,7 +2301,10 @@ dse_status launch_pair_packed(const ScreenArgs &A, int block_len, cudaStream_t s
   note_launches(1);
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
-  launch_k(k_pair_packed<KIND, NT, MI, BATCH>, A.n_tiles, C::THREADS, C::SMEM, st, B, batch, block_len);
+  if (A.n_tiles <= 4 * sm_count())  // one wave
+    launch_spread(k_pair_packed<KIND, NT, MI, BATCH>, A.n_tiles, C::THREADS, C::SMEM, st, B, batch, block_len);
+  else
+    launch_k(k_pair_packed<KIND, NT, MI, BATCH>, A.n_tiles, C::THREADS, C::SMEM, st, B, batch, block_len);
   return DSE_OK;
 }
 
@@ -2336,8 +2341,8 @@ static dse_status launch_pair64(const ScreenArgs &A, int tile, cudaStream_t st) 
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
   note_launches(1);
-  if (tile == 16) launch_k(k_pair64<KIND, 16>, A.n_tiles, 256, 0, st, B);
-  else launch_k(k_pair64<KIND, 8>, A.n_tiles, 64, 0, st, B);
+  if (tile == 16) launch_spread(k_pair64<KIND, 16>, A.n_tiles, 256, 0, st, B);
+  else launch_spread(k_pair64<KIND, 8>, A.n_tiles, 64, 0, st, B);
   return DSE_OK;
 }
 
@@ -2373,7 +2378,7 @@ static void launch_pairlist_split(const ScreenArgs &A, const int2 *pairs, int64_
     cudaFuncSetAttribute(k_pairlist_split<NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     attr[dev & 63] = true;
   }
-  launch_k(k_pairlist_split<NT>, (unsigned)n_pairs, 256, smem, st, A, pairs, gamma);
+  launch_spread(k_pairlist_split<NT>, (unsigned)n_pairs, 256, smem, st, A, pairs, gamma);
 }
 
 void launch_pairlist(int prec64, int nt, const ScreenArgs &A, const int2 *pairs, int64_t n_pairs, float gamma,
@@ -2394,8 +2399,8 @@ void launch_pairlist(int prec64, int nt, const ScreenArgs &A, const int2 *pairs,
     return;
   }
   if (prec64) {
-    if (nt == 1) launch_k(k_pairlist<double, 1>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
-    else launch_k(k_pairlist<double, 16>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
+    if (nt == 1) launch_spread(k_pairlist<double, 1>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
+    else launch_spread(k_pairlist<double, 16>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
   } else {
     if (nt == 1) launch_k(k_pairlist<float, 1>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);
     else launch_k(k_pairlist<float, 16>, (unsigned)blocks, 256, 0, st, B, pairs, n_pairs, gamma);

@@ -1181,7 +1181,7 @@ __global__ void __launch_bounds__(256, (sizeof(R) == 4 && NT == 1) ? 2 : 1)
 //     instruction cache.
 // Block totals lie in shared memory, [sum][thread].
 // N = 9973, 449 k pairs, one target: 3.86 -> 2.61 ms a launch; the 256-problem
-// batch: 48.9 -> 35 ms; 4 targets, N = 1000, 224 k pairs: 874 -> 320 us.
+// batch: 48.9 -> 35 ms; 4 targets, N = 1000, 224 k pairs: 874 -> 297 us.
 template <int NT, int MI>
 struct PackedPairCfg {
   static constexpr int WARPS = 4, THREADS = 32 * WARPS;

@@ -415,7 +415,8 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
 
 // Per candidate, for the scan: the pivot test, its FP64 root L, z = b / L and
 // q = z^2 (valid < 0: the candidate is rejected), and the scale-free FP32
-// forms w = 1 / sqrt(its G32 diagonal) and cr = z / sqrt(Syy).
+// forms w = 1 / sqrt(its G32 diagonal) and cr = z / sqrt(Syy) (0 for a
+// constant target: every subset then explains nothing, and all are taken).
 struct Cand {
   const double *L, *z, *q;
   const float *w, *cr;
@@ -432,7 +433,7 @@ __global__ void k_l0_cands(const double *Gm, const float *G32, const double *b, 
   z[p] = zz;
   q[p] = ok ? zz * zz : -1.0;
   w[p] = ok ? rsqrtf(G32[p * n + p]) : 0.f;
-  cr[p] = ok ? (float)(zz / sqrt(*syy)) : 0.f;
+  cr[p] = ok && *syy > 0.0 ? (float)(zz / sqrt(*syy)) : 0.f;
 }
 
 // (q, subset) ordering: larger explained q first, then positions ascending
@@ -603,7 +604,8 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
         p0 = (int64_t)lo, p1 = (int64_t)hi;
         const float r = G32[p1 * n + p0] * C.w[p0] * C.w[p1], c0 = C.cr[p0];
         const float d = fmaf(-r, r, 1.0f), x = fabsf(fmaf(-r, c0, C.cr[p1])) + 2e-6f;
-        maybe = !(d > 1e-3f) || fmaf(c0, c0, x * x / (d - 4e-6f)) * (1.0f + 1e-5f) + 1e-6f >= need;
+        // (a NaN excludes nothing)
+        maybe = !(d > 1e-3f) || !(fmaf(c0, c0, x * x / (d - 4e-6f)) * (1.0f + 1e-5f) + 1e-6f < need);
       }
       if (!__any_sync(0xffffffffu, maybe)) continue;
       double q = -1.0;
@@ -639,7 +641,7 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
           const float w2 = C.w[p2], l1 = f0[p2] * w0 * w2, l2 = fmaf(-l1, r, f1[p2] * w1 * w2) * i2;
           const float d3 = fmaf(-l2, l2, fmaf(-l1, l1, 1.0f));
           const float x = fabsf(fmaf(-l2, c1, fmaf(-l1, c0, C.cr[p2]))) + 2e-4f;
-          maybe = !(d3 > 1e-2f) || (q2 + x * x / (d3 - 2e-4f)) * (1.0f + 1e-5f) + 3e-4f >= need;
+          maybe = !(d3 > 1e-2f) || !((q2 + x * x / (d3 - 2e-4f)) * (1.0f + 1e-5f) + 3e-4f < need);
         }
         if (!__any_sync(0xffffffffu, maybe)) continue;
         if (!have) {

@@ -157,6 +157,7 @@ constexpr int KC = 16;                       // samples of a stage: one MMA deep
 constexpr int TILE = RB * KC * 2;            // bytes of a digit's tile: 2048
 constexpr int CHUNK = DIG * TILE;            // bytes of a block's chunk: 16 KB
 constexpr int KB = 32;                       // chunks of an exact block: 512 samples
+constexpr int64_t PANEL = 1 << 15;           // samples of an image at most: see dbl in k_l0_gram
 constexpr int STAGE = 3 * CHUNK, NS = 4;     // A: two blocks (128 columns), B: one
 constexpr int EPI = 8, WARPS = 2 + EPI, THREADS = 32 * WARPS;
 constexpr uint32_t LBO = 128, SBO = 256;     // K-major 8 x 8 core matrices, no swizzle
@@ -382,7 +383,9 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
     const int ei = i < n ? ex[i] : INT32_MIN;
     if (ok) {
       // 64-bit integers below 2^51 to doubles: the bits of 1.5 * 2^52 plus the
-      // integer, less 1.5 * 2^52 (exact; one FP64 addition)
+      // integer, less 1.5 * 2^52 (exact; one FP64 addition).  A sample adds at
+      // most (1 + 2/2^7 + 3/2^14 + ..) 2^33 to hi and (5 + 6/2^7 + ..) 2^33 to
+      // lo, so PANEL samples stay below 2^50.4.
       auto dbl = [](long long v) { return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0; };
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
@@ -830,8 +833,8 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
       }
   // digit images: panels of samples, 16 n bytes a sample, 2 GB at most
   const int nblk = 2 * (int)((n + 127) / 128);
-  const int64_t panel = std::min<int64_t>((N + 511) / 512 * 512,
-                                          std::max<int64_t>(512, ((int64_t)2 << 30) / (16 * 64 * (int64_t)nblk) / 512 * 512));
+  const int64_t fit = std::max<int64_t>(512, ((int64_t)2 << 30) / (16 * 64 * (int64_t)nblk) / 512 * 512);
+  const int64_t panel = std::min<int64_t>(std::min<int64_t>(fit, sliced::PANEL), (N + 511) / 512 * 512);
   const int sms = sm_count();
   const int nb = std::min<int64_t>(2 * sms, 8192 / kTop);  // scan blocks (their kTop bests fit the merge)
   // scratch

@@ -64,3 +64,26 @@ def test_constant_target(env, dim, value):
     assert len(pos) == len(opos) == 10 and np.all(rm == 0.0) and np.all(np.abs(orm) < 1e-12)
     assert np.all(cf[:, 0] == value) and np.all(cf[:, 1:] == 0.0)
     assert pos.tolist() == opos.tolist()
+
+
+def test_many_samples_of_one_magnitude(env):
+    """A two-valued column over 300 000 samples: its squared sum is the largest that the digits' integer sums hold
+    (several panels of samples).  It explains half of the target, 79 others 46 to 49%."""
+    N, n, at = 300_000, 80, 41
+    g = np.random.Generator(np.random.PCG64(5))
+    X = np.empty((n, N))
+    X[at] = np.where(np.arange(N) % 2, 2.998, 1.0)
+    t = (X[at] - X[at].mean()) / X[at].std()
+    w = g.standard_normal(N)
+    w -= w.mean()
+    w -= t * (w @ t) / N
+    y = t + w / w.std()
+    for k in range(n):
+        if k != at:
+            a = 0.46 + 0.03 * k / n
+            X[k] = np.sqrt(a / 2) * y + np.sqrt(1 - a) * g.standard_normal(N)
+    pos, rm, cf = search(env, X, y, 1, 16)
+    ref = [rmse_of(X[k:k + 1], y) for k in range(n)]
+    order = np.argsort(ref)
+    assert pos[:, 0].tolist() == order[:16].tolist() and order[0] == at
+    assert np.all(np.abs(rm - np.array(ref)[order[:16]]) <= 1e-9 * rm)

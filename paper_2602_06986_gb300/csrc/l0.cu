@@ -392,15 +392,19 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
         const int64_t j = j0 + k;
         if (i < n && j < n && i <= j) {
           const int ej = ex[j];
+          // hi takes over what lo holds above its own unit
+          const long long h = hi[k] + (lo[k] >> 28), l = lo[k] & ((1ll << 28) - 1);
           // the value without the columns' scales, then scaled (a zero column has digits 0)
-          const double v = fma(dbl(hi[k]), 2.9103830456733704e-11, dbl(lo[k]) * 1.0842021724855044e-19);
+          const double v = fma(dbl(h), 2.9103830456733704e-11, dbl(l) * 1.0842021724855044e-19);
           const int e = (ei == INT32_MIN ? 0 : ei) + (ej == INT32_MIN ? 0 : ej);
-          double g = e > -1000 && e < 1000 ? v * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(v, e);
-          float f = __ll2float_rn(hi[k]) * 2.9103830456733704e-11f;  // (lo adds less than 2^-40 of it or of N 2^-35)
+          const bool plain = e > -1000 && e < 1000;
+          double g = plain ? v * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(v, e);
+          // what l adds is below 2^-35, against 2^-4 for the product of the columns' norms at least
+          float f = __ll2float_rn(h) * 2.9103830456733704e-11f;
           const int64_t at_g = upper ? i * n + j : j * n + i;
           if (add) {
             g += Gm[at_g];
-            f += G32[at_g];
+            f = (float)(plain ? g * __longlong_as_double((long long)(1023 - e) << 52) : scalbn(g, -e));
           }
           Gm[at_g] = g;
           G32[at_g] = f;
@@ -418,13 +422,13 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
 
 // Per candidate, for the scan: the pivot test, its FP64 root L, z = b / L and
 // q = z^2 (valid < 0: the candidate is rejected), and the scale-free FP32
-// forms w = 1 / sqrt(its G32 diagonal) and cr = z / sqrt(Syy) (0 for a
+// forms w = 2^e / L (so that G32 w w is the correlation) and cr = z / sqrt(Syy) (0 for a
 // constant target: every subset then explains nothing, and all are taken).
 struct Cand {
   const double *L, *z, *q;
   const float *w, *cr;
 };
-__global__ void k_l0_cands(const double *Gm, const float *G32, const double *b, const double *nrm2, int64_t n,
+__global__ void k_l0_cands(const double *Gm, const int *ex, const double *b, const double *nrm2, int64_t n,
                            const double *syy, double *L, double *z, double *q, float *w, float *cr) {
   pdl_enter();
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -435,7 +439,7 @@ __global__ void k_l0_cands(const double *Gm, const float *G32, const double *b, 
   L[p] = l;
   z[p] = zz;
   q[p] = ok ? zz * zz : -1.0;
-  w[p] = ok ? rsqrtf(G32[p * n + p]) : 0.f;
+  w[p] = ok ? (float)scalbn(1.0 / l, ex[p]) : 0.f;
   cr[p] = ok && *syy > 0.0 ? (float)(zz / sqrt(*syy)) : 0.f;
 }
 
@@ -552,12 +556,15 @@ __device__ __forceinline__ double explained3(const Step2 &s, double g20, double 
 }
 
 // Scan of every D-subset; each block writes its kTop best to out[block].
-// An FP32 bound of q / Syy from the candidates' correlations (G32 w w, within
-// 5e-7) excludes nearly every subset.  Pairs: 1 - r^2 is within 1e-6 and the
-// numerator within 1e-6.  Triples, where 1 - r^2 > 1e-2: its root is within
-// 5e-5, the second row within 6.5e-5, the last pivot within 1.4e-4 and the
-// numerator within 1.3e-4.  The margins below are wider; where a pivot is
-// smaller the bound is not used. The exact evaluation of each (about 12 FP64
+// An FP32 bound of q / Syy from the candidates' correlations excludes nearly
+// every subset.  A correlation G32 w w has five roundings of 2^-24 (G32, both
+// w, two products) and what G32 leaves of the entry, 2^-31 of the norms'
+// product: within 5e-7.  Pairs: 1 - r^2 is within 1.1e-6 and the numerator
+// within 1e-6.  Triples, where 1 - r^2 > 1e-2: its reciprocal root is within
+// 5.6e-5 of itself, the second row within 7.3e-5, the last pivot within
+// 1.5e-4 and the numerator within 1.4e-4.  The margins below are wider; where
+// a pivot is smaller the bound is not used.  The exact evaluation of each
+// (about 12 FP64
 // operations, two divisions and a root) took 0.96 ms for 4.5 M pairs (0.15 now).
 // `floor`: the best 32nd-best q of any warp so far; a subset below it by
 // more than 1e-9 cannot be among the kMore best that matter.
@@ -910,7 +917,7 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
     launch_k(k_l0_slices, dim3((unsigned)nc, (unsigned)nblk), 128, 0, st, X, ex, n, N, s0, ns, nc, img);
     launch_k(k_l0_gram, (unsigned)tiles, sliced::THREADS, sliced::SMEM, st, img, ex, n, nc, s0 > 0 ? 1 : 0, D == 3 ? 1 : 0, Gm, G32, err);
   }
-  launch_k(k_l0_cands, (unsigned)((n + 127) / 128), 128, 0, st, Gm, G32, bv, nrm2, n, syy, cL, cz, cq, cw, cc);
+  launch_k(k_l0_cands, (unsigned)((n + 127) / 128), 128, 0, st, Gm, ex, bv, nrm2, n, syy, cL, cz, cq, cw, cc);
   const Cand cands{cL, cz, cq, cw, cc};
   if (D == 1) launch_k(k_l0_scan<1>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
   else if (D == 2) launch_k(k_l0_scan<2>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);

@@ -87,3 +87,29 @@ def test_many_samples_of_one_magnitude(env):
     order = np.argsort(ref)
     assert pos[:, 0].tolist() == order[:16].tolist() and order[0] == at
     assert np.all(np.abs(rm - np.array(ref)[order[:16]]) <= 1e-9 * rm)
+
+
+def test_bound_of_columns_with_a_far_value(env):
+    """Two columns of which one sample each holds 40% of the squared norm explain slightly more (3e-6 of the target's
+    square) than each of the 600 pairs around another column: the FP32 bound may not exclude them."""
+    N, n, q = 60_000, 700, 2 * 0.68 ** 2 / 1.5
+    g = np.random.Generator(np.random.PCG64(6))
+    E0, E1, u, v0, v1, w, g2 = frame(g, N, 5, spikes=(1234, 45678))
+    p = [np.sqrt(0.4) * E + np.sqrt(0.5) * u + np.sqrt(0.1) * v for E, v in ((E0, v0), (E1, v1))]
+    c = 0.68
+    y = c / np.sqrt(0.5) * u + np.sqrt(1 - 2 * c * c) * w
+    a = q - 3e-6
+    good = np.sqrt(a) * y + np.sqrt(1 - a) * g2
+    X = np.empty((n, N))
+    X[:] = g.standard_normal((n, N))
+    X -= X.mean(1, keepdims=True)
+    for b in (y, g2):
+        X -= np.outer(X @ b, b)
+    X[70] = good
+    X[n - 2], X[n - 1] = (1.0001 * v / np.abs(v).max() for v in p)  # just above a power of two
+    pos, rm, _ = search(env, X, y, 2, 8)
+    found = [tuple(v) for v in pos.tolist()]
+    assert (n - 2, n - 1) in found[:3]
+    for (i, j), r in list(zip(found, rm))[:3]:
+        ref = rmse_of(X[[i, j]], y)
+        assert abs(r - ref) <= 1e-9 * ref

@@ -139,25 +139,31 @@ __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, in
 // G = X X^T of the centred columns to FP64 accuracy on the tensor cores.  In
 // FP64 instructions the contraction is bound by the FP64 pipe (2 a clock and
 // SM: n = 3000, N = 1000 took 7.69 ms).  Here each column is scaled by a power
-// of two and cut into eight signed 7-bit digits, x = 2^e sum_k d_k 2^-7k + r
-// with |d_k| <= 64 and |r| <= 2^(e-57) (at most 2^-55 of the column's largest
-// value; the FP64 sum of products loses more).  The digits are BF16 numbers,
-// their products integers up to 2^12, and the 36 digit products with
+// of two and cut into eight signed 8-bit digits, x = 2^e sum_k d_k 2^-8(k+1) +
+// r with |d_k| <= 128 and |r| <= 2^(e-65), after the error-free splitting of
+// Ozaki, Ogita, Oishi and Rump ("Error-free transformations of matrix
+// multiplication by using fast routines of matrix multiplication and its
+// applications", Numer. Algorithms 59, 2012).  The digits are BF16 numbers,
+// their products integers up to 2^14, and the 36 digit products with
 // i + j <= 7 are added by class s = i + j, at most 8 of them a class, over
-// blocks of 512 samples: every partial sum is an integer up to 2^24, so the
+// blocks of 128 samples: every partial sum is an integer up to 2^24, so the
 // FP32 accumulation in tensor memory is exact in any order.  The blocks' sums
-// meet in 64-bit integers; one rounding per entry follows at the end.  (The
-// dropped products, i + j > 7, are below 2^-56 of the product of the columns'
-// largest values a sample.)  36 BF16 contractions cost 1/30 of the FP64 one:
-// 7.69 -> 0.29 ms.
+// meet in 64-bit integers; one rounding per entry follows at the end.
+// What is dropped (r and i + j > 7) is below 2^-62.8 of 2^(e_i + e_j) a sample,
+// and each column's norm at least 2^(e-2): below N 2^-58 of the product of the
+// norms, where the FP64 sum is within N 2^-53.  Measured against extended
+// precision at N = 20000: 2e-17 of the diagonal of lognormal products (FP64
+// 9e-16), 7e-16 with one value 3000 times the others, whose dropped squares all
+// add (FP64 1e-16 to 8e-15, by that value's place).  (Digits of 7 bits, in
+// blocks of 512 samples, left 2e-13 there.)
 namespace sliced {
-constexpr int DIG = 8, BITS = 7;
+constexpr int DIG = 8, BITS = 8;
 constexpr int RB = 64;                       // columns of X in an image block
 constexpr int KC = 16;                       // samples of a stage: one MMA deep
 constexpr int TILE = RB * KC * 2;            // bytes of a digit's tile: 2048
 constexpr int CHUNK = DIG * TILE;            // bytes of a block's chunk: 16 KB
-constexpr int KB = 32;                       // chunks of an exact block: 512 samples
-constexpr int64_t PANEL = 1 << 15;           // samples of an image at most: see dbl in k_l0_gram
+constexpr int KB = 8;                        // chunks of an exact block: 128 samples
+constexpr int64_t PANEL = 1 << 12;           // samples of an image at most: see dbl in k_l0_gram
 constexpr int STAGE = 3 * CHUNK, NS = 4;     // A: two blocks (128 columns), B: one
 constexpr int EPI = 8, WARPS = 2 + EPI, THREADS = 32 * WARPS;
 constexpr uint32_t LBO = 128, SBO = 256;     // K-major 8 x 8 core matrices, no swizzle
@@ -213,13 +219,13 @@ __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *e
     const double *x = X + col * N + s0 + k0;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      // the digits of x 2^(56 - e), an integer up to 2^55, lowest first
+      // the digits of x 2^(64 - e), an integer below 2^63, lowest first
       long long q = k0 + i < ns ? __double2ll_rn(scalbn(x[i], DIG * BITS - e)) : 0ll;
 #pragma unroll
       for (int k = DIG - 1; k >= 0; --k) {
-        const int v = k ? (int)((q + 64) & 127) - 64 : (int)q;
+        const int v = k ? (int)((q + 128) & 255) - 128 : (int)q;
         q = (q - v) >> BITS;
-        const uint32_t bits = __float_as_uint((float)v) >> 16;  // exact: |v| <= 64
+        const uint32_t bits = __float_as_uint((float)v) >> 16;  // exact: |v| <= 128
         d[k][i >> 1] |= bits << (16 * (i & 1));
       }
     }
@@ -234,8 +240,9 @@ __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *e
 // bi) per CTA.  Warp 0: producer; warp 1: tensor memory and the MMAs (36 a
 // chunk, accumulators s = 0..7 of 64 columns each: all of tensor memory);
 // warps 2-9: the block sums into 64-bit integers, 32 entries a lane, then the
-// entries i <= j of the tile, both G[i][j] and G[j][i], and the scale-free
-// FP32 values the scan's bound reads.  `add`: onto an earlier panel's.
+// entries i <= j of the tile, as G[i][j] (upper) or G[j][i] (the other half of
+// G is not written), and the scale-free FP32 values the scan's bound reads.
+// `add`: onto an earlier panel's.
 __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned char *img, const int *ex, int64_t n,
                                                                 int nc, int add, int upper, double *Gm, float *G32,
                                                                 int *err) {
@@ -362,7 +369,7 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
         break;
       }
       tc::fence_after();
-      // hi counts in units of 2^-35, lo of 2^-63 (class s: 2^(-7 (s + 2)))
+      // hi counts in units of 2^-40, lo of 2^-72 (class s: 2^(-8 (s + 2)))
 #pragma unroll
       for (int s = 0; s < DIG; ++s) {
         float v[32];
@@ -384,8 +391,9 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
     if (ok) {
       // 64-bit integers below 2^51 to doubles: the bits of 1.5 * 2^52 plus the
       // integer, less 1.5 * 2^52 (exact; one FP64 addition).  A sample adds at
-      // most (1 + 2/2^7 + 3/2^14 + ..) 2^33 to hi and (5 + 6/2^7 + ..) 2^33 to
-      // lo, so PANEL samples stay below 2^50.4.
+      // most (1 + 2/2^8 + 3/2^16 + ..) 2^38 to hi and (5 + 6/2^8 + ..) 2^38 to
+      // lo, which hands over what it holds above 2^32: PANEL samples of hi
+      // stay below 2^50.1.
       auto dbl = [](long long v) { return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0; };
 #pragma unroll
       for (int k = 0; k < 32; ++k) {
@@ -393,14 +401,14 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
         if (i < n && j < n && i <= j) {
           const int ej = ex[j];
           // hi takes over what lo holds above its own unit
-          const long long h = hi[k] + (lo[k] >> 28), l = lo[k] & ((1ll << 28) - 1);
+          const long long h = hi[k] + (lo[k] >> 32), l = lo[k] & 0xffffffffll;
           // the value without the columns' scales, then scaled (a zero column has digits 0)
-          const double v = fma(dbl(h), 2.9103830456733704e-11, dbl(l) * 1.0842021724855044e-19);
+          const double v = fma(dbl(h), 0x1p-40, dbl(l) * 0x1p-72);
           const int e = (ei == INT32_MIN ? 0 : ei) + (ej == INT32_MIN ? 0 : ej);
           const bool plain = e > -1000 && e < 1000;
           double g = plain ? v * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(v, e);
-          // what l adds is below 2^-35, against 2^-4 for the product of the columns' norms at least
-          float f = __ll2float_rn(h) * 2.9103830456733704e-11f;
+          // what l adds is below 2^-40, against 2^-4 for the product of the columns' norms at least
+          float f = __ll2float_rn(h) * 0x1p-40f;
           const int64_t at_g = upper ? i * n + j : j * n + i;
           if (add) {
             g += Gm[at_g];
@@ -558,7 +566,7 @@ __device__ __forceinline__ double explained3(const Step2 &s, double g20, double 
 // Scan of every D-subset; each block writes its kTop best to out[block].
 // An FP32 bound of q / Syy from the candidates' correlations excludes nearly
 // every subset.  A correlation G32 w w has five roundings of 2^-24 (G32, both
-// w, two products) and what G32 leaves of the entry, 2^-31 of the norms'
+// w, two products) and what G32 leaves of the entry, 2^-36 of the norms'
 // product: within 5e-7.  Pairs: 1 - r^2 is within 1.1e-6 and the numerator
 // within 1e-6.  Triples, where 1 - r^2 > 1e-2: its reciprocal root is within
 // 5.6e-5 of itself, the second row within 7.3e-5, the last pivot within

@@ -113,3 +113,19 @@ def test_bound_of_columns_with_a_far_value(env):
     for (i, j), r in list(zip(found, rm))[:3]:
         ref = rmse_of(X[[i, j]], y)
         assert abs(r - ref) <= 1e-9 * ref
+
+
+def test_near_equal_columns_with_a_far_value(env):
+    """Two columns that one sample dominates and whose angle is 6e-7 explain 98% of the target: their squared sine,
+    4e-13, has to survive the Gram matrix's rounding."""
+    N, n = 20_000, 20
+    g = np.random.Generator(np.random.PCG64(7))
+    E0, z, w = frame(g, N, 2, spikes=(777,))
+    X = g.standard_normal((n, N))
+    x = E0 + 0.01 * (X[0] / np.linalg.norm(X[0]))
+    x *= 1.0001 / np.abs(x).max()
+    X[3], X[11] = x, x + np.sqrt(4e-13) * np.linalg.norm(x) * z
+    y = np.sqrt(0.98) * z + np.sqrt(0.02) * w
+    pos, rm, _ = search(env, X, y, 2, 4)
+    assert pos[0].tolist() == [3, 11]
+    assert abs(rm[0] / y.std() - np.sqrt(0.02)) <= 0.01

@@ -434,9 +434,10 @@ dse_status dse_residual_loop(dse_space *space, const dse_loop_desc *desc, dse_lo
    top_pos[n_top][dim] positions into ids (ascending within a subset),
    top_rmse[n_top], top_coefs[n_top][dim+1] (intercept first; may be NULL),
    host arrays; n_found = how many (fewer if fewer subsets have full rank).
-   Limits: dim 1..3, n_ids <= 65536 (the Gram matrix and its FP32 copy take 12
-   n_ids^2 bytes),
-   n_top <= 32.  Synchronises. */
+   Limits: dim 1..3, n_ids <= 65536, n_top <= 32.  Device memory: 12 n_ids^2
+   bytes (the Gram matrix and an FP32 copy), 8 n_ids N (the columns) and up to
+   min(2^31, 65536 n_ids) for their digits; where that does not fit, 8 n_ids^2
+   + 8 n_ids N + 2048 n_ids bytes, and a slower search.  Synchronises. */
 typedef struct {
   const double *y;        /* N values, host or device                       */
   int32_t y_on_device;

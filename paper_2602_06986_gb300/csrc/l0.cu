@@ -412,10 +412,10 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
           const int64_t at_g = upper ? i * n + j : j * n + i;
           if (add) {
             g += Gm[at_g];
-            f = (float)(plain ? g * __longlong_as_double((long long)(1023 - e) << 52) : scalbn(g, -e));
+            if (G32) f = (float)(plain ? g * __longlong_as_double((long long)(1023 - e) << 52) : scalbn(g, -e));
           }
           Gm[at_g] = g;
-          G32[at_g] = f;
+          if (G32) G32[at_g] = f;
         }
       }
     }
@@ -575,7 +575,8 @@ __device__ __forceinline__ double explained3(const Step2 &s, double g20, double 
 // (about 12 FP64
 // operations, two divisions and a root) took 0.96 ms for 4.5 M pairs (0.15 now).
 // `floor`: the best 32nd-best q of any warp so far; a subset below it by
-// more than 1e-9 cannot be among the kMore best that matter.
+// more than 1e-9 cannot be among the kMore best that matter.  Without G32
+// (little memory) every subset is evaluated exactly.
 template <int D>
 __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *G32, const double *b,
                                                  const double *nrm2, const Cand C, const double *syy, int64_t n,
@@ -614,12 +615,14 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
     for (uint64_t base = base0; base < npairs; base += stride) {
       const uint64_t idx = base + lane;
       if ((++turn & 15) == 0) renew();
-      bool maybe = false;
+      bool maybe = idx < npairs;
       int64_t p0 = 0, p1 = 0;
-      if (idx < npairs) {
+      if (maybe) {
         uint64_t hi, lo;
         pair_from_index(idx, &hi, &lo);  // lo < hi
         p0 = (int64_t)lo, p1 = (int64_t)hi;
+      }
+      if (maybe && G32) {
         const float r = G32[p1 * n + p0] * C.w[p0] * C.w[p1], c0 = C.cr[p0];
         const float d = fmaf(-r, r, 1.0f), x = fabsf(fmaf(-r, c0, C.cr[p1])) + 2e-6f;
         // (a NaN excludes nothing)
@@ -645,9 +648,9 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
       if ((++turn & 7) == 0) renew();
       if (p1 + 1 >= n || C.q[p0] < 0.0) continue;
       // the FP32 forms of the two pivots; the exact ones at the first need
-      const float *f0 = G32 + p0 * n, *f1 = G32 + p1 * n;
+      const float *f0 = G32 ? G32 + p0 * n : nullptr, *f1 = G32 ? G32 + p1 * n : nullptr;
       const float w0 = C.w[p0], w1 = C.w[p1], c0 = C.cr[p0];
-      const float r = f0[p1] * w0 * w1, d2 = fmaf(-r, r, 1.0f);
+      const float r = G32 ? f0[p1] * w0 * w1 : 1.0f, d2 = fmaf(-r, r, 1.0f);
       const bool fine = d2 > 1e-2f;
       const float i2 = fine ? rsqrtf(d2) : 0.f, c1 = fmaf(-r, c0, C.cr[p1]) * i2, q2 = fmaf(c0, c0, c1 * c1);
       bool have = false, bad = false;
@@ -846,10 +849,13 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
         set_error("candidate id %llu out of range", (unsigned long long)d->ids[i]);
         return DSE_ERANGE;
       }
-  // digit images: panels of samples, 16 n bytes a sample, 2 GB at most
+  // digit images: panels of samples, 16 n bytes a sample, 2 GB at most.  Where
+  // this and the Gram matrix's FP32 copy do not fit, the shortest panel (one
+  // exact block of samples) and no copy.
   const int nblk = 2 * (int)((n + 127) / 128);
-  const int64_t fit = std::max<int64_t>(512, ((int64_t)2 << 30) / (16 * 64 * (int64_t)nblk) / 512 * 512);
-  const int64_t panel = std::min<int64_t>(std::min<int64_t>(fit, sliced::PANEL), (N + 511) / 512 * 512);
+  constexpr int64_t kBlock = sliced::KB * sliced::KC;
+  const int64_t fit = std::max<int64_t>(kBlock, ((int64_t)2 << 30) / (16 * 64 * (int64_t)nblk) / kBlock * kBlock);
+  int64_t panel = std::min<int64_t>(std::min<int64_t>(fit, sliced::PANEL), (N + kBlock - 1) / kBlock * kBlock);
   const int sms = sm_count();
   const int nb = std::min<int64_t>(2 * sms, 8192 / kTop);  // scan blocks (their kTop bests fit the merge)
   // scratch
@@ -874,9 +880,7 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
   sc.add(&Gm, (size_t)n * n);
   sc.add(&part, (size_t)nb * kTop);
   sc.add(&best, kMore);
-  sc.add(&G32, (size_t)n * n);
   sc.add(&ex, (size_t)n);
-  sc.add(&img, (size_t)nblk * (size_t)(panel / sliced::KC) * sliced::CHUNK);
   sc.add(&cL, (size_t)n);
   sc.add(&cz, (size_t)n);
   sc.add(&cq, (size_t)n);
@@ -888,7 +892,20 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
   sc.add(&cf, (size_t)kMore * 4);
   void *base = nullptr;
   size_t bytes = 0;
-  DSE_TRY(sc.alloc(&base, &bytes));
+  auto allocate = [&](bool copy) {
+    Scratch all = sc;
+    if (copy) all.add(&G32, (size_t)n * n);
+    all.add(&img, (size_t)nblk * (size_t)(panel / sliced::KC) * sliced::CHUNK);
+    return all.alloc(&base, &bytes);
+  };
+  dse_status as = allocate(true);
+  if (as == DSE_ENOMEM) {
+    clear_error();
+    panel = kBlock;
+    G32 = nullptr;
+    as = allocate(false);
+  }
+  DSE_TRY(as);
   struct Free {
     void *p;
     ~Free() { dfree(p); }

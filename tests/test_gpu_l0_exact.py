@@ -129,3 +129,24 @@ def test_near_equal_columns_with_a_far_value(env):
     pos, rm, _ = search(env, X, y, 2, 4)
     assert pos[0].tolist() == [3, 11]
     assert abs(rm[0] / y.std() - np.sqrt(0.02)) <= 0.01
+
+
+@pytest.mark.parametrize("dim", [1, 2, 3])
+def test_little_memory(env, dim):
+    """Where the first allocation fails, the search does without the FP32 copy and with short panels: the same subsets."""
+    torch, oracle, dse, W = env
+    N, n = 700, 130 if dim < 3 else 40
+    g = np.random.Generator(np.random.PCG64(8))
+    X = g.lognormal(0.0, 0.7, size=(n, N))
+    y = X[3] / X[3].std() + 0.7 * X[n // 2] / X[n // 2].std() + 0.5 * g.standard_normal(N)
+    ref = search(env, X, y, dim, 12)
+    sp = dse.Space(torch.from_numpy(X).cuda(), None, W.mask(W.MUL), 1)
+    yd, ids = torch.from_numpy(y).cuda(), torch.arange(n, dtype=torch.int64, device="cuda")
+    try:
+        dse.debug_fail_alloc(0)
+        got = sp.l0_search(yd, ids, dim, 12)
+    finally:
+        dse.debug_fail_alloc(-1)
+    assert len(ref[0]) == 12
+    for a, b in zip(ref, got):
+        assert np.array_equal(a, b)

@@ -17,6 +17,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -76,8 +77,11 @@ struct dse_batch {
   int64_t launches = 0;
   std::vector<dse_stats> host_stats;
   std::vector<int64_t> h_out_n;
-  int64_t fetches = 0;              // lists fetched of the current screen
-  std::vector<uint64_t> h_id;       // every list of it, from the second fetch on (empty before)
+  std::mutex mu;                    // fetches and statistics may come from several threads
+  // lists of the current screen copied ahead (dse_batch_fetch): [h_first,
+  // h_first + h_count); h_next: the item after the last copy's, h_ahead: its lists
+  int64_t h_first = 0, h_count = 0, h_next = -1, h_ahead = 1;
+  std::vector<uint64_t> h_id;
   std::vector<double> h_score, h_eps;
 };
 
@@ -131,8 +135,8 @@ dse_status upload_targets(dse_batch *b, const double *Y, bool on_device) {
 // first use) or enqueue eagerly.
 dse_status run(dse_batch *b, bool use_graph) {
   b->fetched = false;
-  b->fetches = 0;
-  b->h_id.clear();
+  b->h_count = 0;
+  b->h_next = -1;
   b->reruns = 0;
   if (!use_graph) return enqueue(b, b->stream, true, true);
   if (!b->exec) {
@@ -545,6 +549,7 @@ dse_status dse_batch_rescreen(dse_batch *b, const double *Y, int32_t y_on_device
     return DSE_EINVAL;
   }
   AllocStream as(b->stream);
+  std::lock_guard<std::mutex> lk(b->mu);
   DSE_TRY(upload_targets(b, Y, y_on_device != 0));
   return run(b, (b->flags & DSE_BATCH_GRAPH) != 0);
 }
@@ -558,29 +563,49 @@ dse_status dse_batch_fetch(dse_batch *b, int32_t item, uint64_t *idx, double *sc
     return DSE_EINVAL;
   }
   AllocStream as(b->stream);
+  std::lock_guard<std::mutex> lk(b->mu);
   DSE_TRY(finish(b));
   const int64_t n = b->h_out_n[item];
   if (n_out) *n_out = n;
   const int64_t m = std::min(n, cap);
   if (m == 0) return DSE_OK;
   const size_t off = (size_t)item * b->k;
-  // From the second list fetched of a screen on, lists for the host come out
-  // of one copy of them all (three blocking copies a list took 9 ms for 256).
-  const size_t all = (size_t)b->n * b->k;
+  // Lists for the host that are fetched one after the other are copied ahead,
+  // 4, 16, 64 .. of them at a time up to 2^19 entries (three blocking copies a
+  // list took 9 ms for 256 lists of 200); a list out of order is copied alone.
   auto on_host = [](const void *p) { return !p || !is_device_pointer(p); };
-  if (b->fetches++ > 0 && all <= ((size_t)1 << 22) && on_host(idx) && on_host(score) && on_host(err_bound)) {
-    if (b->h_id.empty()) {
-      b->h_id.resize(all);
-      b->h_score.resize(all);
-      b->h_eps.resize(all);
-      DSE_CUDA(cudaMemcpy(b->h_id.data(), b->out_id, 8 * all, cudaMemcpyDeviceToHost));
-      DSE_CUDA(cudaMemcpy(b->h_score.data(), b->out_score, 8 * all, cudaMemcpyDeviceToHost));
-      DSE_CUDA(cudaMemcpy(b->h_eps.data(), b->out_eps, 8 * all, cudaMemcpyDeviceToHost));
+  if (on_host(idx) && on_host(score) && on_host(err_bound)) {
+    if (item < b->h_first || item >= b->h_first + b->h_count) {
+      const int64_t most = std::min<int64_t>(b->n - item, std::max<int64_t>(1, ((int64_t)1 << 19) / b->k));
+      b->h_ahead = item == b->h_next ? std::min<int64_t>(b->h_ahead * 4, 1 << 19) : 1;
+      int64_t count = std::min(b->h_ahead, most);
+      b->h_count = 0;
+      const size_t all = (size_t)count * b->k;
+      try {
+        if (count > 1) {
+          b->h_id.resize(all);
+          b->h_score.resize(all);
+          b->h_eps.resize(all);
+        }
+      } catch (const std::bad_alloc &) {
+        count = 1;
+      }
+      if (count > 1) {
+        DSE_CUDA(cudaMemcpy(b->h_id.data(), b->out_id + off, 8 * all, cudaMemcpyDeviceToHost));
+        DSE_CUDA(cudaMemcpy(b->h_score.data(), b->out_score + off, 8 * all, cudaMemcpyDeviceToHost));
+        DSE_CUDA(cudaMemcpy(b->h_eps.data(), b->out_eps + off, 8 * all, cudaMemcpyDeviceToHost));
+        b->h_first = item;
+        b->h_count = count;
+      }
+      b->h_next = item + count;
     }
-    if (idx) memcpy(idx, b->h_id.data() + off, 8 * m);
-    if (score) memcpy(score, b->h_score.data() + off, 8 * m);
-    if (err_bound) memcpy(err_bound, b->h_eps.data() + off, 8 * m);
-    return DSE_OK;
+    if (b->h_count > 0) {
+      const size_t at = (size_t)(item - b->h_first) * b->k;
+      if (idx) memcpy(idx, b->h_id.data() + at, 8 * m);
+      if (score) memcpy(score, b->h_score.data() + at, 8 * m);
+      if (err_bound) memcpy(err_bound, b->h_eps.data() + at, 8 * m);
+      return DSE_OK;
+    }
   }
   if (idx) DSE_CUDA(cudaMemcpy(idx, b->out_id + off, 8 * m, cudaMemcpyDefault));
   if (score) DSE_CUDA(cudaMemcpy(score, b->out_score + off, 8 * m, cudaMemcpyDefault));
@@ -595,6 +620,7 @@ dse_status dse_batch_stats(dse_batch *b, int32_t item, dse_stats *out) {
     return DSE_EINVAL;
   }
   AllocStream as(b->stream);
+  std::lock_guard<std::mutex> lk(b->mu);
   DSE_TRY(finish(b));
   *out = b->host_stats[item];
   return DSE_OK;

@@ -1,5 +1,6 @@
 // api.cu -- the C ABI: argument checks, handles, and the orchestration of the
 // build, screen and selection kernels.
+#include <cuda.h>
 #include <math.h>
 #include <stdio.h>
 #include <string.h>
@@ -897,6 +898,33 @@ static dse_status finish(dse_result *R) {
 }
 
 
+// Whether p is memory of device dev, not managed, aligned to 8 bytes, with m
+// 8-byte words left in its allocation.  (The driver's query comes through the
+// runtime's entry-point table: the library links the runtime only.)
+static bool holds_words(const void *p, int64_t m, int dev) {
+  typedef CUresult (*Query)(unsigned, CUpointer_attribute *, void **, CUdeviceptr);
+  static const Query query = [] {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion("cuPointerGetAttributes", &fn, 12000, cudaEnableDefault, &q);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e == cudaSuccess && q == cudaDriverEntryPointSuccess ? reinterpret_cast<Query>(fn) : nullptr;
+  }();
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+  if (!query || at % 8 != 0) return false;
+  unsigned type = 0, managed = 0;
+  int of = -1;
+  CUdeviceptr first = 0;
+  size_t bytes = 0;
+  CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED,
+                                CU_POINTER_ATTRIBUTE_DEVICE_ORDINAL, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR,
+                                CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+  void *to[] = {&type, &managed, &of, &first, &bytes};
+  if (query(5, what, to, (CUdeviceptr)at) != CUDA_SUCCESS) return false;
+  return type == CU_MEMORYTYPE_DEVICE && !managed && of == dev && at >= first &&
+         at - first <= bytes && (uint64_t)m <= (bytes - (at - first)) / 8;
+}
+
 // A list's ids, scores and bounds into a caller's device arrays (either may be
 // absent).
 __global__ void k_fetch(const uint64_t *id, const double *score, const double *eps, int64_t n, uint64_t *o_id,
@@ -1414,18 +1442,12 @@ dse_status dse_topk_fetch(dse_result *r, int32_t list, uint64_t *idx, double *sc
   int64_t m = std::min(n, cap);
   if (m == 0) return DSE_OK;
   const size_t off = (size_t)list * r->k;
-  // into this device's memory: one kernel for the three arrays
+  // into this device's memory: one kernel for the three arrays, where each is
+  // aligned and lies within one allocation (the copies below take the rest,
+  // and refuse what does not fit)
   int dev = -1;
   cudaGetDevice(&dev);
-  auto here = [&](const void *p) {
-    cudaPointerAttributes at;
-    if (!p) return true;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
-  };
+  auto here = [&](const void *p) { return !p || holds_words(p, m, dev); };
   if (r->space->device == dev && here(idx) && here(score) && here(err_bound)) {
     note_launches(1);
     launch_k(k_fetch, (unsigned)std::min<int64_t>(64, (m + 255) / 256), 256, 0, r->stream, r->out_id + off,

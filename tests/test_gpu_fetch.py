@@ -85,3 +85,22 @@ def test_batch_lists_from_several_threads(env, batch):
     for t in threads:
         t.join()
     assert not wrong
+
+
+@pytest.mark.parametrize("shift", [0, 1, 4, 8])
+def test_device_arrays_of_any_alignment(env, shift):
+    """A list of a screen into device bytes at any offset: the values of the host fetch, and nothing beyond them."""
+    torch, dse, W = env
+    w = W.tiny(0)
+    sp = dse.Space(torch.from_numpy(w["X"]).cuda(), w["units"], w["op_mask"], w["max_rung"])
+    res = sp.screen(torch.from_numpy(w["Y"]).cuda(), K)
+    ref = res.fetch(0)
+    out = [torch.full((8 * K + 32,), 0x5A, dtype=torch.uint8, device="cuda") for _ in range(3)]
+    n = C.c_int64()
+    assert dse.lib().dse_topk_fetch(res._h, 0, *(t.data_ptr() + shift for t in out), K, C.byref(n)) == dse.OK
+    torch.cuda.synchronize()
+    assert n.value == len(ref[0]) > 0
+    for t, r in zip(out, ref):
+        b = t.cpu().numpy()
+        assert b[shift:shift + 8 * n.value].tobytes() == r.tobytes()
+        assert np.all(b[:shift] == 0x5A) and np.all(b[shift + 8 * n.value:] == 0x5A)

@@ -495,8 +495,8 @@ typedef struct {
                                 (the b-blocks are swept once per group),
                                 1..4096 (2)                                  */
   int32_t gmt_cluster;       /* multi-target Gram kernel: CTAs per thread-
-                                block cluster sharing each b-image chunk by
-                                multicast, 1 or 2 (2; one CTA per tile also
+                                block cluster (neighbours in the tile order,
+                                each with its own copies), 1 or 2 (2; 1 also
                                 where the device cannot co-schedule pairs)   */
   int32_t reserved[1];
 } dse_tuning;

@@ -762,7 +762,7 @@ __device__ __forceinline__ void gmt_epilogue(const ScreenArgs &A, const GmtArgs<
     __syncwarp();
     const int64_t i = (int64_t)tl.x * FA + q * 32 + lane;
     const int64_t j0 = (int64_t)tl.y * FB + BPW * hh;
-    const bool own = tl.x >= 0 && i < A.F.n;  // (tl.x < 0: the empty partner of a pair)
+    const bool own = i < A.F.n;
     gram::EpiFeat Fi;
     if (own) Fi = gmt_rec(A, GA.gf, i);
     // this lane's a-feature target sums (x family), target-major in shared
@@ -817,13 +817,8 @@ __device__ __forceinline__ void gmt_epilogue(const ScreenArgs &A, const GmtArgs<
   flush_stats(A, ls);
 }
 
-// CL = 2: the two CTAs of a cluster take the two tiles of a pair (the same
-// b-block, two a-blocks): each copies its own a-image chunk and one half
-// (BF16 hi or lo part) of the shared b-image chunk, multicast into both
-// CTAs' stages, so the b-side is read from L2 once per pair; a stage is
-// refilled once both CTAs' MMAs have released it (each MMA commit arrives on
-// the empty barriers of both CTAs).  CL = 1: one CTA per tile.
-template <class SH, int CL>
+// A CTA copies both image chunks of its tiles itself.
+template <class SH>
 __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A, const GmtArgs<SH> GA) {
   pdl_enter();
   using namespace gmt;
@@ -831,18 +826,16 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
   constexpr int NTP = SH::NTP, NG = SH::NG, N1 = SH::N1, SET = SH::SET;
   constexpr uint32_t B_PART = SH::B_PART, B_IMG = SH::B_IMG, STAGE = SH::STAGE, G_OFF = SH::G_OFF;
   using namespace tc;
-  static_assert(CL == 1 || CL == 2, "clusters of one or two CTAs");
   extern __shared__ __align__(1024) unsigned char smem[];
   Shared &sh = *reinterpret_cast<Shared *>(smem);
   unsigned char *stages = smem + SH::shared_bytes();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nchunks = GA.nchunks, nblocks = GA.nblocks;
-  const uint32_t crank = CL == 2 ? cluster_ctarank() : 0u;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(&sh.full[s], 1);
-      mbar_init(&sh.empty[s], CL);
+      mbar_init(&sh.empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sh.acc_full[b], 1);
@@ -862,8 +855,6 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
   fence_before();
   __syncthreads();
   fence_after();
-  // (the peer's barriers are initialised before any copy or commit reaches them)
-  if (CL == 2) cluster_sync_all();
   const uint32_t tmem = sh.tmem_base;
 
   volatile int *abort_flag = &sh.abort;
@@ -890,7 +881,6 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
       uint32_t issued = 0;
       for (int tile = blockIdx.x; tile < GA.n_tiles && !*abort_flag; tile += gridDim.x, ++lt) {
         int2 tl = GA.tiles[tile];
-        if (tl.x < 0) tl.x = 0;  // the empty partner of a pair: any a-block, nothing is scored
         if (!(DSE_IN_BOUNDS(tl.x, GA.na, A.err) && DSE_IN_BOUNDS(tl.y, GA.nb, A.err))) tl = make_int2(0, 0);
         bool ok = true;
         for (int c = 0; c < nchunks; ++c) {
@@ -902,11 +892,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
           unsigned char *S = stages + (size_t)st * STAGE;
           mbar_arrive_expect_tx(&sh.full[st], STAGE);
           bulk_g2s(S, GA.aimg + ((size_t)tl.x * nchunks + c) * A_IMG, A_IMG, &sh.full[st]);
-          const unsigned char *bsrc = GA.bimg + ((size_t)tl.y * nchunks + c) * B_IMG;
-          if (CL == 2)
-            bulk_g2s_mc(S + A_IMG + crank * B_PART, bsrc + crank * B_PART, B_PART, &sh.full[st], (uint16_t)3);
-          else
-            bulk_g2s(S + A_IMG, bsrc, B_IMG, &sh.full[st]);
+          bulk_g2s(S + A_IMG, GA.bimg + ((size_t)tl.y * nchunks + c) * B_IMG, B_IMG, &sh.full[st]);
           issued = gc + 1;
         }
         if (!ok) break;
@@ -955,10 +941,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
               mma_bf16(d, pl + koff, bh + koff, IDESC1, 1u);
               mma_bf16(d + N1, p2l + koff, bh + G_OFF / 16 + koff, IDESC2, 1u);
             }
-            if (CL == 2)
-              mma_commit_mc(&sh.empty[st], (uint16_t)3);
-            else
-              mma_commit(&sh.empty[st]);
+            mma_commit(&sh.empty[st]);
           }
           if (!ok) break;
           mma_commit(&sh.acc_full[set]);
@@ -979,8 +962,6 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
   fence_after();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
-  // neither CTA leaves while the other's copies or commits may still reach it
-  if (CL == 2) cluster_sync_all();
 }
 
 // ------------------------------------------------------------------- host
@@ -1067,15 +1048,10 @@ void gmt_tiles(const dse_space *sp, uint64_t id_begin, uint64_t id_end, int T, s
   auto pidx = [&](int64_t i, int64_t j) { return g.um + (tri((uint64_t)i) + (uint64_t)j - g.tri_o) * (uint64_t)g.nb; };
   const int64_t FB = gmt_shape(T, [](auto shape) { return (int64_t)decltype(shape)::FB; });
   const int64_t na = gmt_na(n), nb = (n + FB - 1) / FB;
-  // (an even group: the tiles of a b-block within a group pair up for the
-  // two CTAs of a cluster)
-  int64_t group = std::max(1, tuning().gmt_group);
-  group += group & 1;
-  std::vector<int> as;
+  const int64_t group = std::max(1, tuning().gmt_group);
   for (int64_t ga = 0; ga < na; ga += group) {
     for (int64_t c = 0; c < nb; ++c) {
       const int64_t b0 = c * FB, b1 = std::min<int64_t>(b0 + FB, n) - 1;
-      as.clear();
       for (int64_t a = ga; a < std::min(na, ga + group); ++a) {
         const int64_t a0 = a * gmt::FA, a1 = std::min<int64_t>(a0 + gmt::FA, n) - 1;
         const int64_t Ilo = std::max<int64_t>(std::max(a0, b0), std::max<int64_t>(o, 1));
@@ -1084,10 +1060,8 @@ void gmt_tiles(const dse_space *sp, uint64_t id_begin, uint64_t id_end, int T, s
         if (a0 == b1 && a1 == b0) continue;  // a single feature on both sides: only i == j
         const uint64_t lo = pidx(Ilo, 0), hi = pidx(Ihi, Ihi - 1) + (uint64_t)g.nb;
         if (hi <= p_lo || lo >= p_hi) continue;
-        as.push_back((int)a);
+        out.push_back(make_int2((int)a, (int)c));
       }
-      if (as.size() & 1) as.push_back(-1);  // an empty partner: the pair's second tile scores nothing
-      for (int a : as) out.push_back(make_int2(a, (int)c));
     }
   }
 }
@@ -1118,29 +1092,28 @@ static dse_status launch_gmt(const ScreenArgs &A, const void *space_buf, void *s
   const unsigned char *bimg = static_cast<const unsigned char *>(scr);
   auto *gt = reinterpret_cast<const typename S::Tgt *>(bimg + (size_t)gmt_nb<S>(n) * nchunks * S::B_IMG);
   note_launches(1);
-  // pairs of CTAs per cluster where the device co-schedules them (the count
-  // of clusters that fit at once, per device)
+  // the clusters of two CTAs that fit at once (per device; -1: none)
   static int clusters[64] = {0};
   int dev = 0;
   cudaGetDevice(&dev);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(sms - sms % 2));
+  cfg.blockDim = dim3(gmt::THREADS);
+  cfg.dynamicSmemBytes = S::smem_total();
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   if (clusters[dev & 63] == 0) {
-    DSE_CUDA(cudaFuncSetAttribute(k_pair_gmt<S, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_total()));
-    DSE_CUDA(cudaFuncSetAttribute(k_pair_gmt<S, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_total()));
-    cudaLaunchConfig_t q = {};
-    cudaLaunchAttribute qa[1];
-    qa[0].id = cudaLaunchAttributeClusterDimension;
-    qa[0].val.clusterDim.x = 2;
-    qa[0].val.clusterDim.y = 1;
-    qa[0].val.clusterDim.z = 1;
-    q.gridDim = dim3((unsigned)(sms - sms % 2));
-    q.blockDim = dim3(gmt::THREADS);
-    q.dynamicSmemBytes = S::smem_total();
-    q.attrs = qa;
-    q.numAttrs = 1;
+    DSE_CUDA(cudaFuncSetAttribute(k_pair_gmt<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_total()));
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, k_pair_gmt<S, 2>, &q) != cudaSuccess || nc < 1) {
+    if (cudaOccupancyMaxActiveClusters(&nc, k_pair_gmt<S>, &cfg) != cudaSuccess || nc < 1) {
       cudaGetLastError();
-      nc = -1;  // no clusters: one CTA per tile
+      nc = -1;
     }
     clusters[dev & 63] = nc;
   }
@@ -1152,30 +1125,19 @@ static dse_status launch_gmt(const ScreenArgs &A, const void *space_buf, void *s
   // top-k over candidates in arbitrary order buffers about k (1 + ln(n / k))
   // entries per list whatever the start, and the sample's thresholds rise
   // no faster)
+  // CTA x of the grid takes tiles x, x + grid, ..: neighbours read the same
+  // b-image chunks (the tile list runs through the a-blocks of a b-block
+  // first) at about the same time.  In a cluster they lie side by side on the
+  // chip, which alone is worth 3% at N = 20000, 16 targets, 2531 rows (39.2 ->
+  // 38.0 ms a step); they neither wait for nor write to each other.
   const int nc = clusters[dev & 63];
-  if (tuning().gmt_cluster == 2 && nc > 0 && n_tiles % 2 == 0) {
-    // the tile list holds pairs (2p, 2p + 1) of one b-block; CTA x of the
-    // grid takes tiles x, x + grid, ..., so both CTAs of a cluster take the
-    // two tiles of the same pairs
-    int grid = 2 * nc;
-    if (grid > n_tiles) grid = n_tiles;
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = 2;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3(gmt::THREADS);
-    cfg.dynamicSmemBytes = S::smem_total();
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    DSE_CUDA(cudaLaunchKernelEx(&cfg, k_pair_gmt<S, 2>, B, GA));
+  if (tuning().gmt_cluster == 2 && nc > 0 && n_tiles >= 2) {
+    cfg.gridDim = dim3((unsigned)std::min(2 * nc, n_tiles / 2 * 2));
+    DSE_CUDA(cudaLaunchKernelEx(&cfg, k_pair_gmt<S>, B, GA));
     return DSE_OK;
   }
   const int grid = sms < n_tiles ? sms : n_tiles;
-  launch_k(k_pair_gmt<S, 1>, grid, gmt::THREADS, S::smem_total(), st, B, GA);
+  launch_k(k_pair_gmt<S>, grid, gmt::THREADS, S::smem_total(), st, B, GA);
   return DSE_OK;
 }
 

@@ -55,7 +55,7 @@ struct dse_batch {
   int2 *pairs = nullptr;
   Tile *tmul = nullptr, *tadd = nullptr;
   int32_t n_mul = 0, n_add = 0;
-  unsigned int *counters = nullptr;  // feature jobs, product tiles, sum tiles, pair-list jobs
+  unsigned int *counters = nullptr;  // feature jobs, pair-list jobs
   double *Ycat = nullptr;
   int64_t *yoff = nullptr;
   double *y64 = nullptr;
@@ -106,7 +106,7 @@ dse_status enqueue(dse_batch *b, cudaStream_t st, bool with_targets, bool reset_
   DSE_CUDA(cudaMemsetAsync(b->A0_esc.esc_count, 0, sizeof(unsigned), st));
   DSE_CUDA(cudaMemsetAsync(b->stats, 0, sizeof(unsigned long long) * ST_COUNT * n, st));
   DSE_CUDA(cudaMemsetAsync(b->S.n_jobs, 0, sizeof(unsigned), st));
-  DSE_CUDA(cudaMemsetAsync(b->counters, 0, sizeof(unsigned) * 4, st));
+  DSE_CUDA(cudaMemsetAsync(b->counters, 0, sizeof(unsigned) * 2, st));
   DSE_CUDA(cudaMemsetAsync(b->err, 0, sizeof(int), st));
   if (reset_theta) DSE_CUDA(cudaMemsetAsync(b->B.theta, 0, sizeof(float) * n, st));
   if (with_targets)
@@ -114,7 +114,7 @@ dse_status enqueue(dse_batch *b, cudaStream_t st, bool with_targets, bool reset_
   launch_feature_batched(b->prec64, b->args, b->feat_jobs, b->n_feat_jobs, b->counters, sms, st);
   DSE_TRY(launch_pair_batched(b->prec64, KIND_MUL, b->A0_mul, b->args, sms, st));
   DSE_TRY(launch_pair_batched(b->prec64, KIND_ADD, b->A0_add, b->args_add, sms, st));
-  launch_pairlist_batched(b->prec64, b->args, b->pairs, b->pl_jobs, b->n_pl_jobs, b->counters + 3, sms, st);
+  launch_pairlist_batched(b->prec64, b->args, b->pairs, b->pl_jobs, b->n_pl_jobs, b->counters + 1, sms, st);
   launch_escalate(b->A0_esc, sms, st, b->args);
   DSE_TRY(launch_select(b->S, b->A0_esc, sms, st, b->args));
   DSE_CUDA(cudaGetLastError());
@@ -347,7 +347,7 @@ dse_status plan(const dse_batch_item *items, int32_t n, const dse_batch_desc *d,
   sc.add(&b->pairs, (size_t)n_pairs);
   sc.add(&b->tmul, mul.size());
   sc.add(&b->tadd, add.size());
-  sc.add(&b->counters, 4);
+  sc.add(&b->counters, 2);
   sc.add(&b->Ycat, (size_t)b->ytotal);
   sc.add(&b->yoff, (size_t)n);
   sc.add(&b->y64, (size_t)n * ldy);

@@ -857,8 +857,7 @@ struct PairRing {
 // tile names its problem, whose arguments are read from `batch` (A0 then
 // carries only the tile list and the error flag).
 template <typename R, int KIND, int NT, int MI, int MJ, bool BATCH>
-__global__ void __launch_bounds__(256, (sizeof(R) == 4 && NT == 1) ? 2 : 1)
-    k_pair(const ScreenArgs A0, const ScreenArgs *batch, int block_len0) {
+__global__ void __launch_bounds__(256, 1) k_pair(const ScreenArgs A0, const ScreenArgs *batch, int block_len0) {
   pdl_enter();
   using C = PairCfg<R, KIND, NT, MI, MJ>;
   using V2 = typename Vec2<R>::T;

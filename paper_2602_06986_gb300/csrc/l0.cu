@@ -155,7 +155,7 @@ __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, in
 // precision at N = 20000: 2e-17 of the diagonal of lognormal products (FP64
 // 9e-16), 7e-16 with one value 3000 times the others, whose dropped squares all
 // add (FP64 1e-16 to 8e-15, by that value's place).  (Digits of 7 bits, in
-// blocks of 512 samples, left 2e-13 there.)
+// blocks of 512 samples, left 2e-13 there, in 286 us against 335.)
 namespace sliced {
 constexpr int DIG = 8, BITS = 8;
 constexpr int RB = 64;                       // columns of X in an image block
@@ -165,7 +165,7 @@ constexpr int CHUNK = DIG * TILE;            // bytes of a block's chunk: 16 KB
 constexpr int KB = 8;                        // chunks of an exact block: 128 samples
 constexpr int64_t PANEL = 1 << 12;           // samples of an image at most: see dbl in k_l0_gram
 constexpr int STAGE = 3 * CHUNK, NS = 4;     // A: two blocks (128 columns), B: one
-constexpr int EPI = 8, WARPS = 2 + EPI, THREADS = 32 * WARPS;
+constexpr int EPI = 16, WARPS = 2 + EPI, THREADS = 32 * WARPS;
 constexpr uint32_t LBO = 128, SBO = 256;     // K-major 8 x 8 core matrices, no swizzle
 constexpr uint32_t kWait = 1u << 22;
 struct Shared {
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *e
 // One tile of 128 x 64 entries (i-block bi of 128 columns, j-block bj of 64, bj >= 2
 // bi) per CTA.  Warp 0: producer; warp 1: tensor memory and the MMAs (36 a
 // chunk, accumulators s = 0..7 of 64 columns each: all of tensor memory);
-// warps 2-9: the block sums into 64-bit integers, 32 entries a lane, then the
+// warps 2-17: the block sums into 64-bit integers, 16 entries a lane, then the
 // entries i <= j of the tile, as G[i][j] (upper) or G[j][i] (the other half of
 // G is not written), and the scale-free FP32 values the scan's bound reads.
 // `add`: onto an earlier panel's.
@@ -348,19 +348,14 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
       mbar_wait_bounded(&sh.drain, 0, kWait);
     }
   } else {
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + half * 32;
-    long long hi[32], lo[32];
+    const int q = warp & 3, part = (warp - 2) >> 2;
+    const uint32_t at = tmem + ((uint32_t)(q * 32) << 16) + part * 16;
+    long long hi[16], lo[16];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) hi[i] = lo[i] = 0;
+    for (int i = 0; i < 16; ++i) hi[i] = lo[i] = 0;
     bool ok = true;
     for (int kb = 0; kb < nkb && ok; ++kb) {
-      bool done = false;
-      for (uint32_t it = 0; it < kWait && !done; ++it) {
-        done = mbar_try_wait(&sh.acc_full, kb & 1);
-        if (!done) __nanosleep(100);
-      }
-      ok = __all_sync(0xffffffffu, done);
+      ok = __all_sync(0xffffffffu, mbar_wait_bounded(&sh.acc_full, kb & 1, kWait));
       if (!ok) {
         if (lane == 0) {
           atomicExch(err, DSE_ETIMEOUT);
@@ -369,24 +364,29 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
         break;
       }
       tc::fence_after();
-      // hi counts in units of 2^-40, lo of 2^-72 (class s: 2^(-8 (s + 2)))
+      // hi counts in units of 2^-40, lo of 2^-72 (class s: 2^(-8 (s + 2))).
+      // A class is converted while the next one's columns are on their way; the
+      // conversions (16 a clock and SM, 4096 cycles a block) bound the drain, in
+      // which the products wait.  (Eight warps of 32 columns, one load at a
+      // time: 361 us a launch for n = 3000, N = 1000; 335 now.)
+      uint32_t v[2][16];
+      tc::tmem_ld16_start(at, v[0]);
 #pragma unroll
       for (int s = 0; s < DIG; ++s) {
-        float v[32];
-        tc::tmem_ld32(at + s * RB, v);
-        const int sh_ = BITS * (3 - (s & 3));
+        tc::tmem_ld16_wait(v[s & 1]);
+        if (s + 1 < DIG) tc::tmem_ld16_start(at + (s + 1) * RB, v[(s + 1) & 1]);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const long long w = (long long)__float2int_rn(v[i]) << sh_;
-          if (s < 4) hi[i] += w;
-          else lo[i] += w;
+        for (int i = 0; i < 16; ++i) {
+          const int d = __float2int_rn(__uint_as_float(v[s & 1][i])), unit = 1 << (BITS * (3 - (s & 3)));
+          long long &sum = s < 4 ? hi[i] : lo[i];
+          asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(sum) : "r"(d), "r"(unit));
         }
       }
       tc::fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&sh.acc_empty);
     }
-    const int64_t i = (int64_t)bi * 128 + q * 32 + lane, j0 = (int64_t)bj * RB + half * 32;
+    const int64_t i = (int64_t)bi * 128 + q * 32 + lane, j0 = (int64_t)bj * RB + part * 16;
     const int ei = i < n ? ex[i] : INT32_MIN;
     if (ok) {
       // 64-bit integers below 2^51 to doubles: the bits of 1.5 * 2^52 plus the
@@ -396,7 +396,7 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
       // stay below 2^50.1.
       auto dbl = [](long long v) { return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0; };
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
+      for (int k = 0; k < 16; ++k) {
         const int64_t j = j0 + k;
         if (i < n && j < n && i <= j) {
           const int ej = ex[j];

@@ -495,9 +495,10 @@ typedef struct {
                                 (the b-blocks are swept once per group),
                                 1..4096 (2)                                  */
   int32_t gmt_cluster;       /* multi-target Gram kernel: CTAs per thread-
-                                block cluster (neighbours in the tile order,
-                                each with its own copies), 1 or 2 (2; 1 also
-                                where the device cannot co-schedule pairs)   */
+                                block cluster (neighbours in the tile order
+                                that keep step, each with its own copies), 1
+                                or 2 (2; 1 also where the device cannot co-
+                                schedule pairs and below 1 GB of b-images)   */
   int32_t reserved[1];
 } dse_tuning;
 

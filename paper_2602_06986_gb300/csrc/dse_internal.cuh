@@ -313,6 +313,19 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const void *map, int x, i
       : "memory");
 }
 
+// Clusters of two CTAs: an arrival on the mbarrier at this offset in the other
+// CTA, and a barrier over all threads of both (release / acquire).
+__device__ __forceinline__ void mbar_arrive_peer(uint64_t *bar) {
+  asm volatile(
+      "{\n\t.reg .b32 r, a;\n\tmov.u32 r, %%cluster_ctarank;\n\txor.b32 r, r, 1;\n\t"
+      "mapa.shared::cluster.u32 a, %0, r;\n\tmbarrier.arrive.release.cluster.shared::cluster.b64 _, [a];\n\t}" ::"r"(
+          smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // 1-D bulk async copy global -> shared, completing on an mbarrier.
 // dst, src 16-byte aligned, bytes a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {

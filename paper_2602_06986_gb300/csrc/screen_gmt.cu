@@ -106,7 +106,7 @@ struct GmtShape {
   struct Shared {
     uint64_t full[gmt::NS], empty[gmt::NS];
     uint64_t acc_full[2], acc_empty[2];
-    uint64_t drain;
+    uint64_t drain, pair;
     uint32_t tmem_base;
     int abort;
     float theta[gmt::EPI][NTP];  // each epilogue warp's copy of the list thresholds
@@ -762,7 +762,7 @@ __device__ __forceinline__ void gmt_epilogue(const ScreenArgs &A, const GmtArgs<
     __syncwarp();
     const int64_t i = (int64_t)tl.x * FA + q * 32 + lane;
     const int64_t j0 = (int64_t)tl.y * FB + BPW * hh;
-    const bool own = i < A.F.n;
+    const bool own = tl.x >= 0 && i < A.F.n;  // (tl.x < 0: an empty partner)
     gram::EpiFeat Fi;
     if (own) Fi = gmt_rec(A, GA.gf, i);
     // this lane's a-feature target sums (x family), target-major in shared
@@ -817,8 +817,12 @@ __device__ __forceinline__ void gmt_epilogue(const ScreenArgs &A, const GmtArgs<
   flush_stats(A, ls);
 }
 
-// A CTA copies both image chunks of its tiles itself.
-template <class SH>
+// A CTA copies both image chunks of its tiles itself.  PAIR: in clusters of
+// two, whose CTAs take neighbouring tiles (of one b-block, as a rule) and start
+// every accumulation block together, so that the second read of a chunk finds
+// it in L2: left alone, neighbours drift apart by more than the 10 us or so
+// that the L2 holds.
+template <class SH, bool PAIR>
 __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A, const GmtArgs<SH> GA) {
   pdl_enter();
   using namespace gmt;
@@ -842,6 +846,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
       mbar_init(&sh.acc_empty[b], EPI);
     }
     mbar_init(&sh.drain, 1);
+    mbar_init(&sh.pair, 2);
     sh.abort = 0;
     mbar_fence_init();
   }
@@ -855,6 +860,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
   fence_before();
   __syncthreads();
   fence_after();
+  if (PAIR) cluster_sync_all();  // (the peer's barriers are initialised before an arrival reaches them)
   const uint32_t tmem = sh.tmem_base;
 
   volatile int *abort_flag = &sh.abort;
@@ -881,10 +887,21 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
       uint32_t issued = 0;
       for (int tile = blockIdx.x; tile < GA.n_tiles && !*abort_flag; tile += gridDim.x, ++lt) {
         int2 tl = GA.tiles[tile];
+        if (tl.x < 0) tl.x = 0;  // the empty last partner: any a-block, nothing is scored
         if (!(DSE_IN_BOUNDS(tl.x, GA.na, A.err) && DSE_IN_BOUNDS(tl.y, GA.nb, A.err))) tl = make_int2(0, 0);
         bool ok = true;
         for (int c = 0; c < nchunks; ++c) {
           const uint32_t gc = (uint32_t)lt * nchunks + c, st = gc % NS, u = gc / NS;
+          if (PAIR && c % DB == 0) {
+            // both CTAs' arrivals complete a phase of each barrier: neither is a
+            // phase ahead of the other's wait
+            mbar_arrive(&sh.pair);
+            mbar_arrive_peer(&sh.pair);
+            if (!wait(&sh.pair, ((uint32_t)lt * nblocks + c / DB) & 1)) {
+              ok = false;
+              break;
+            }
+          }
           if (u >= 1 && !wait(&sh.empty[st], (u - 1) & 1)) {
             ok = false;
             break;
@@ -962,6 +979,7 @@ __global__ void __launch_bounds__(gmt::THREADS, 1) k_pair_gmt(const ScreenArgs A
   fence_after();
   if (warp == 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS) : "memory");
+  if (PAIR) cluster_sync_all();  // no arrival may reach a CTA that has left
 }
 
 // ------------------------------------------------------------------- host
@@ -1064,6 +1082,7 @@ void gmt_tiles(const dse_space *sp, uint64_t id_begin, uint64_t id_end, int T, s
       }
     }
   }
+  if (out.size() & 1) out.push_back(make_int2(-1, out.back().y));  // an empty partner: nothing is scored
 }
 
 // delta of the contraction entries for N samples: BF16x3 split, the
@@ -1109,9 +1128,10 @@ static dse_status launch_gmt(const ScreenArgs &A, const void *space_buf, void *s
   cfg.attrs = at;
   cfg.numAttrs = 1;
   if (clusters[dev & 63] == 0) {
-    DSE_CUDA(cudaFuncSetAttribute(k_pair_gmt<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_total()));
+    DSE_CUDA(cudaFuncSetAttribute(k_pair_gmt<S, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_total()));
+    DSE_CUDA(cudaFuncSetAttribute(k_pair_gmt<S, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::smem_total()));
     int nc = 0;
-    if (cudaOccupancyMaxActiveClusters(&nc, k_pair_gmt<S>, &cfg) != cudaSuccess || nc < 1) {
+    if (cudaOccupancyMaxActiveClusters(&nc, k_pair_gmt<S, true>, &cfg) != cudaSuccess || nc < 1) {
       cudaGetLastError();
       nc = -1;
     }
@@ -1125,19 +1145,20 @@ static dse_status launch_gmt(const ScreenArgs &A, const void *space_buf, void *s
   // top-k over candidates in arbitrary order buffers about k (1 + ln(n / k))
   // entries per list whatever the start, and the sample's thresholds rise
   // no faster)
-  // CTA x of the grid takes tiles x, x + grid, ..: neighbours read the same
-  // b-image chunks (the tile list runs through the a-blocks of a b-block
-  // first) at about the same time.  In a cluster they lie side by side on the
-  // chip, which alone is worth 3% at N = 20000, 16 targets, 2531 rows (39.2 ->
-  // 38.0 ms a step); they neither wait for nor write to each other.
+  // CTA x of the grid takes tiles x, x + grid, ..; n_tiles is even (gmt_tiles),
+  // so the CTAs of a cluster take equally many.  Pairs pay where the b-images
+  // are many times the L2 (129 MB); one CTA against pairs, a whole screen, 16
+  // targets: 3.0 GB 11.04 and 10.48 ms, 1.2 GB 4.98 and 4.83, 0.6 GB 1.46 and
+  // 1.46, 150 MB 1.77 and 1.81; 7.4 GB (a step) 39.2 and 35.3.
   const int nc = clusters[dev & 63];
-  if (tuning().gmt_cluster == 2 && nc > 0 && n_tiles >= 2) {
-    cfg.gridDim = dim3((unsigned)std::min(2 * nc, n_tiles / 2 * 2));
-    DSE_CUDA(cudaLaunchKernelEx(&cfg, k_pair_gmt<S>, B, GA));
+  const bool many = (double)GA.nb * nchunks * S::B_IMG >= 1073741824.0;
+  if (tuning().gmt_cluster == 2 && nc > 0 && many) {
+    cfg.gridDim = dim3((unsigned)std::min(2 * nc, n_tiles));
+    DSE_CUDA(cudaLaunchKernelEx(&cfg, k_pair_gmt<S, true>, B, GA));
     return DSE_OK;
   }
   const int grid = sms < n_tiles ? sms : n_tiles;
-  launch_k(k_pair_gmt<S>, grid, gmt::THREADS, S::smem_total(), st, B, GA);
+  launch_k(k_pair_gmt<S, false>, grid, gmt::THREADS, S::smem_total(), st, B, GA);
   return DSE_OK;
 }
 

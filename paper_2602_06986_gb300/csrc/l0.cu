@@ -146,16 +146,17 @@ __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, in
 // applications", Numer. Algorithms 59, 2012).  The digits are BF16 numbers,
 // their products integers up to 2^14, and the 36 digit products with
 // i + j <= 7 are added by class s = i + j, at most 8 of them a class, over
-// blocks of 128 samples: every partial sum is an integer up to 2^24, so the
-// FP32 accumulation in tensor memory is exact in any order.  The blocks' sums
-// meet in 64-bit integers; one rounding per entry follows at the end.
+// blocks of 128 samples (classes 0 to 3: of 256): every partial sum is an
+// integer up to 2^24, so the FP32 accumulation in tensor memory is exact in any
+// order.  The blocks' sums meet in 64-bit integers; one rounding per entry
+// follows at the end.
 // What is dropped (r and i + j > 7) is below 2^-62.8 of 2^(e_i + e_j) a sample,
 // and each column's norm at least 2^(e-2): below N 2^-58 of the product of the
 // norms, where the FP64 sum is within N 2^-53.  Measured against extended
 // precision at N = 20000: 2e-17 of the diagonal of lognormal products (FP64
 // 9e-16), 7e-16 with one value 3000 times the others, whose dropped squares all
 // add (FP64 1e-16 to 8e-15, by that value's place).  (Digits of 7 bits, in
-// blocks of 512 samples, left 2e-13 there, in 286 us against 335.)
+// blocks of 512 samples, left 2e-13 there, in 286 us against 311.)
 namespace sliced {
 constexpr int DIG = 8, BITS = 8;
 constexpr int RB = 64;                       // columns of X in an image block
@@ -332,9 +333,10 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
           // four of them are one MMA of 256 columns
 #pragma unroll
           for (int i = 0; i < DIG; ++i) {
-            const uint32_t acc = c > kb * KB || i > 0 ? 1u : 0u;
 #pragma unroll
             for (int j = 0; i + j < DIG; j += 4) {
+              // classes 0..3 are read every other block only
+              const uint32_t acc = c > kb * KB || i > 0 || (j == 0 && (kb & 1)) ? 1u : 0u;
               const int w = i + j + 4 <= DIG ? 4 : DIG - i - j;
               tc::mma_bf16<tc::desc_hi(SBO)>(tmem + (i + j) * RB, A + 2 * i * TILE / 16, B + j * TILE / 16,
                                              tc::idesc_bf16(128, w * RB), acc);
@@ -365,14 +367,17 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
       }
       tc::fence_after();
       // hi counts in units of 2^-40, lo of 2^-72 (class s: 2^(-8 (s + 2))).
+      // Classes 0..3 add at most 4 products a sample: two blocks of them fit.
       // A class is converted while the next one's columns are on their way; the
-      // conversions (16 a clock and SM, 4096 cycles a block) bound the drain, in
-      // which the products wait.  (Eight warps of 32 columns, one load at a
-      // time: 361 us a launch for n = 3000, N = 1000; 335 now.)
+      // conversions (16 a clock and SM, 4096 cycles for all classes) bound the
+      // drain, in which the products wait.  (Eight warps of 32 columns, every
+      // class each time: 361 us a launch for n = 3000, N = 1000; 311 now.)
       uint32_t v[2][16];
-      tc::tmem_ld16_start(at, v[0]);
+      const bool all = (kb & 1) || kb + 1 == nkb;
+      tc::tmem_ld16_start(at + (all ? 0 : 4 * RB), v[0]);
 #pragma unroll
       for (int s = 0; s < DIG; ++s) {
+        if (s < 4 && !all) continue;
         tc::tmem_ld16_wait(v[s & 1]);
         if (s + 1 < DIG) tc::tmem_ld16_start(at + (s + 1) * RB, v[(s + 1) & 1]);
 #pragma unroll
@@ -402,17 +407,18 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
           const int ej = ex[j];
           // hi takes over what lo holds above its own unit
           const long long h = hi[k] + (lo[k] >> 32), l = lo[k] & 0xffffffffll;
-          // the value without the columns' scales, then scaled (a zero column has digits 0)
-          const double v = fma(dbl(h), 0x1p-40, dbl(l) * 0x1p-72);
+          // scaled by the columns' powers of two (a zero column has digits 0)
           const int e = (ei == INT32_MIN ? 0 : ei) + (ej == INT32_MIN ? 0 : ej);
-          const bool plain = e > -1000 && e < 1000;
-          double g = plain ? v * __longlong_as_double((long long)(1023 + e) << 52) : scalbn(v, e);
+          const bool plain = e > -900 && e < 900;
+          auto pow2 = [](int k) { return __longlong_as_double((long long)(1023 + k) << 52); };
+          double g = plain ? fma(dbl(h), pow2(e - 40), dbl(l) * pow2(e - 72))
+                           : scalbn(fma(dbl(h), 0x1p-40, dbl(l) * 0x1p-72), e);
           // what l adds is below 2^-40, against 2^-4 for the product of the columns' norms at least
           float f = __ll2float_rn(h) * 0x1p-40f;
           const int64_t at_g = upper ? i * n + j : j * n + i;
           if (add) {
             g += Gm[at_g];
-            if (G32) f = (float)(plain ? g * __longlong_as_double((long long)(1023 - e) << 52) : scalbn(g, -e));
+            if (G32) f = (float)(plain ? g * pow2(-e) : scalbn(g, -e));
           }
           Gm[at_g] = g;
           if (G32) G32[at_g] = f;

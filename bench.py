@@ -148,7 +148,7 @@ def measured_bf16(key):
         return (1900.0 if key == "bf16_tflops" else 1700.0), f"fallback {key}"
 
 
-def profiled_traffic(name="k_pair_mul_medium.txt"):
+def profiled_traffic(name):
     """DRAM bytes (read + write) per launch of the dominant kernel from the
     committed ncu summary of the same kernel and workload, or None."""
     scale = {"byte": 1.0, "Kbyte": 1e3, "Mbyte": 1e6, "Gbyte": 1e9}
@@ -625,9 +625,7 @@ def tc_roofline(dse, T, N, mul_ms, mul_valid, step_ms, stats, tc_peak, tc_src):
     return {"bound": "alu", "kernel": f"k_pair_tc<KIND_MUL,{ntp}> (a*b, a/b, b/a; BF16x3 tcgen05 numerators)",
             "achieved": alu, "peak": alu_pk, "unit": "T fp32-lane-ops/s",
             "frac": alu / alu_pk if alu else None,
-            "traffic": profiled_traffic("k_pair_tc_large.txt"),
-            "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch "
-                              "(profiles/k_pair_tc_large.txt)",
+            "traffic": None, "traffic_source": "none: no capture of this workload's launch is kept",
             "peak_source": alu_src,
             "ops_per_candidate_sample": TC_ALU_OPS_PER_EVAL, "valid_candidates_per_launch": mul_valid / len(stats),
             "launch_ms": mul_ms / len(stats), "share_of_step": mul_ms / sum(step_ms),
@@ -1025,11 +1023,9 @@ def bench_medium(args):
         roofline = {"bound": "tensor", "kernel": "k_pair_gram (BF16x3 tcgen05 Gram contraction: a*b, a/b, b/a, a+b, a-b)",
                     "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                     "frac": (achieved / peak) if achieved else None,
-                    # (the committed capture predates the kernel's a+b / a-b slots: no
-                    # counters of the current kernel, so no traffic figure)
-                    "traffic": None,
-                    "traffic_source": "none: profiles/k_pair_gram_medium.txt was captured before the kernel "
-                                      "took the a+b and a-b slots",
+                    "traffic": profiled_traffic("k_pair_gram_medium.txt"),
+                    "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch "
+                                      "(profiles/k_pair_gram_medium.txt)",
                     "peak_source": tc_src + " (of measured, burst: the kernel runs ~0.06 ms at a time inside a short step)",
                     "flops_per_launch": flops, "flops_per_pair_sample": GRAM_FLOPS_PER_PAIR_SAMPLE,
                     "pairs": pairs, "launch_ms": launch_ms, "share_of_step": mul_ms / tot_ms}

@@ -254,15 +254,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
 }
 
 // One lane of a converged warp.  Warp roles that issue tensor-core products
-// and bulk copies choose their thread with it: the operands of these
-// instructions are uniform registers, and only here does the compiler know
-// that a single thread is active; under a test of the lane number it wraps
-// every one of them in a loop over the active lanes.  One
-// product issued that way took 190 cycles whatever its shape, elected 115 to
-// 160, against 130 of tensor work for M = 128, N = 256, K = 16.  With the
+// and bulk copies choose their thread with it: elect.sync tells the compiler
+// that a single thread is active, a test of the lane number does not.  One
+// product issued under such a test took 190 cycles whatever its shape, elected
+// 115 to 160, against 130 of tensor work for M = 128, N = 256, K = 16.  With the
 // constant descriptor offsets of tcgen05.cuh: k_pair_tc (64 targets, 40 M
-// candidates, N = 500) 14.4 -> 12.9 ms, k_pair_gmt (16 targets, N = 20000)
-// 23.1 -> 22.4 ms, k_l0_gram (3000 columns, N = 1000) 294 -> 286 us.
+// candidates, N = 500) 14.4 -> 12.9 ms, k_pair_gmt (16 targets, N = 20000, as
+// it was then) 23.1 -> 22.4 ms, k_l0_gram (3000 columns, N = 1000, 7-bit digits)
+// 294 -> 286 us.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));

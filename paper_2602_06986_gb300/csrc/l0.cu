@@ -152,11 +152,12 @@ __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, in
 // follows at the end.
 // What is dropped (r and i + j > 7) is below 2^-62.8 of 2^(e_i + e_j) a sample,
 // and each column's norm at least 2^(e-2): below N 2^-58 of the product of the
-// norms, where the FP64 sum is within N 2^-53.  Measured against extended
-// precision at N = 20000: 2e-17 of the diagonal of lognormal products (FP64
-// 9e-16), 7e-16 with one value 3000 times the others, whose dropped squares all
-// add (FP64 1e-16 to 8e-15, by that value's place).  (Digits of 7 bits, in
-// blocks of 512 samples, left 2e-13 there, in 286 us against 311.)
+// norms, where the FP64 sum is within N 2^-53.  A model of the arithmetic against
+// extended precision, N = 20000, errors of a diagonal entry: lognormal products
+// 2e-17 (FP64 9e-16); 1/normal, whose dropped squares all add, 3e-16 to 8e-16
+// (FP64 2e-15 to 4e-15); one value 3000 times the others 7e-16 (FP64 2e-17 to
+// 9e-15, by its place).  (Digits of 7 bits, in blocks of 512 samples, left 2e-13
+// there, in 286 us against 311.)
 namespace sliced {
 constexpr int DIG = 8, BITS = 8;
 constexpr int RB = 64;                       // columns of X in an image block

@@ -2300,7 +2300,7 @@ dse_status launch_pair_packed(const ScreenArgs &A, int block_len, cudaStream_t s
   note_launches(1);
   ScreenArgs B = A;
   B.group = KIND == KIND_MUL ? 1 : 2;
-  if (A.n_tiles <= 4 * sm_count())  // one wave
+  if (A.n_tiles <= 4 * sm_count())  // one wave: see launch_spread
     launch_spread(k_pair_packed<KIND, NT, MI, BATCH>, A.n_tiles, C::THREADS, C::SMEM, st, B, batch, block_len);
   else
     launch_k(k_pair_packed<KIND, NT, MI, BATCH>, A.n_tiles, C::THREADS, C::SMEM, st, B, batch, block_len);

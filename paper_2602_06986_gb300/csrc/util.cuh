@@ -63,9 +63,11 @@ inline void launch_k(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, c
 // A kernel whose blocks run long, fewer than the chip holds: placed while the
 // kernel before it still runs, they pile up on the SMs that are free first
 // and the fullest SM sets the time.  Launched after it they are spread evenly.
-// FP64 screen of 185 rows, N = 500 (296 blocks of k_pair64): 1160 us
-// overlapped, 498 us spread; a grid of several waves gains from the overlap
-// (928 tiles of k_pair_packed at N = 10000: 2.98 against 3.12 ms).
+// Whole screens, overlapped and spread: FP64, 185 rows, N = 500 (296 blocks of
+// k_pair64) 1160 and 498 us; k_pair_packed, 132 tiles, N = 2100: 747 and 447 us;
+// 441 tiles, N = 9973: 3561 and 2839 us.  Grids of several waves run alike either
+// way (k_pair_packed, 900 tiles, N = 2100: 1287 and 1290 us; 1122 tiles, N = 9973:
+// 6620 and 6608) and take the overlapped launch.
 template <typename... X>
 inline void launch_spread(X &&...x) {
   launch_k<false>(std::forward<X>(x)...);

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(kCol) k_l0_columns(FeatTable F, RungGeom G, in
 // 2e-17 (FP64 9e-16); 1/normal, whose dropped squares all add, 3e-16 to 8e-16
 // (FP64 2e-15 to 4e-15); one value 3000 times the others 7e-16 (FP64 2e-17 to
 // 9e-15, by its place).  (Digits of 7 bits, in blocks of 512 samples, left 2e-13
-// there, in 286 us against 311.)
+// there, in 286 us against 294.)
 namespace sliced {
 constexpr int DIG = 8, BITS = 8;
 constexpr int RB = 64;                       // columns of X in an image block
@@ -165,7 +165,7 @@ constexpr int KC = 16;                       // samples of a stage: one MMA deep
 constexpr int TILE = RB * KC * 2;            // bytes of a digit's tile: 2048
 constexpr int CHUNK = DIG * TILE;            // bytes of a block's chunk: 16 KB
 constexpr int KB = 8;                        // chunks of an exact block: 128 samples
-constexpr int64_t PANEL = 1 << 12;           // samples of an image at most: see dbl in k_l0_gram
+constexpr int64_t PANEL = 1 << 12;           // samples of an image at most: see its epilogue
 constexpr int STAGE = 3 * CHUNK, NS = 4;     // A: two blocks (128 columns), B: one
 constexpr int EPI = 16, WARPS = 2 + EPI, THREADS = 32 * WARPS;
 constexpr uint32_t LBO = 128, SBO = 256;     // K-major 8 x 8 core matrices, no swizzle
@@ -236,6 +236,31 @@ __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *e
 #pragma unroll
   for (int k = 0; k < DIG; ++k)
     *reinterpret_cast<uint4 *>(o + k * TILE) = make_uint4(d[k][0], d[k][1], d[k][2], d[k][3]);
+}
+
+// (h 2^32 + l) 2^e rounded to FP64, for |h| < 2^51 and results in the normal
+// range, in integer instructions: the FP64 pipe (2 operations a clock and SM)
+// takes 16000 cycles for a tile's entries, after the products and alone (311 us
+// a launch for n = 3000, N = 1000; 294 with integers).
+__device__ __forceinline__ double wide_to_double(long long h, uint32_t l, int e) {
+  const bool neg = h < 0;
+  const unsigned long long a = neg ? (unsigned long long)~h + (l == 0u) : (unsigned long long)h;
+  const uint32_t b = neg ? 0u - l : l;
+  unsigned long long m = a << 32 | b;
+  int n;  // significant bits
+  if (a >> 21) {
+    n = 96 - __clzll((long long)a);
+    const int s = n - 53;  // 1 to 30 bits are dropped
+    m = a << (32 - s) | b >> s;
+    const uint32_t rest = b << (32 - s);
+    m += rest > 0x80000000u || (rest == 0x80000000u && (m & 1)) ? 1u : 0u;
+  } else {
+    n = 64 - __clzll((long long)m);
+    m = m ? m << (53 - n) : 0ull;
+  }
+  // (m's leading bit adds the last unit of the exponent field, a carry one more)
+  const unsigned long long bits = m ? ((unsigned long long)(1021 + n + e) << 52) + m : 0ull;
+  return __longlong_as_double((long long)(bits | (neg ? 1ull << 63 : 0ull)));
 }
 
 // One tile of 128 x 64 entries (i-block bi of 128 columns, j-block bj of 64, bj >= 2
@@ -372,7 +397,7 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
       // A class is converted while the next one's columns are on their way; the
       // conversions (16 a clock and SM, 4096 cycles for all classes) bound the
       // drain, in which the products wait.  (Eight warps of 32 columns, every
-      // class each time: 361 us a launch for n = 3000, N = 1000; 311 now.)
+      // class each time: 361 us a launch for n = 3000, N = 1000; 311 so.)
       uint32_t v[2][16];
       const bool all = (kb & 1) || kb + 1 == nkb;
       tc::tmem_ld16_start(at + (all ? 0 : 4 * RB), v[0]);
@@ -395,31 +420,28 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
     const int64_t i = (int64_t)bi * 128 + q * 32 + lane, j0 = (int64_t)bj * RB + part * 16;
     const int ei = i < n ? ex[i] : INT32_MIN;
     if (ok) {
-      // 64-bit integers below 2^51 to doubles: the bits of 1.5 * 2^52 plus the
-      // integer, less 1.5 * 2^52 (exact; one FP64 addition).  A sample adds at
-      // most (1 + 2/2^8 + 3/2^16 + ..) 2^38 to hi and (5 + 6/2^8 + ..) 2^38 to
-      // lo, which hands over what it holds above 2^32: PANEL samples of hi
-      // stay below 2^50.1.
-      auto dbl = [](long long v) { return __longlong_as_double(0x4338000000000000ll + v) - 6755399441055744.0; };
+      // A sample adds at most (1 + 2/2^8 + 3/2^16 + ..) 2^38 to hi and (5 +
+      // 6/2^8 + ..) 2^38 to lo, which hands over what it holds above 2^32:
+      // PANEL samples of hi stay below 2^50.1, as wide_to_double wants it.
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const int64_t j = j0 + k;
         if (i < n && j < n && i <= j) {
           const int ej = ex[j];
           // hi takes over what lo holds above its own unit
-          const long long h = hi[k] + (lo[k] >> 32), l = lo[k] & 0xffffffffll;
+          const long long h = hi[k] + (lo[k] >> 32);
+          const uint32_t l = (uint32_t)lo[k];
           // scaled by the columns' powers of two (a zero column has digits 0)
           const int e = (ei == INT32_MIN ? 0 : ei) + (ej == INT32_MIN ? 0 : ej);
           const bool plain = e > -900 && e < 900;
-          auto pow2 = [](int k) { return __longlong_as_double((long long)(1023 + k) << 52); };
-          double g = plain ? fma(dbl(h), pow2(e - 40), dbl(l) * pow2(e - 72))
-                           : scalbn(fma(dbl(h), 0x1p-40, dbl(l) * 0x1p-72), e);
+          double g = wide_to_double(h, l, (plain ? e : 0) - 72);
+          if (!plain) g = scalbn(g, e);
           // what l adds is below 2^-40, against 2^-4 for the product of the columns' norms at least
           float f = __ll2float_rn(h) * 0x1p-40f;
           const int64_t at_g = upper ? i * n + j : j * n + i;
           if (add) {
             g += Gm[at_g];
-            if (G32) f = (float)(plain ? g * pow2(-e) : scalbn(g, -e));
+            if (G32) f = (float)(plain ? g * __longlong_as_double((long long)(1023 - e) << 52) : scalbn(g, -e));
           }
           Gm[at_g] = g;
           if (G32) G32[at_g] = f;

@@ -436,7 +436,7 @@ dse_status dse_residual_loop(dse_space *space, const dse_loop_desc *desc, dse_lo
    host arrays; n_found = how many (fewer if fewer subsets have full rank).
    Limits: dim 1..3, n_ids <= 65536, n_top <= 32.  Device memory: 12 n_ids^2
    bytes (the Gram matrix and an FP32 copy), 8 n_ids N (the columns) and up to
-   min(2^31, 65536 n_ids) for their digits; where that does not fit, 8 n_ids^2
+   min(2^31, 2^18 n_ids) for their digits; where that does not fit, 8 n_ids^2
    + 8 n_ids N + 2048 n_ids bytes, and a slower search.  Synchronises. */
 typedef struct {
   const double *y;        /* N values, host or device                       */

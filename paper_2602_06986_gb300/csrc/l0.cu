@@ -165,7 +165,7 @@ constexpr int KC = 16;                       // samples of a stage: one MMA deep
 constexpr int TILE = RB * KC * 2;            // bytes of a digit's tile: 2048
 constexpr int CHUNK = DIG * TILE;            // bytes of a block's chunk: 16 KB
 constexpr int KB = 8;                        // chunks of an exact block: 128 samples
-constexpr int64_t PANEL = 1 << 12;           // samples of an image at most: see its epilogue
+constexpr int64_t PANEL = 1 << 14;           // samples of an image at most: see its epilogue
 constexpr int STAGE = 3 * CHUNK, NS = 4;     // A: two blocks (128 columns), B: one
 constexpr int EPI = 16, WARPS = 2 + EPI, THREADS = 32 * WARPS;
 constexpr uint32_t LBO = 128, SBO = 256;     // K-major 8 x 8 core matrices, no swizzle
@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(128) k_l0_slices(const double *X, const int *e
     *reinterpret_cast<uint4 *>(o + k * TILE) = make_uint4(d[k][0], d[k][1], d[k][2], d[k][3]);
 }
 
-// (h 2^32 + l) 2^e rounded to FP64, for |h| < 2^51 and results in the normal
+// (h 2^32 + l) 2^e rounded to FP64, for |h| < 2^53 and results in the normal
 // range, in integer instructions: the FP64 pipe (2 operations a clock and SM)
 // takes 16000 cycles for a tile's entries, after the products and alone (311 us
 // a launch for n = 3000, N = 1000; 294 with integers).
@@ -250,8 +250,8 @@ __device__ __forceinline__ double wide_to_double(long long h, uint32_t l, int e)
   int n;  // significant bits
   if (a >> 21) {
     n = 96 - __clzll((long long)a);
-    const int s = n - 53;  // 1 to 30 bits are dropped
-    m = a << (32 - s) | b >> s;
+    const int s = n - 53;  // 1 to 32 bits are dropped
+    m = a << (32 - s) | (unsigned long long)b >> s;
     const uint32_t rest = b << (32 - s);
     m += rest > 0x80000000u || (rest == 0x80000000u && (m & 1)) ? 1u : 0u;
   } else {
@@ -422,7 +422,7 @@ __global__ void __launch_bounds__(sliced::THREADS, 1) k_l0_gram(const unsigned c
     if (ok) {
       // A sample adds at most (1 + 2/2^8 + 3/2^16 + ..) 2^38 to hi and (5 +
       // 6/2^8 + ..) 2^38 to lo, which hands over what it holds above 2^32:
-      // PANEL samples of hi stay below 2^50.1, as wide_to_double wants it.
+      // PANEL samples of hi stay below 2^52.1, as wide_to_double wants it.
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const int64_t j = j0 + k;
@@ -604,9 +604,9 @@ __device__ __forceinline__ double explained3(const Step2 &s, double g20, double 
 // (about 12 FP64
 // operations, two divisions and a root) took 0.96 ms for 4.5 M pairs (0.15 now).
 // `floor`: the best 32nd-best q of any warp so far; a subset below it by
-// more than 1e-9 cannot be among the kMore best that matter.  Without G32
-// (little memory) every subset is evaluated exactly.
-template <int D>
+// more than 1e-9 cannot be among the kMore best that matter.  Without BOUND
+// (little memory: no G32) every subset is evaluated exactly.
+template <int D, bool BOUND>
 __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *G32, const double *b,
                                                  const double *nrm2, const Cand C, const double *syy, int64_t n,
                                                  unsigned long long *floor_bits, Hit *out) {
@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
         pair_from_index(idx, &hi, &lo);  // lo < hi
         p0 = (int64_t)lo, p1 = (int64_t)hi;
       }
-      if (maybe && G32) {
+      if (BOUND && maybe) {
         const float r = G32[p1 * n + p0] * C.w[p0] * C.w[p1], c0 = C.cr[p0];
         const float d = fmaf(-r, r, 1.0f), x = fabsf(fmaf(-r, c0, C.cr[p1])) + 2e-6f;
         // (a NaN excludes nothing)
@@ -677,9 +677,9 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
       if ((++turn & 7) == 0) renew();
       if (p1 + 1 >= n || C.q[p0] < 0.0) continue;
       // the FP32 forms of the two pivots; the exact ones at the first need
-      const float *f0 = G32 ? G32 + p0 * n : nullptr, *f1 = G32 ? G32 + p1 * n : nullptr;
+      const float *f0 = G32 + p0 * n, *f1 = G32 + p1 * n;
       const float w0 = C.w[p0], w1 = C.w[p1], c0 = C.cr[p0];
-      const float r = G32 ? f0[p1] * w0 * w1 : 1.0f, d2 = fmaf(-r, r, 1.0f);
+      const float r = BOUND ? f0[p1] * w0 * w1 : 1.0f, d2 = fmaf(-r, r, 1.0f);
       const bool fine = d2 > 1e-2f;
       const float i2 = fine ? rsqrtf(d2) : 0.f, c1 = fmaf(-r, c0, C.cr[p1]) * i2, q2 = fmaf(c0, c0, c1 * c1);
       bool have = false, bad = false;
@@ -687,7 +687,7 @@ __global__ void __launch_bounds__(256) k_l0_scan(const double *Gm, const float *
       for (int64_t base = p1 + 1; base < n && !bad; base += 32) {
         const int64_t p2 = base + lane;
         bool maybe = p2 < n;
-        if (maybe && fine) {
+        if (BOUND && maybe && fine) {
           const float w2 = C.w[p2], l1 = f0[p2] * w0 * w2, l2 = fmaf(-l1, r, f1[p2] * w1 * w2) * i2;
           const float d3 = fmaf(-l2, l2, fmaf(-l1, l1, 1.0f));
           const float x = fabsf(fmaf(-l2, c1, fmaf(-l1, c0, C.cr[p2]))) + 2e-4f;
@@ -973,9 +973,10 @@ dse_status l0_search_impl(dse_space *sp, const dse_l0_desc *d, int64_t *top_pos,
   }
   launch_k(k_l0_cands, (unsigned)((n + 127) / 128), 128, 0, st, Gm, ex, bv, nrm2, n, syy, cL, cz, cq, cw, cc);
   const Cand cands{cL, cz, cq, cw, cc};
-  if (D == 1) launch_k(k_l0_scan<1>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
-  else if (D == 2) launch_k(k_l0_scan<2>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
-  else launch_k(k_l0_scan<3>, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part);
+  auto scan = [&](auto kernel) { launch_k(kernel, nb, 256, 0, st, Gm, G32, bv, nrm2, cands, syy, n, floor_bits, part); };
+  if (D == 1) scan(k_l0_scan<1, false>);
+  else if (D == 2) G32 ? scan(k_l0_scan<2, true>) : scan(k_l0_scan<2, false>);
+  else G32 ? scan(k_l0_scan<3, true>) : scan(k_l0_scan<3, false>);
   launch_k(k_l0_merge, 1, 1024, 0, st, part, (int64_t)nb * kTop, floor_bits, best);
   launch_k(k_l0_exact, kMore, 32, 0, st, best, D, X, bv, nrm2, N, ge);
   launch_k(k_l0_refit, kMore, kCol, 0, st, best, D, X, yc, mean, ge, bv, nrm2, N, 0.0, rm, cf);
